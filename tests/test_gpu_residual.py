@@ -144,3 +144,18 @@ def test_errors():
     rc = sp.spmesl_fit_residual(X, 30, 50, 50, prob.lambda0, 1e-6, 100, opts, Theta, sig, None,
                                 ws, nb)
     assert rc == sp.SPMESL_EINVAL
+
+
+@pytest.mark.parametrize("p", [2, 127, 128, 129, 257, 640])
+@pytest.mark.parametrize("n", [64, 95])
+def test_quiet_chunks_at_the_edges(p, n):
+    """Chunks of which only the support coordinates are formed: sizes around
+    the 128-coordinate chunk and the 4- and 32-sample strides (coordinates
+    enter and leave the support as sigma falls).  FP64 at tol 1e-10 is held to
+    the bar of the oracle comparison above."""
+    prob = synth.make_problem("ar1", p, n, 3 + p + n, dtype=np.float64)
+    T, sig, st = _res(prob.X, prob.lambda0, 1e-10, "fp64")
+    assert st["status"] == sp.SPMESL_OK
+    S, ref = _oracle(prob.X, prob.lambda0, 1e-10)
+    res = compare_theta(T, ref["Theta"], ref["B"], ref["sigma"], rel=1e-7)
+    assert res["ok"], res

@@ -100,6 +100,55 @@ __device__ __forceinline__ T soft(T x, T lam) {
     return x > lam ? x - lam : (x < -lam ? x + lam : T(0));
 }
 
+// The same for the standardised working matrix, where every operand is finite
+// (|S| <= 1; non-finite input ends the fit before its solvers), in fewer
+// dependent instructions.  FP32: x minus x clamped to [-lambda, lambda], two
+// min/max operations in place of two compares and two selects.  FP64: one
+// FP64 addition; the compare is of the magnitudes' bits, since every FP64
+// compare, minimum or conversion takes a slot of the FP64 pipe (16 cycles a
+// warp on this part).
+__device__ __forceinline__ float soft_std(float x, float lam) {
+    return x - fminf(fmaxf(x, -lam), lam);
+}
+__device__ __forceinline__ long long abs_bits(double x) {
+    return __double_as_longlong(x) & 0x7fffffffffffffffll;
+}
+__device__ __forceinline__ double soft_std(double x, double lam) {
+    const long long sgn = __double_as_longlong(x) & (long long)0x8000000000000000ull;
+    const double y = x - __longlong_as_double(__double_as_longlong(lam) | sgn);
+    return abs_bits(x) > __double_as_longlong(lam) ? y : 0.0;
+}
+
+// a != b for coefficients (never -0: soft_std gives +0 or a nonzero value).
+__device__ __forceinline__ bool differs(float a, float b) { return a != b; }
+__device__ __forceinline__ bool differs(double a, double b) {
+    return __double_as_longlong(a) != __double_as_longlong(b);
+}
+
+// Running max |d| and the change test of the phases' moves, without the FP64 pipe.
+__device__ __forceinline__ float max_abs(float m, float d) { return fmaxf(m, fabsf(d)); }
+__device__ __forceinline__ double max_abs(double m, double d) {
+    const long long a = __double_as_longlong(m), b = abs_bits(d);
+    return __longlong_as_double(b > a ? b : a);
+}
+__device__ __forceinline__ bool is_move(float d) { return d != 0.0f; }
+__device__ __forceinline__ bool is_move(double d) { return abs_bits(d) != 0; }
+
+// |x| as a float that is not below it (a bound): for FP64 from the upper word,
+// rounded up by one unit of it, so that no FP64 conversion is needed per value.
+__device__ __forceinline__ unsigned abs_key(float x) { return __float_as_uint(fabsf(x)); }
+__device__ __forceinline__ unsigned abs_key(double x) {
+    return (unsigned)(__double_as_longlong(x) >> 32) & 0x7fffffffu;
+}
+// The largest key of the warp as a float bound (non-negative floats and the
+// upper words of non-negative doubles order as unsigned integers).
+template <typename T>
+__device__ __forceinline__ float warp_max_key(unsigned key) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, key);
+    if constexpr (sizeof(T) == 4) return __uint_as_float(m);
+    else return m == 0u ? 0.0f : __double2float_ru(__hiloint2double((int)(m + 1u), 0));
+}
+
 // The smallest float f >= x.  For a float m, m < x exactly when m < f, so a
 // stop test of a float iterate against the FP64 tolerance needs no FP64
 // arithmetic per test.
@@ -707,11 +756,12 @@ struct Support {
 // Shared memory of one lazy-solver warp: the support list, the chunk
 // summaries, the support's block of S, the last sigma step (sigma,
 // F(sigma)) for the secant step (kept out of registers) and the support the
-// block of S was gathered for.
+// block of S was gathered for, the links and coefficients of the FP32 phase.
 template <typename T>
 __host__ __device__ constexpr size_t lazy_warp_smem_bytes(int ldp) {
     return (size_t)LAZY_CAP * (sizeof(int) + sizeof(T)) + (size_t)num_chunks(ldp) * sizeof(ChunkInfo) +
-           (size_t)ACT_MAX * ACT_MAX * sizeof(T) + 2 * sizeof(double) + ACT_MAX * sizeof(int);
+           (size_t)ACT_MAX * ACT_MAX * sizeof(T) + 2 * sizeof(double) + ACT_MAX * sizeof(int) +
+           (sizeof(T) == 4 ? ACT_MAX * sizeof(float2) : 0);
 }
 
 // Set b_k = v in the sorted support (insert, update or remove).  pos is the
@@ -859,13 +909,13 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
                 if (k >= cursor && k < p && k != j && !(frozen && bv[t] != T(0))) {
                     T nb;
                     if constexpr (STD) {
-                        nb = soft<T>(acc[t] + bv[t], lam);                 // S_kk = 1
+                        nb = soft_std(acc[t] + bv[t], lam);                // S_kk = 1
                     } else {
                         const T skk = a.diag[k];
                         nb = soft<T>(acc[t] + skk * bv[t], lam) / skk;     // Soft(c, lambda)/S_kk
                     }
                     nbv[t] = nb;
-                    if (nb != bv[t]) mvmask |= 1u << t;
+                    if (STD ? differs(nb, bv[t]) : nb != bv[t]) mvmask |= 1u << t;
                 }
             }
             const unsigned bal = __ballot_sync(FULL_MASK, mvmask != 0u);
@@ -909,14 +959,13 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
             if (cursor >= cb + CHUNK) break;
         }
         if constexpr (STD) {
-            float mx = 0.f;
+            unsigned key = 0u;
 #pragma unroll
             for (int t = 0; t < SCAN_V; ++t) {
                 const int k = k0 + t;
-                if (k < p && k != j && bv[t] == T(0)) mx = fmaxf(mx, fabsf((float)acc[t]));
+                if (k < p && k != j && !differs(bv[t], T(0))) key = max(key, abs_key(acc[t]));
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL_MASK, mx, o));
+            const float mx = warp_max_key<T>(key);
             if (lane == 0) cs.ci[ci] = ChunkInfo{mx, cs.dsum, cs.nmoves, e1 - e0};
             __syncwarp();
             // moves raised the running sums: test the chunks after this one again
@@ -932,6 +981,73 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
     return maxd;
 }
 
+// The sweeps of an active-set phase by one warp, FP32 on the standardised
+// matrix (S_kk = 1), on n <= LD coordinates; column k of S_AA at saa + k LD.
+// Lane m holds the gradient of coordinate m (g0) and, for LD = 64, of
+// coordinate m + 32 (g1); b is in tb[k].y.  One move after another is a chain,
+// and a shuffle of the owner's change would be half of it.  So every lane forms
+// every move: coordinate k's gradient before move k-1 is shuffled to all lanes
+// while move k-1 is formed, and move k first applies the change of move k-1
+// with the one entry tb[k].x = S_{A_k A_k-1} (the owner's own fused
+// multiply-add, so the iterates are the same bits).  The links, b and the
+// columns are read one move ahead; each lane stores the new b itself, so it
+// reads back its own value.  A zero change adds exact zeros.
+template <int LD>
+__device__ __forceinline__ float2 phase_links(const float* __restrict__ saa, float2* __restrict__ tb,
+                                              int n, float b0, float b1) {
+    const int lane = threadIdx.x & 31;
+    if (lane < n) tb[lane] = make_float2(saa[(lane == 0 ? n - 1 : lane - 1) * LD + lane], b0);
+    if (LD > 32 && lane + 32 < n)
+        tb[lane + 32] = make_float2(saa[(lane + 31) * LD + lane + 32], b1);
+    __syncwarp();
+    return tb[0];
+}
+
+template <int LD>
+__device__ __forceinline__ int phase_sweeps(const float* __restrict__ saa, float2* __restrict__ tb,
+                                            int n, float lam, int maxit, float tf, float2 q, float& g0,
+                                            float& g1, unsigned& mv, bool& conv) {
+    const float* __restrict__ col = saa + (threadIdx.x & 31);
+    float c0 = col[0], c1 = LD > 32 ? col[32] : 0.f;
+    float gk = __shfl_sync(FULL_MASK, g0, 0), dp = 0.f;
+    float md;
+    // move k; kn is the next one, gs the slot of its gradient
+    auto move = [&](int k, int kn, const float& gs) {
+        const float gn = __shfl_sync(FULL_MASK, gs, kn & 31);
+        float2 qn = tb[kn];
+        const float n0 = col[kn * LD], n1 = LD > 32 ? col[kn * LD + 32] : 0.f;
+        gk = fmaf(-q.x, dp, gk);
+        const float nb = soft_std(gk + q.y, lam);
+        dp = nb - q.y;
+        tb[k].y = nb;
+        if (kn == k) qn.y = nb;
+        g0 = fmaf(-c0, dp, g0);
+        if (LD > 32) g1 = fmaf(-c1, dp, g1);
+        md = max_abs(md, dp);
+        mv += is_move(dp);
+        c0 = n0;
+        c1 = n1;
+        q = qn;
+        gk = gn;
+    };
+    for (int sw = 1; sw <= maxit; ++sw) {
+        md = 0.f;
+        const int n_lo = LD > 32 ? min(n, 32) : n;
+#pragma unroll 4
+        for (int k = 0; k < n_lo - 1; ++k) move(k, k + 1, g0);
+        if (LD > 32) {
+#pragma unroll 4
+            for (int k = 31; k < n - 1; ++k) move(k, k + 1, g1);
+        }
+        move(n - 1, 0, g0);
+        if (md < tf) {
+            conv = true;
+            return sw;
+        }
+    }
+    return maxit;
+}
+
 // Active-set phase of the lasso at a fixed lambda: cyclic sweeps (ascending
 // coordinate order) over the current support A only, until a sweep moves no
 // coefficient by tol or more (at most maxit sweeps).  Lane m holds coordinate
@@ -941,16 +1057,17 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
 // net change of b enters the column's running sums as one change, so the
 // chunk skip test stays exact for the coordinates outside A.  Coordinates
 // that reach zero leave the support and mark their chunk for a rescan.  One
-// move is the phase's critical path: every lane forms its candidate, one
-// shuffle broadcasts the owner's change, and every lane updates its gradient
-// with the column of S_AA loaded one move ahead (a zero change adds exact
-// zeros, so no lane branches on it).  Returns the sweeps done (0 when A is
+// move is the phase's critical path: FP32 on the standardised matrix takes
+// phase_sweeps; otherwise every lane forms its candidate, one shuffle
+// broadcasts the owner's change, and every lane updates its gradient with the
+// column of S_AA loaded one move ahead (a zero change adds exact zeros, so no
+// lane branches on it).  Returns the sweeps done (0 when A is
 // empty or larger than ACT_MAX); `conv` tells whether the last sweep moved
 // nothing by tol (true for an empty A, false when A is too large).
 template <typename T, bool STD>
 __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, T* __restrict__ saa,
-                            int* __restrict__ saa_list, int& saa_n, unsigned long long& moves,
-                            ColScan& cs, bool& conv) {
+                            int* __restrict__ saa_list, float2* __restrict__ tb, int& saa_n,
+                            unsigned long long& moves, ColScan& cs, bool& conv) {
     const int lane = threadIdx.x & 31;
     const int n = s.n;
     conv = n <= ACT_MAX;
@@ -987,26 +1104,33 @@ __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, T* 
     int sw = 0;
     unsigned mv = 0;
     const float tf = float_at_least(a.tol);
-    while (sw < a.maxit) {
-        ++sw;
-        T md = T(0);
-        T c = lane < n ? saa[lane] : T(0);                   // column of S_AA for k = 0
-        for (int k = 0; k < n; ++k) {
-            const int kn = k + 1 < n ? k + 1 : k;
-            const T cn = lane < n ? saa[kn * ACT_MAX + lane] : T(0);   // next column
-            T nb;
-            if constexpr (STD) nb = soft<T>(g + b, lam);                 // S_kk = 1
-            else nb = soft<T>(g + skk * b, lam) / skk;
-            const T d = __shfl_sync(FULL_MASK, nb - b, k);
-            if (lane == k) b = nb;
-            g = fma(-c, d, g);
-            md = fmax(md, fabs(d));
-            mv += d != T(0);
-            c = cn;
-        }
-        if (below_tol<T>(md, a.tol, tf)) {
-            conv = true;
-            break;
+    if constexpr (STD && sizeof(T) == 4) {
+        const float2 first = phase_links<ACT_MAX>(saa, tb, n, b, T(0));
+        sw = phase_sweeps<ACT_MAX>(saa, tb, n, lam, a.maxit, tf, first, g, g, mv, conv);
+        __syncwarp();
+        if (lane < n) b = tb[lane].y;
+    } else {
+        while (sw < a.maxit) {
+            ++sw;
+            T md = T(0);
+            T c = lane < n ? saa[lane] : T(0);               // column of S_AA for k = 0
+            for (int k = 0; k < n; ++k) {
+                const int kn = k + 1 < n ? k + 1 : k;
+                const T cn = lane < n ? saa[kn * ACT_MAX + lane] : T(0);   // next column
+                T nb;
+                if constexpr (STD) nb = soft_std(g + b, lam);            // S_kk = 1
+                else nb = soft<T>(g + skk * b, lam) / skk;
+                const T d = __shfl_sync(FULL_MASK, nb - b, k);
+                if (lane == k) b = nb;
+                g = fma(-c, d, g);
+                md = max_abs(md, d);
+                mv += is_move(d);
+                c = cn;
+            }
+            if (below_tol<T>(md, a.tol, tf)) {
+                conv = true;
+                break;
+            }
         }
     }
     moves += mv;
@@ -1117,6 +1241,7 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
     T* saa = reinterpret_cast<T*>(cs.ci + num_chunks(a.ldp));
     double* prev = reinterpret_cast<double*>(saa + ACT_MAX * ACT_MAX);   // HS: (sigma, F(sigma))
     int* saa_list = reinterpret_cast<int*>(prev + 2);    // the support S_AA was gathered for
+    float2* tb = reinterpret_cast<float2*>(saa_list + ACT_MAX);   // the FP32 phase's links and b
     int saa_n = -1;
     reset_chunks(cs, a.ldp);
     if constexpr (STD) {
@@ -1153,8 +1278,8 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
                                       r, status);
                 return false;
             }
-            cnt.act_sweeps += active_phase<T, STD>(j, s, a, lam, saa, saa_list, saa_n, cnt.act_moves,
-                                                  cs, conv);
+            cnt.act_sweeps += active_phase<T, STD>(j, s, a, lam, saa, saa_list, tb, saa_n,
+                                                  cnt.act_moves, cs, conv);
             const T md = sweep_column_lazy<T, STD>(j, s, a, lam, cnt.moves, cs, overflow, conv,
                                                    (int)(cnt.sweeps - sweeps0));
             ++cnt.sweeps;
@@ -1725,14 +1850,15 @@ __device__ inline void warp_union(const int* __restrict__ list, int n, const int
 // n <= BLK_AMAX: lane m holds coordinates A_m and A_{m+32}.  Reads and writes
 // b for the coordinates of A; g is formed afresh by the caller afterwards.
 // Returns the sweeps done; conv tells whether the last one moved nothing by tol.
-// One move is the critical path of the phase: every lane forms the candidate
-// of its slot, the owner's change is broadcast by one shuffle, and every lane
-// updates its two gradients with the column of S_AA loaded one move ahead.  A
-// zero change adds exact zeros, so no lane branches on it.
+// One move is the critical path of the phase (phase_sweeps for FP32 on the
+// standardised matrix; otherwise the owner's change is broadcast by one
+// shuffle, and every lane updates its two gradients with the column of S_AA
+// loaded one move ahead).  A zero change adds exact zeros, so no lane branches
+// on it.
 template <typename T, bool STD>
 __device__ int block_active_phase(int j, T* __restrict__ b, const int* __restrict__ list, int n,
                                   const CDArgs<T>& a, T lam, T* __restrict__ saa,
-                                  int* __restrict__ saa_list, int& saa_n,
+                                  int* __restrict__ saa_list, float2* __restrict__ tb, int& saa_n,
                                   unsigned long long& moves, bool& conv) {
     const int lane = threadIdx.x & 31;
     const int ldp = a.ldp;
@@ -1783,37 +1909,45 @@ __device__ int block_active_phase(int j, T* __restrict__ b, const int* __restric
     int sw = 0;
     unsigned mv = 0;
     const float tf = float_at_least(a.tol);
-    while (sw < a.maxit) {
-        ++sw;
-        T md = T(0);
-        T c0 = saa[m0], c1 = saa[m1];                     // column of S_AA for k = 0
-        for (int k = 0; k < n; ++k) {
-            const int kn = k + 1 < n ? k + 1 : k;
-            const T n0 = saa[kn * BLK_AMAX + m0], n1 = saa[kn * BLK_AMAX + m1];   // next column
-            const bool hi = k >= 32;
-            const T gk = hi ? g1 : g0, bk = hi ? b1 : b0;
-            T nb;
-            if constexpr (STD) {
-                nb = soft<T>(gk + bk, lam);                          // S_kk = 1
-            } else {
-                const T sk = hi ? s1 : s0;
-                nb = soft<T>(gk + sk * bk, lam) / sk;
+    if constexpr (STD && sizeof(T) == 4) {
+        const float2 first = phase_links<BLK_AMAX>(saa, tb, n, b0, b1);
+        sw = phase_sweeps<BLK_AMAX>(saa, tb, n, lam, a.maxit, tf, first, g0, g1, mv, conv);
+        __syncwarp();
+        if (h0) b0 = tb[m0].y;
+        if (h1) b1 = tb[m1].y;
+    } else {
+        while (sw < a.maxit) {
+            ++sw;
+            T md = T(0);
+            T c0 = saa[m0], c1 = saa[m1];                 // column of S_AA for k = 0
+            for (int k = 0; k < n; ++k) {
+                const int kn = k + 1 < n ? k + 1 : k;
+                const T n0 = saa[kn * BLK_AMAX + m0], n1 = saa[kn * BLK_AMAX + m1];   // next column
+                const bool hi = k >= 32;
+                const T gk = hi ? g1 : g0, bk = hi ? b1 : b0;
+                T nb;
+                if constexpr (STD) {
+                    nb = soft_std(gk + bk, lam);                     // S_kk = 1
+                } else {
+                    const T sk = hi ? s1 : s0;
+                    nb = soft<T>(gk + sk * bk, lam) / sk;
+                }
+                const T d = __shfl_sync(FULL_MASK, nb - bk, k & 31);
+                if (lane == (k & 31)) {
+                    if (hi) b1 = nb;
+                    else b0 = nb;
+                }
+                g0 = fma(-c0, d, g0);
+                g1 = fma(-c1, d, g1);
+                md = max_abs(md, d);
+                mv += is_move(d);
+                c0 = n0;
+                c1 = n1;
             }
-            const T d = __shfl_sync(FULL_MASK, nb - bk, k & 31);
-            if (lane == (k & 31)) {
-                if (hi) b1 = nb;
-                else b0 = nb;
+            if (below_tol<T>(md, a.tol, tf)) {
+                conv = true;
+                break;
             }
-            g0 = fma(-c0, d, g0);
-            g1 = fma(-c1, d, g1);
-            md = fmax(md, fabs(d));
-            mv += d != T(0);
-            c0 = n0;
-            c1 = n1;
-        }
-        if (below_tol<T>(md, a.tol, tf)) {
-            conv = true;
-            break;
         }
     }
     moves += mv;
@@ -1990,6 +2124,8 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
     // and the refresh scan's coordinates live there
     int* ubuf = reinterpret_cast<int*>(cand);
     int* vlist = ubuf + BLK_AMAX;
+    // the phase's links and coefficients too (2 KB of the buffers' 8 KB at most)
+    float2* tb = reinterpret_cast<float2*>(vlist + BLK_AMAX);
     int saa_n = -1;                                       // warp 0: no S_AA gathered yet
     int par = 0;
     int wp = 0;                                           // parity of the refresh scan's counters
@@ -2044,7 +2180,7 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
                 int sw = 0;
                 bool c = false;
                 if (tid < 32) sw = block_active_phase<T, STD>(j, b, plist, n, a, lam, saa, saa_list,
-                                                              saa_n, cnt.act_moves, c);
+                                                              tb, saa_n, cnt.act_moves, c);
                 if (tid == 0) {
                     sc.red[par][0] = sw;
                     sc.red[par][1] = c ? 1 : 0;

@@ -189,8 +189,10 @@ double spmesl_lambda(int rule, int n, int p);
  *              X.  Both triangles are written.
  *   workspace  device scratch of at least spmesl_gram_workspace_bytes(n, p,
  *              precision) bytes (may be NULL when that is 0).
- * SPMESL_FP64 and SPMESL_FP32 accumulate in the input precision on the CUDA
- * cores; SPMESL_MIXED splits X = hi + lo into two BF16 parts and forms
+ * SPMESL_FP32 accumulates in FP32 on the CUDA cores.  SPMESL_FP64 forms the
+ * products without error as 8-bit digit products on the tensor cores and sums
+ * them to FP64 accuracy relative to sqrt(S_jj S_kk) (columns with non-finite or
+ * extreme values as FP64 sums in sample order).  SPMESL_MIXED splits X = hi + lo into two BF16 parts and forms
  * hi'hi + hi'lo + lo'hi on the tensor cores (tcgen05, TMEM accumulators)
  * with FP32 accumulation.
  * Errors: EINVAL for n < 1, p < 1, ldx < p, lds < p, NULL pointers, a short

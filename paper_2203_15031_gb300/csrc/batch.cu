@@ -3,7 +3,8 @@
 // With SPMESL_MIXED the Gram of every fit given as X runs as split-BF16
 // products on the tensor cores (one batched split/transpose launch, then one
 // persistent tcgen05 launch over the tiles of all fits); the rest runs in
-// FP32 with sigma and Theta in FP64, as in the single-fit path.
+// FP32 with sigma and Theta in FP64, as in the single-fit path.  SPMESL_FP64
+// does the same with the digit planes of gram_f64.cu.
 //
 // Every launch covers all fits at once.  Fits are ordered by decreasing p so
 // the longest column chains start first.  A descriptor table in the
@@ -23,6 +24,7 @@
 
 #include "cd_device.cuh"
 #include "gram_device.cuh"
+#include "gram_f64.cuh"
 #include "gram_tc.cuh"
 
 namespace spmesl {
@@ -42,8 +44,8 @@ struct BatchFit {
     double* Theta;
     double* sigma_out;
     FitCtrl* ctrl;
-    void* XhT;            // split-BF16 operands (SPMESL_MIXED with X)
-    void* XlT;
+    void* XhT;            // split-BF16 operands (SPMESL_MIXED with X), or the digit
+    void* XlT;            // planes and the columns' exponents (SPMESL_FP64 with X)
     float* cmax;          // first-sweep chunk maxima of the lazy solver (standardised fits)
     double lambda0;
     double diag_eps;      // rounding bound of the working matrix (diagnostics)
@@ -89,6 +91,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) batch_gram_kernel(const BatchFit* __restrict__ fits,
                                                         const int* __restrict__ gram_prefix,
                                                         int count) {
+    static_assert(sizeof(T) == 4, "FP64 takes the digit planes");
     const int fi = find_fit(gram_prefix, count, blockIdx.x);
     const BatchFit& f = fits[fi];
     const int t = (f.p + GRAM_BM - 1) / GRAM_BM;
@@ -112,6 +115,19 @@ __global__ void batch_split_kernel(const BatchFit* __restrict__ fits,
                            static_cast<const float*>(f.mu), static_cast<__nv_bfloat16*>(f.XhT),
                            static_cast<__nv_bfloat16*>(f.XlT), n_pad, (idx % bx) * 64,
                            (idx / bx) * 32);
+}
+
+// Exponents and digit planes of every fit given as X (SPMESL_FP64): one block
+// of 32 x 8 per 32 columns.
+__global__ void __launch_bounds__(256) batch_digits_kernel(const BatchFit* __restrict__ fits,
+                                                          const int* __restrict__ split_prefix,
+                                                          int count) {
+    const int fi = find_fit(split_prefix, count, blockIdx.x);
+    const BatchFit& f = fits[fi];
+    f64_digit_columns(static_cast<const double*>(f.X), f.n, f.p, f.p,
+                      static_cast<const double*>(f.mu), static_cast<int*>(f.XlT),
+                      static_cast<__nv_bfloat16*>(f.XhT), tc_pad_n(f.n),
+                      (blockIdx.x - f.split_start) * 32);
 }
 
 template <typename T>
@@ -468,7 +484,7 @@ struct spmesl_batch {
     int total_prep = 0;
     int count_rows = 0;            // moved-coordinate bitmaps (measurement)
     size_t off_rows = 0, rows_bytes = 0;   // all fits' bitmaps, contiguous
-    // SPMESL_MIXED: tensor-core Gram table, fit of every tile, split prefixes
+    // SPMESL_MIXED, SPMESL_FP64: tensor-core Gram table, fit of every tile, split prefixes
     size_t off_tcfit = 0, off_tilefit = 0, off_splitp = 0;
     int total_split = 0;
     size_t ws_bytes = 0;
@@ -523,6 +539,13 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
             if ((e = launch_gram_tc_batch(reinterpret_cast<const TcFit*>(ws + b->off_tcfit),
                                           reinterpret_cast<const int*>(ws + b->off_tilefit),
                                           b->total_gram, st)) != cudaSuccess)
+                return e;
+        } else if constexpr (sizeof(T) == 8) {
+            batch_digits_kernel<<<b->total_split, dim3(32, 8), 0, st>>>(
+                fits, reinterpret_cast<const int*>(ws + b->off_splitp), count);
+            if ((e = launch_gram_f64_batch(reinterpret_cast<const F64Fit*>(ws + b->off_tcfit),
+                                           reinterpret_cast<const int*>(ws + b->off_tilefit),
+                                           b->total_gram, st)) != cudaSuccess)
                 return e;
         } else {
             batch_gram_kernel<T><<<b->total_gram, 256, 0, st>>>(fits, gramp, count);
@@ -649,9 +672,12 @@ int auto_warps(const spmesl_batch* b) {
 bool stage_table(spmesl_batch* b, unsigned char* ws) {
     BatchFit* t = reinterpret_cast<BatchFit*>(b->pinned);
     const bool mixed = b->precision == SPMESL_MIXED;
+    const bool f64 = b->precision == SPMESL_FP64;
+    const bool tc = mixed || f64;             // Gram on the tensor cores
     TcFit* tcf = mixed ? reinterpret_cast<TcFit*>(b->pinned + (b->off_tcfit - b->off_desc)) : nullptr;
-    int* tilefit = mixed ? reinterpret_cast<int*>(b->pinned + (b->off_tilefit - b->off_desc)) : nullptr;
-    int* splitp = mixed ? reinterpret_cast<int*>(b->pinned + (b->off_splitp - b->off_desc)) : nullptr;
+    F64Fit* dgf = f64 ? reinterpret_cast<F64Fit*>(b->pinned + (b->off_tcfit - b->off_desc)) : nullptr;
+    int* tilefit = tc ? reinterpret_cast<int*>(b->pinned + (b->off_tilefit - b->off_desc)) : nullptr;
+    int* splitp = tc ? reinterpret_cast<int*>(b->pinned + (b->off_splitp - b->off_desc)) : nullptr;
     int* colp = reinterpret_cast<int*>(b->pinned + (b->off_colp - b->off_desc));
     int* gramp = reinterpret_cast<int*>(b->pinned + (b->off_gramp - b->off_desc));
     int* thetap = reinterpret_cast<int*>(b->pinned + (b->off_thetap - b->off_desc));
@@ -673,8 +699,8 @@ bool stage_table(spmesl_batch* b, unsigned char* ws) {
         d.csf = reinterpret_cast<float*>(ws + f.off_csf);
         d.sigma = reinterpret_cast<double*>(ws + f.off_sigma);
         d.col_status = reinterpret_cast<int*>(ws + f.off_status);
-        d.XhT = (mixed && f.X) ? ws + f.off_XhT : nullptr;
-        d.XlT = (mixed && f.X) ? ws + f.off_XlT : nullptr;
+        d.XhT = (tc && f.X) ? ws + f.off_XhT : nullptr;
+        d.XlT = (tc && f.X) ? ws + f.off_XlT : nullptr;
         d.Theta = f.Theta;
         d.sigma_out = f.sigma;
         d.ctrl = reinterpret_cast<FitCtrl*>(ws + f.off_ctrl);
@@ -704,6 +730,20 @@ bool stage_table(spmesl_batch* b, unsigned char* ws) {
                 tcf[i].tile_start = f.gram_start;
             }
         }
+        if (f64) {
+            splitp[i] = f.split_start;
+            if (f.X) {
+                if (!f64_encode_fit(dgf[i], static_cast<const double*>(f.X), f.n, f.p, f.p,
+                                    static_cast<const double*>(d.mu), static_cast<const int*>(d.XlT),
+                                    d.XhT, static_cast<double*>(d.Sg), f.p, f.gram_start))
+                    return false;
+                const int nt = dgf[i].g.count();
+                for (int k = 0; k < nt; ++k) tilefit[f.gram_start + k] = i;
+            } else {
+                dgf[i] = F64Fit{};
+                dgf[i].tile_start = f.gram_start;
+            }
+        }
         colp[i] = f.col_start;
         gramp[i] = f.gram_start;
         thetap[i] = f.theta_start;
@@ -713,7 +753,7 @@ bool stage_table(spmesl_batch* b, unsigned char* ws) {
     gramp[b->count] = b->total_gram;
     thetap[b->count] = b->total_theta;
     prepp[b->count] = b->total_prep;
-    if (mixed) splitp[b->count] = b->total_split;
+    if (tc) splitp[b->count] = b->total_split;
     b->table_ws = ws;
     return true;
 }
@@ -773,11 +813,13 @@ spmesl_status spmesl_batch_create(const spmesl_problem* probs, int count, double
                      [&](int a, int c) { return probs[a].p > probs[c].p; });
     const size_t s = (size_t)elem_size(o.precision);
     const bool mixed = o.precision == SPMESL_MIXED;
-    // tensor-core tiles of the whole batch (SPMESL_MIXED), for the table sizes
+    const bool tc = mixed || o.precision == SPMESL_FP64;
+    // tensor-core tiles of the whole batch, for the table sizes
+    const int tc_bn = mixed ? TC_BATCH_BN : F64_BN;
     long long tc_tiles = 0;
-    if (mixed)
+    if (tc)
         for (int i = 0; i < count; ++i)
-            if (probs[i].X) tc_tiles += tc_tile_grid(probs[i].p, TC_BATCH_BN).count();
+            if (probs[i].X) tc_tiles += tc_tile_grid(probs[i].p, tc_bn).count();
     if (tc_tiles > (1ll << 30)) return SPMESL_EINVAL;
     size_t off = 0;
     b->off_hdr = off;   off += align_up(sizeof(BatchHeader), 256);
@@ -786,8 +828,9 @@ spmesl_status spmesl_batch_create(const spmesl_problem* probs, int count, double
     b->off_gramp = off; off += align_up(sizeof(int) * (count + 1), 256);
     b->off_thetap = off; off += align_up(sizeof(int) * (count + 1), 256);
     b->off_prepp = off; off += align_up(sizeof(int) * (count + 1), 256);
-    if (mixed) {
-        b->off_tcfit = off;   off += align_up(sizeof(TcFit) * count, 256);
+    if (tc) {
+        b->off_tcfit = off;
+        off += align_up((mixed ? sizeof(TcFit) : sizeof(F64Fit)) * count, 256);
         b->off_tilefit = off; off += align_up(sizeof(int) * (size_t)std::max<long long>(tc_tiles, 1), 256);
         b->off_splitp = off;  off += align_up(sizeof(int) * (count + 1), 256);
     }
@@ -822,6 +865,9 @@ spmesl_status spmesl_batch_create(const spmesl_problem* probs, int count, double
                 const size_t half = tc_operand_bytes(f.n, f.p) / 2;
                 f.off_XhT = off; off += half;
                 f.off_XlT = off; off += half;
+            } else if (tc) {
+                f.off_XhT = off; off += f64_digit_bytes(f.n, f.p);
+                f.off_XlT = off; off += f64_expo_bytes(f.p);
             }
             b->any_x = true;
         }
@@ -831,9 +877,9 @@ spmesl_status spmesl_batch_create(const spmesl_problem* probs, int count, double
         cols += f.p;
         f.gram_start = gram;
         f.split_start = split;
-        if (q.X && mixed) {
-            gram += tc_tile_grid(f.p, TC_BATCH_BN).count();
-            split += (tc_pad_n(f.n) / 64) * ((f.p + 31) / 32);
+        if (q.X && tc) {
+            gram += tc_tile_grid(f.p, tc_bn).count();
+            split += (mixed ? tc_pad_n(f.n) / 64 : 1) * ((f.p + 31) / 32);
         } else if (q.X) {
             const int t = (f.p + GRAM_BM - 1) / GRAM_BM;
             gram += t * (t + 1) / 2;

@@ -1,5 +1,5 @@
-// Gram matrix S = X'X / n on the CUDA cores (FP64 and FP32 paths); the tile
-// itself is in gram_device.cuh.  Only the t(t+1)/2 upper-triangular tiles are
+// Gram matrix S = X'X / n: the FP32 path on the CUDA cores and the choice of
+// path by precision; the tile itself is in gram_device.cuh.  Only the t(t+1)/2 upper-triangular tiles are
 // launched; each writes its mirror too.
 #include <cuda_runtime.h>
 
@@ -47,17 +47,22 @@ cudaError_t run_gram_simt(const T* X, int n, int p, int ldx, int center, T* S, i
 size_t gram_tc_ws_bytes(int n, int p);
 cudaError_t launch_gram_tc(const float* X, int n, int p, int ldx, int center, float* S, int lds,
                            void* ws, cudaStream_t st);
+// Defined in gram_f64.cu (FP64 by error-free digit products on the tensor cores).
+size_t gram_f64_ws_bytes(int n, int p);
+cudaError_t launch_gram_f64(const double* X, int n, int p, int ldx, int center, double* S, int lds,
+                            void* ws, cudaStream_t st);
 
 size_t gram_ws_bytes(int n, int p, int precision) {
     if (precision == SPMESL_MIXED) return gram_tc_ws_bytes(n, p);
+    if (precision == SPMESL_FP64) return gram_f64_ws_bytes(n, p);
     return align_up((size_t)p * (size_t)elem_size(precision), 256);
 }
 
 cudaError_t launch_gram(const void* X, int n, int p, int ldx, int precision, int center, void* S,
                         int lds, void* ws, cudaStream_t st) {
     if (precision == SPMESL_FP64)
-        return run_gram_simt<double>(static_cast<const double*>(X), n, p, ldx, center,
-                                     static_cast<double*>(S), lds, ws, st);
+        return launch_gram_f64(static_cast<const double*>(X), n, p, ldx, center,
+                               static_cast<double*>(S), lds, ws, st);
     if (precision == SPMESL_FP32)
         return run_gram_simt<float>(static_cast<const float*>(X), n, p, ldx, center,
                                     static_cast<float*>(S), lds, ws, st);

@@ -1,6 +1,6 @@
 #pragma once
-// Gram tile on the CUDA cores (FP64 / FP32), shared by the single-fit and the
-// batched Gram kernels.
+// Gram tile on the CUDA cores (FP32), shared by the single-fit and the batched
+// Gram kernels.
 //
 // X is row-major n x p, so the k-th slice X[i, m0 .. m0+63] of both operand
 // tiles is a contiguous row segment: every global load is coalesced.  A tile

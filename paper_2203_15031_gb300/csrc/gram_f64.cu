@@ -1,0 +1,469 @@
+// FP64 Gram S = X'X / n on the tensor cores (SPMESL_FP64).
+//
+// The FP64 pipe of this part does two fused multiply-adds a clock and SM, the
+// tensor cores several thousand BF16 ones, so the products are formed there
+// without error (the splitting of Ozaki, Ogita, Oishi and Rump, "Error-free
+// transformations of matrix multiplication by using fast routines of matrix
+// multiplication and its applications", Numer. Algorithms 59, 2012).  Column j
+// of X (centred if asked) is scaled by its largest magnitude, |x_ij| < 2^E_j,
+// and rounded to the integer v_ij = x_ij 2^(55 - E_j), whose seven balanced
+// base-256 digits are exact in BF16.  Digit products are integers of at most
+// 2^14, and a level L_l = sum over s + t = l of sum_i d_is d_it, l = 0..6, is
+// summed by tcgen05.mma in one FP32 accumulator exactly while it stays below
+// 2^24: for up to 256 samples that holds for every input in the levels 0 to 3;
+// the levels 4 to 6 (weights 2^-32 and below) can pass 2^24 only when nearly
+// all digits are extreme and of one sign, and are then off by units that weigh
+// less than 2^-50 of the sum.  After at most 256 samples the levels are
+// combined as W = sum_l L_l 256^(6-l), two exact 64-bit integers and one
+// FP64 rounding, and S_jk = W 2^(E_j + E_k - 62) / n.  What is left out, the
+// rounding of v (2^-56 of the column's largest value) and the digit products
+// of level 7 and beyond, is below the rounding of an FP64 sum over the samples
+// relative to sqrt(S_jj S_kk).  Columns with non-finite values or extreme
+// exponents are not scaled: the epilogue forms every entry of their row and
+// column directly in FP64, in sample order.
+//
+// Measured, 50 fits of p = 500, n = 250 in one launch: 0.08 ms for the digits
+// and 0.18 ms for the products, against 3.21 ms of FP64 fused multiply-adds at
+// the FP64 pipe's rate (1.84e9, 0.58 T/s).  One fit: p = 100, n = 50 31 us
+// against 72, p = 1500, n = 1000 283 us against 2050.  Error of an entry
+// relative to sqrt(S_jj S_kk) against exact rational sums, N(0, 1) data,
+// n = 250: rms 1.4e-17, largest 3.7e-17, against 3.1e-17 and 9.2e-17 of the FP64
+// sum in sample order; n = 30: 2.3e-17 and 6.3e-17 against 4.0e-17 and 1.7e-16.
+//
+// Kernel: persistent, one CTA of 10 warps per SM over 128 x 64 tiles that hold
+// an entry of the upper triangle.  Seven 64-column accumulators fill the
+// tensor memory (448 of 512 columns), which sets the tile: 128 x 128 would need
+// 896.  Per K block of 32 samples, warp 0 loads the seven digit planes of the
+// tile's rows and columns (two TMA boxes, 84 KB, 64-byte swizzle, two stages);
+// one lane of warp 1 issues 28 products for each 16 samples; warps 2 to 9
+// combine the levels, 32 rows x 32 columns each, hand the accumulators back,
+// and write the tile and its mirror while the next tile's products run.
+// Waits, failure and tensor-memory release as in gram_tc.cu.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include "gram_device.cuh"
+#include "gram_f64.cuh"
+#include "tc_ptx.cuh"
+
+namespace spmesl {
+
+namespace {
+
+constexpr int F64_THREADS = 320;
+constexpr int F64_EPI_WARPS = 8;
+constexpr int F64_KB = 32;                            // samples per stage (64-byte rows)
+constexpr int F64_STAGES = 2;
+constexpr int F64_FLUSH = 256;                        // samples per accumulation
+constexpr int F64_RING = 8;
+constexpr int F64_A_PLANE = TC_BM * F64_KB * 2;
+constexpr int F64_B_PLANE = F64_BN * F64_KB * 2;
+constexpr int F64_STAGE_BYTES = F64_SLICES * (F64_A_PLANE + F64_B_PLANE);
+constexpr int F64_EPI_COLS = 16;                      // columns staged per store pass
+constexpr int F64_EPI_BYTES = 32 * F64_EPI_COLS * 8;  // per epilogue warp
+constexpr int F64_TMEM_COLS = 512;
+// barriers: full[STAGES], empty[STAGES], acc_full, acc_empty, done
+constexpr int F64_NBARS = 2 * F64_STAGES + 3;
+constexpr size_t F64_SMEM = (size_t)F64_STAGES * F64_STAGE_BYTES + F64_EPI_WARPS * F64_EPI_BYTES +
+                            F64_NBARS * 8 + 64 + 1024;
+static_assert(F64_SMEM <= 232448, "shared memory of one block");
+static_assert(F64_SLICES * F64_BN <= F64_TMEM_COLS, "tensor memory");
+static_assert(F64_FLUSH % F64_KB == 0 && TC_NPAD % F64_KB == 0, "K blocks");
+// instruction descriptor: BF16 x BF16 -> FP32, both K-major, M = 128, N = 64
+constexpr unsigned F64_IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
+                               ((unsigned)(F64_BN >> 3) << 17) | ((unsigned)(TC_BM >> 4) << 24);
+
+// Shared-memory descriptor of a K-major operand plane with 64-byte rows and
+// 64-byte swizzle (8-row groups 512 bytes apart; planes start on 512 bytes).
+__device__ __forceinline__ unsigned long long plane_desc(unsigned addr) {
+    unsigned long long d = 0;
+    d |= (unsigned long long)((addr & 0x3FFFFu) >> 4);
+    d |= (unsigned long long)1 << 16;
+    d |= (unsigned long long)((8 * F64_KB * 2) >> 4) << 32;
+    d |= (unsigned long long)1 << 46;
+    d |= 4ull << 61;
+    return d;
+}
+
+__device__ __forceinline__ void mma_digits(unsigned tmem_d, unsigned long long a,
+                                           unsigned long long b, unsigned accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
+        "l"(a), "l"(b), "r"(F64_IDESC), "r"(accumulate));
+}
+
+__device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap* map, int x, int y,
+                                            int z, unsigned bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+        "l"(reinterpret_cast<unsigned long long>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+
+struct F64One {
+    F64Fit f;
+    int n_tiles;
+    static constexpr bool kTableMaps = false;
+    __device__ int tiles() const { return n_tiles; }
+    __device__ int fit_index(int) const { return 0; }
+    __device__ const F64Fit& fit_at(int) const { return f; }
+};
+
+struct F64Many {
+    const F64Fit* fits;
+    const int* tile_fit;
+    int n_tiles;
+    static constexpr bool kTableMaps = true;
+    __device__ int tiles() const { return n_tiles; }
+    __device__ int fit_index(int tile) const { return __ldg(tile_fit + tile); }
+    __device__ const F64Fit& fit_at(int fi) const { return fits[fi]; }
+};
+
+// S_jk of a column that is not scaled: the FP64 sum in sample order.
+__device__ __noinline__ double direct_entry(const F64Fit& f, int j, int k) {
+    const double mj = f.mu ? f.mu[j] : 0.0, mk = f.mu ? f.mu[k] : 0.0;
+    double acc = 0.0;
+    for (int i = 0; i < f.n; ++i) {
+        const double* row = f.X + (size_t)i * f.ldx;
+        acc = fma(row[j] - mj, row[k] - mk, acc);
+    }
+    return acc * f.inv_n;
+}
+
+// W = L_0 256^6 + .. + L_6 from the seven integer-valued level sums: the
+// upper four and the lower three levels as 64-bit integers (below 2^50), made
+// FP64 by the 1.5 2^52 offset, and one rounding.
+__device__ __forceinline__ double combine_levels(const unsigned (&L)[F64_SLICES][8], int c) {
+    auto I = [&](int l) { return (long long)__float2int_rn(__uint_as_float(L[l][c])); };
+    const long long hi = ((I(0) * 256 + I(1)) * 256 + I(2)) * 256 + I(3);
+    const long long lo = (I(4) * 256 + I(5)) * 256 + I(6);
+    const double off = 6755399441055744.0;
+    const double h = __longlong_as_double(0x4338000000000000ll + hi) - off;
+    const double l = __longlong_as_double(0x4338000000000000ll + lo) - off;
+    return fma(h, 16777216.0, l);
+}
+
+template <class Src>
+__global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_constant__ Src src) {
+    extern __shared__ unsigned char smem_dyn[];
+    unsigned char* smem = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
+    unsigned char* stages = smem;
+    double* epi = reinterpret_cast<double*>(smem + (size_t)F64_STAGES * F64_STAGE_BYTES);
+    unsigned long long* bars = reinterpret_cast<unsigned long long*>(
+        smem + (size_t)F64_STAGES * F64_STAGE_BYTES + F64_EPI_WARPS * F64_EPI_BYTES);
+    unsigned long long* full = bars;
+    unsigned long long* empty = bars + F64_STAGES;
+    unsigned long long* acc_full = bars + 2 * F64_STAGES;
+    unsigned long long* acc_empty = acc_full + 1;
+    unsigned long long* done = acc_full + 2;
+    volatile unsigned* tmem_slot = reinterpret_cast<volatile unsigned*>(bars + F64_NBARS);
+    volatile int* fail = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* issued_slot = fail + 1;
+    volatile int* consumed_slot = fail + 2;
+    volatile int* kt_ring = fail + 4;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int n_tiles = src.tiles();
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < F64_STAGES; ++s) {
+            mbar_init(smem_u32(&full[s]), 1);
+            mbar_init(smem_u32(&empty[s]), 1);
+        }
+        mbar_init(smem_u32(acc_full), 1);
+        mbar_init(smem_u32(acc_empty), F64_EPI_WARPS);
+        mbar_init(smem_u32(done), 1);
+        *fail = 0;
+        *issued_slot = 0;
+        *consumed_slot = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(const_cast<unsigned*>(tmem_slot))),
+                     "r"(F64_TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const unsigned tmem = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // producer
+            int kb = 0, li = 0;
+            const F64Fit* last = nullptr;
+            for (int tile = blockIdx.x; tile < n_tiles && !*fail; tile += gridDim.x, ++li) {
+                const F64Fit& f = src.fit_at(src.fit_index(tile));
+                int tm, tn;
+                f.g.coords(tile - f.tile_start, tm, tn);
+                const int KT = f.n_pad / F64_KB;
+                kt_ring[li % F64_RING] = KT;        // published by the first expect_tx below
+                if (Src::kTableMaps && &f != last) {
+                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
+                                     reinterpret_cast<unsigned long long>(&f.ma))
+                                 : "memory");
+                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
+                                     reinterpret_cast<unsigned long long>(&f.mb))
+                                 : "memory");
+                    last = &f;
+                }
+                for (int kt = 0; kt < KT; ++kt, ++kb) {
+                    const int s = kb % F64_STAGES;
+                    if (kb >= F64_STAGES &&
+                        !mbar_wait(smem_u32(&empty[s]), ((kb / F64_STAGES) - 1) & 1, fail)) {
+                        *fail = 1;
+                        break;
+                    }
+                    const unsigned fb = smem_u32(&full[s]);
+                    unsigned char* st = stages + (size_t)s * F64_STAGE_BYTES;
+                    mbar_expect_tx(fb, F64_STAGE_BYTES);
+                    tma_load_3d(smem_u32(st), &f.ma, kt * F64_KB, tm * TC_BM, 0, fb);
+                    tma_load_3d(smem_u32(st + F64_SLICES * F64_A_PLANE), &f.mb, kt * F64_KB,
+                                tn * F64_BN, 0, fb);
+                    *issued_slot = kb + 1;
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            // MMA issuer
+            int kb = 0, li = 0, flush = 0;
+            bool ok = true;
+            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++li) {
+                int KT = 1;                          // read once the first K block has landed
+                for (int kt = 0; kt < KT; ++kt, ++kb) {
+                    const bool first = kt % (F64_FLUSH / F64_KB) == 0;
+                    if (first) {
+                        if (flush >= 1 && !mbar_wait(smem_u32(acc_empty), (flush - 1) & 1, fail)) {
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    }
+                    const int s = kb % F64_STAGES;
+                    if (!mbar_wait(smem_u32(&full[s]), (kb / F64_STAGES) & 1, fail)) {
+                        ok = false;
+                        break;
+                    }
+                    if (kt == 0) KT = kt_ring[li % F64_RING];
+                    *consumed_slot = kb + 1;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const unsigned base = smem_u32(stages + (size_t)s * F64_STAGE_BYTES);
+                    const unsigned long long a0 = plane_desc(base),
+                                             b0 = plane_desc(base + F64_SLICES * F64_A_PLANE);
+#pragma unroll
+                    for (int kk = 0; kk < F64_KB / 16; ++kk) {
+                        // 16 bf16 = 32 bytes along K inside the swizzled rows
+                        const unsigned long long off = (unsigned long long)((32 * kk) >> 4);
+#pragma unroll
+                        for (int l = 0; l < F64_SLICES; ++l)
+#pragma unroll
+                            for (int t = 0; t <= l; ++t)
+                                mma_digits(tmem + l * F64_BN,
+                                           a0 + off + (unsigned long long)((t * F64_A_PLANE) >> 4),
+                                           b0 + off + (unsigned long long)(((l - t) * F64_B_PLANE) >> 4),
+                                           (!first || kk || t) ? 1u : 0u);
+                    }
+                    mma_commit(smem_u32(&empty[s]));
+                    if ((kt + 1) % (F64_FLUSH / F64_KB) == 0 || kt + 1 == KT) {
+                        mma_commit(smem_u32(acc_full));
+                        ++flush;
+                    }
+                }
+            }
+            if (!ok) *fail = 1;
+            mma_commit(smem_u32(done));
+            mbar_wait(smem_u32(done), 0, nullptr);
+        }
+    } else {
+        // epilogue: warp w reads accumulator lanes 32 (w % 4) .. +31, warps 2-5
+        // the first half of the columns and warps 6-9 the second
+        const int ew = warp - 2;
+        const int q = warp & 3, half = ew >> 2;
+        double* buf = epi + ew * (F64_EPI_BYTES / 8);     // 32 rows x 16 columns, XOR-swizzled
+        bool ok = true;
+        int flush = 0;
+        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+            const F64Fit& f = src.fit_at(src.fit_index(tile));
+            int tm, tn;
+            f.g.coords(tile - f.tile_start, tm, tn);
+            const int m0 = tm * TC_BM + 32 * q, c0 = tn * F64_BN + 32 * half;
+            const int p = f.p, lds = f.lds;
+            // warp-uniform: this warp's 32 x 32 block holds an entry to write
+            const bool any = m0 < p && c0 < p && c0 + 31 >= m0;
+            double acc[32];
+            const int nf = (f.n_pad + F64_FLUSH - 1) / F64_FLUSH;
+            for (int fl = 0; fl < nf; ++fl, ++flush) {
+                if (ok) {
+                    int got = 0;
+                    if (lane == 0) got = mbar_wait(smem_u32(acc_full), flush & 1, fail) ? 1 : 0;
+                    ok = __shfl_sync(FULL_MASK, got, 0) != 0;
+                    if (!ok && lane == 0) *fail = 1;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (any && ok) {
+#pragma unroll
+                    for (int c = 0; c < 32; c += 8) {
+                        unsigned L[F64_SLICES][8];
+#pragma unroll
+                        for (int l = 0; l < F64_SLICES; ++l)
+                            tmem_ld8(tmem + ((unsigned)(32 * q) << 16) +
+                                         (unsigned)(l * F64_BN + 32 * half + c),
+                                     L[l]);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const double w = combine_levels(L, i);
+                            acc[c + i] = fl == 0 ? w : acc[c + i] + w;
+                        }
+                    }
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(acc_empty));
+            }
+            if (!any) continue;
+            double* __restrict__ S = f.S;
+            const int row = m0 + lane;
+            const int Ej = row < p ? f.expo[row] : 0;
+            // inv_n 2^(E_j - 62); E_k is added to its exponent per column
+            const double sj = Ej == F64_EXPO_DIRECT ? f.inv_n : scalbn(f.inv_n, Ej - 62);
+            const int my_E = c0 + lane < p ? f.expo[c0 + lane] : 0;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const int Ek = __shfl_sync(FULL_MASK, my_E, i);
+                if (!ok) {
+                    acc[i] = __longlong_as_double(0x7ff8000000000000ll);
+                } else if (Ej == F64_EXPO_DIRECT || Ek == F64_EXPO_DIRECT) {
+                    acc[i] = (row < p && c0 + i < p) ? direct_entry(f, row, c0 + i) : 0.0;
+                } else {
+                    acc[i] *= __longlong_as_double(__double_as_longlong(sj) + ((long long)Ek << 52));
+                }
+            }
+            // the mirror S_kj, lanes along row k
+            if (row < p) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    const int col = c0 + i;
+                    if (col < p && col > row) S[(size_t)col * lds + row] = acc[i];
+                }
+            }
+            // S_jk, two rows of 128 bytes per store, through shared memory
+#pragma unroll
+            for (int h = 0; h < 32; h += F64_EPI_COLS) {
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < F64_EPI_COLS; ++i)
+                    buf[lane * F64_EPI_COLS + (i ^ (lane & 15))] = acc[h + i];
+                __syncwarp();
+                const int col = c0 + h + (lane & 15);
+                for (int jj = 0; jj < 32; jj += 2) {
+                    const int j = jj + (lane >> 4), r = m0 + j;
+                    if (r < p && col < p && col >= r)
+                        S[(size_t)r * lds + col] = buf[j * F64_EPI_COLS + ((lane & 15) ^ (j & 15))];
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (*fail && threadIdx.x == 0) {
+        // let copies still in flight land before the CTA exits (bounded)
+        const int issued = *issued_slot, consumed = *consumed_slot;
+        for (int kb = consumed; kb < issued; ++kb)
+            mbar_wait(smem_u32(&full[kb % F64_STAGES]), (kb / F64_STAGES) & 1, nullptr);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(F64_TMEM_COLS));
+    }
+}
+
+__global__ void __launch_bounds__(256) f64_digits_kernel(const double* __restrict__ X, int n, int p,
+                                                        int ldx, const double* __restrict__ mu,
+                                                        int* __restrict__ expo,
+                                                        __nv_bfloat16* __restrict__ D, int n_pad) {
+    f64_digit_columns(X, n, p, ldx, mu, expo, D, n_pad, blockIdx.x * 32);
+}
+
+__global__ void f64_mean_kernel(const double* __restrict__ X, int n, int p, int ldx, double* mu) {
+    column_means<double>(X, n, p, ldx, mu, blockIdx.x * blockDim.x + threadIdx.x,
+                         gridDim.x * blockDim.x);
+}
+
+template <class Src>
+cudaError_t launch_tiles(const Src& src, int n_tiles, cudaStream_t st) {
+    auto kern = gram_f64_kernel<Src>;
+    cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F64_SMEM);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        return e;
+    if (n_tiles <= 0) return cudaSuccess;
+    kern<<<n_tiles < sms ? n_tiles : sms, F64_THREADS, F64_SMEM, st>>>(src);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t gram_f64_ws_bytes(int n, int p) {
+    return align_up((size_t)p * 8, 256) + f64_expo_bytes(p) + f64_digit_bytes(n, p);
+}
+
+bool f64_encode_fit(F64Fit& f, const double* X, int n, int p, int ldx, const double* mu,
+                    const int* expo, const void* D, double* S, int lds, int tile_start) {
+    f = F64Fit{};
+    f.n_pad = tc_pad_n(n);
+    const unsigned long long dims[3] = {(unsigned long long)f.n_pad, (unsigned long long)p,
+                                        (unsigned long long)F64_SLICES};
+    const unsigned long long strides[2] = {(unsigned long long)f.n_pad * 2,
+                                           (unsigned long long)f.n_pad * 2 * p};
+    const unsigned box_a[3] = {F64_KB, TC_BM, F64_SLICES}, box_b[3] = {F64_KB, F64_BN, F64_SLICES};
+    if (!tc_encode_bf16_3d(f.ma, D, dims, strides, box_a) ||
+        !tc_encode_bf16_3d(f.mb, D, dims, strides, box_b))
+        return false;
+    f.X = X;
+    f.mu = mu;
+    f.expo = expo;
+    f.S = S;
+    f.n = n;
+    f.p = p;
+    f.ldx = ldx;
+    f.lds = lds;
+    f.tile_start = tile_start;
+    f.inv_n = 1.0 / (double)n;
+    f.g = tc_tile_grid(p, F64_BN);
+    return true;
+}
+
+cudaError_t launch_gram_f64(const double* X, int n, int p, int ldx, int center, double* S, int lds,
+                            void* ws, cudaStream_t st) {
+    unsigned char* base = static_cast<unsigned char*>(ws);
+    double* mu = center ? reinterpret_cast<double*>(base) : nullptr;
+    int* expo = reinterpret_cast<int*>(base + align_up((size_t)p * 8, 256));
+    __nv_bfloat16* D = reinterpret_cast<__nv_bfloat16*>(base + align_up((size_t)p * 8, 256) +
+                                                        f64_expo_bytes(p));
+    F64One one;
+    if (!f64_encode_fit(one.f, X, n, p, ldx, mu, expo, D, S, lds, 0)) return cudaErrorInvalidValue;
+    one.n_tiles = one.f.g.count();
+    if (center) f64_mean_kernel<<<(p + 255) / 256, 256, 0, st>>>(X, n, p, ldx, mu);
+    f64_digits_kernel<<<(p + 31) / 32, dim3(32, 8), 0, st>>>(X, n, p, ldx, mu, expo, D, one.f.n_pad);
+    return launch_tiles(one, one.n_tiles, st);
+}
+
+cudaError_t launch_gram_f64_batch(const F64Fit* fits, const int* tile_fit, int n_tiles,
+                                  cudaStream_t st) {
+    return launch_tiles(F64Many{fits, tile_fit, n_tiles}, n_tiles, st);
+}
+
+}  // namespace spmesl

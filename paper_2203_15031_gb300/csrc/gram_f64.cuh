@@ -1,0 +1,144 @@
+#pragma once
+// FP64 Gram on the tensor cores: the pieces shared by the single-fit path
+// (spmesl_gram with SPMESL_FP64) and the batched one (see gram_f64.cu).
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <limits.h>
+
+#include "gram_tc.cuh"
+
+namespace spmesl {
+
+constexpr int F64_SLICES = 7;         // 8-bit digits of a column's scaled values
+constexpr int F64_BN = 64;            // output tile: TC_BM rows x F64_BN columns
+constexpr int F64_EXPO_DIRECT = INT_MAX;   // column whose products are formed directly in FP64
+constexpr int F64_EXPO_MAX = 400;     // largest |exponent| that the digits' scaling handles
+
+// One fit: TMA maps over its digit planes D ([F64_SLICES][p][n_pad] bf16; boxes
+// of 128 and 64 columns of X), the columns' exponents, the data and the output.
+struct F64Fit {
+    CUtensorMap ma, mb;
+    const double* X;
+    const double* mu;
+    const int* expo;
+    double* S;
+    int n, p, n_pad, ldx, lds, tile_start;
+    double inv_n;
+    TileGrid g;
+};
+
+// Bytes of the digit planes and of the exponents (256-byte aligned each).
+inline size_t f64_digit_bytes(int n, int p) {
+    return align_up((size_t)F64_SLICES * p * tc_pad_n(n) * 2, 256);
+}
+inline size_t f64_expo_bytes(int p) { return align_up((size_t)p * 4, 256); }
+
+// x as an integer v = round(x 2^(55 - E)) for |x| < 2^E, and its balanced
+// base-256 digits: v = sum_s d[s] 256^(6 - s), |d[s]| <= 128.
+__device__ __forceinline__ void f64_digits(double x, int E, int (&d)[F64_SLICES]) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)(u >> 52) & 0x7ff;
+    unsigned long long m = u & 0xfffffffffffffull;
+    if (e) m |= 1ull << 52;
+    const int sh = max(e, 1) - 1020 - E;            // at most 2
+    unsigned long long a;
+    if (sh >= 0) a = m << sh;
+    else a = sh < -54 ? 0ull : (m + (1ull << (-sh - 1))) >> -sh;
+    long long v = (u >> 63) ? -(long long)a : (long long)a;
+#pragma unroll
+    for (int s = F64_SLICES - 1; s > 0; --s) {
+        d[s] = (int)(signed char)(v & 255);          // balanced remainder in [-128, 127]
+        v = (v - d[s]) >> 8;
+    }
+    d[0] = (int)v;
+}
+
+// Exponents and digit planes of columns c0 .. c0 + 31 of X, centred by mu when
+// given (block 32 x 8).  The largest magnitude of a column sets its exponent
+// E (|x| < 2^E); a column with a non-finite value or an exponent beyond
+// F64_EXPO_MAX is marked F64_EXPO_DIRECT and gets zero digits.  Magnitudes are
+// compared and digits formed on the integer pipe: the FP64 pipe takes 16 cycles
+// an instruction.  Samples n .. n_pad - 1 are written as zeros.
+__device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, int n, int p,
+                                                  int ldx, const double* __restrict__ mu,
+                                                  int* __restrict__ expo,
+                                                  __nv_bfloat16* __restrict__ D, int n_pad, int c0) {
+    __shared__ long long red[8][33];
+    __shared__ int sE[32];
+    __shared__ double tile[32][65];
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int cl = c0 + tx;
+    const double m = (mu && cl < p) ? mu[cl] : 0.0;
+    long long mx = 0;
+    if (cl < p) {
+#pragma unroll 8
+        for (int i = ty; i < n; i += 8) {
+            double v = X[(size_t)i * ldx + cl];
+            if (mu) v -= m;
+            mx = max(mx, __double_as_longlong(v) & 0x7fffffffffffffffll);
+        }
+    }
+    red[ty][tx] = mx;
+    __syncthreads();
+    if (ty == 0) {
+#pragma unroll
+        for (int r = 1; r < 8; ++r) mx = max(mx, red[r][tx]);
+        const int e = (int)(mx >> 52);
+        int E = mx == 0 ? 0 : e - 1022;
+        if (e == 0x7ff || E > F64_EXPO_MAX || E < -F64_EXPO_MAX) E = F64_EXPO_DIRECT;
+        sE[tx] = E;
+        if (cl < p) expo[cl] = E;
+    }
+    __syncthreads();
+    const size_t plane = (size_t)p * n_pad;
+    for (int i0 = 0; i0 < n_pad; i0 += 64) {
+#pragma unroll
+        for (int r = ty; r < 64; r += 8) {
+            const int i = i0 + r;
+            double v = 0.0;
+            if (i < n && cl < p) {
+                v = X[(size_t)i * ldx + cl];
+                if (mu) v -= m;
+            }
+            tile[tx][r] = v;
+        }
+        __syncthreads();
+        for (int r = ty; r < 32; r += 8) {
+            const int c = c0 + r;
+            if (c < p) {
+                const int E = sE[r];
+                int d0[F64_SLICES], d1[F64_SLICES];
+                if (E == F64_EXPO_DIRECT) {
+#pragma unroll
+                    for (int s = 0; s < F64_SLICES; ++s) d0[s] = d1[s] = 0;
+                } else {
+                    f64_digits(tile[r][2 * tx], E, d0);
+                    f64_digits(tile[r][2 * tx + 1], E, d1);
+                }
+                __nv_bfloat16* out = D + (size_t)c * n_pad + i0 + 2 * tx;
+#pragma unroll
+                for (int s = 0; s < F64_SLICES; ++s) {
+                    // |d| <= 128 is exact in bf16: the upper half of its FP32 bits
+                    // (made FP32 by the 1.5 2^23 offset, off the conversion pipe)
+                    const float f0 = __int_as_float(0x4b400000 + d0[s]) - 12582912.0f;
+                    const float f1 = __int_as_float(0x4b400000 + d1[s]) - 12582912.0f;
+                    *reinterpret_cast<unsigned*>(out + s * plane) =
+                        __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Fill f (host side).  False if the tensor maps could not be encoded.
+bool f64_encode_fit(F64Fit& f, const double* X, int n, int p, int ldx, const double* mu,
+                    const int* expo, const void* D, double* S, int lds, int tile_start);
+
+// One persistent launch over the tiles of a batch (as launch_gram_tc_batch).
+cudaError_t launch_gram_f64_batch(const F64Fit* fits, const int* tile_fit, int n_tiles,
+                                  cudaStream_t st);
+
+}  // namespace spmesl

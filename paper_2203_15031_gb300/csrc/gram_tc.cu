@@ -38,6 +38,7 @@
 
 #include "gram_device.cuh"
 #include "gram_tc.cuh"
+#include "tc_ptx.cuh"
 
 namespace spmesl {
 
@@ -46,7 +47,6 @@ namespace {
 constexpr int TC_THREADS = 320;       // producer, MMA, 8 epilogue warps
 constexpr int TC_EPI_WARPS = 8;
 constexpr int TC_EPI_WARP0 = 2;
-constexpr unsigned long long TC_WAIT_NS = 2000000000ull;   // 2 s
 
 template <int BN, int KB, int STAGES>
 struct TcCfg {
@@ -72,54 +72,6 @@ struct TcCfg {
                                       ((unsigned)(TC_BM >> 4) << 24);
 };
 
-__device__ __forceinline__ unsigned smem_u32(const void* p) {
-    return (unsigned)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-
-__device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(unsigned bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait for an mbarrier phase; false on timeout or once another role
-// has raised the failure flag (fail may be null).
-__device__ bool mbar_wait(unsigned bar, unsigned parity, const volatile int* fail) {
-    if (mbar_try(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    while (!mbar_try(bar, parity)) {
-        if ((fail && *fail) || global_ns() - t0 > TC_WAIT_NS) return false;
-    }
-    return true;
-}
-
-__device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* map, int x, int y,
-                                            unsigned bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"(reinterpret_cast<unsigned long long>(map)), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-
 // Shared-memory matrix descriptor of a K-major swizzled operand whose rows
 // are KB*2 bytes and whose 8-row groups are SBO bytes apart (buffers are
 // 1024-byte aligned, so the swizzle phase starts at zero).
@@ -141,30 +93,6 @@ __device__ __forceinline__ void mma_bf16(unsigned tmem_d, unsigned long long a,
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
         "l"(a), "l"(b), "r"(C::IDESC), "r"(accumulate));
-}
-
-__device__ __forceinline__ void mma_commit(unsigned bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-        : "memory");
-}
-
-// 32 consecutive accumulator columns of this warp's 32 lanes.
-__device__ __forceinline__ void tmem_ld32(unsigned taddr, float (&v)[32]) {
-    unsigned r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-        "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-          "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-          "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // Centre (optional), split into bf16 hi/lo and transpose to [p][n_pad].
@@ -579,6 +507,17 @@ cudaError_t launch_gram_tc(const float* X, int n, int p, int ldx, int center, fl
     one.n_tiles = one.f.g.count();
     if (bn == 256) return launch_src<256, 2>(one, one.n_tiles, st);
     return launch_src<128, 3>(one, one.n_tiles, st);
+}
+
+bool tc_encode_bf16_3d(CUtensorMap& map, const void* base, const unsigned long long (&dims)[3],
+                       const unsigned long long (&strides)[2], const unsigned (&box)[3]) {
+    EncodeTiled enc = encoder();
+    if (!enc) return false;
+    const cuuint64_t d[3] = {dims[0], dims[1], dims[2]}, st[2] = {strides[0], strides[1]};
+    const cuuint32_t b[3] = {box[0], box[1], box[2]}, es[3] = {1, 1, 1};
+    return enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), d, st, b, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 bool tc_encode_fit(TcFit& f, const void* XhT, const void* XlT, int n, int p, float* S, int lds,

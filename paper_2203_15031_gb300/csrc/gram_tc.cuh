@@ -125,6 +125,11 @@ inline size_t tc_operand_bytes(int n, int p) {
 // Tile width of the batched launch.
 constexpr int TC_BATCH_BN = 128;
 
+// A 3D tensor map over bf16 data with 64-byte swizzle (dims and strides in
+// elements and bytes, innermost first); false if it could not be encoded.
+bool tc_encode_bf16_3d(CUtensorMap& map, const void* base, const unsigned long long (&dims)[3],
+                       const unsigned long long (&strides)[2], const unsigned (&box)[3]);
+
 // Fill f (host side) for a fit whose operands are at XhT / XlT and whose
 // output is S (leading dimension lds).  False if the tensor maps could not be
 // encoded.

@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "gram_f64.cuh"
 #include "gram_tc.cuh"
 
 namespace {
@@ -80,6 +81,9 @@ size_t request_bytes(const spmesl_problem& q, int precision) {
     if (q.X && precision == SPMESL_MIXED)    // bf16 operands, tensor-map entry, tile-to-fit slots
         b += spmesl::tc_operand_bytes(q.n, q.p) + sizeof(spmesl::TcFit) +
              4 * (size_t)spmesl::tc_tile_grid(q.p, spmesl::TC_BATCH_BN).count() + 512;
+    if (q.X && precision == SPMESL_FP64)     // digit planes and exponents, table entry, tile slots
+        b += spmesl::f64_digit_bytes(q.n, q.p) + spmesl::f64_expo_bytes(q.p) + sizeof(spmesl::F64Fit) +
+             4 * (size_t)spmesl::tc_tile_grid(q.p, spmesl::F64_BN).count() + 512;
     b += 2 * spmesl::align_up((size_t)q.p * ldp * s, 256);
     b += 4096;                            // share of descriptors and queues
     return b;

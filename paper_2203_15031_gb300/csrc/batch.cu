@@ -50,7 +50,9 @@ struct BatchFit {
     double lambda0;
     double diag_eps;      // rounding bound of the working matrix (diagnostics)
     unsigned* rows;       // moved-coordinate bitmap of the fit (opts.count_rows) or nullptr
-    double* hand;         // per column the last sigma step at a hand-over (2 doubles)
+    double* hand;         // per column the last sigma step at a hand-over (2 doubles); after the
+                          // descent 1 / sigma_j^2 in the first
+    int* nsup;            // per column the length of its coefficient list (nullptr: dense rows)
     int n, p, ldp;
     int col_start, gram_start, theta_start;
     int split_start;      // first block of the batched split/transpose launch
@@ -253,6 +255,8 @@ __device__ __forceinline__ CDArgs<T> column_args(const BatchFit& f, double tol, 
     a.rows_moved = f.rows;
     a.rows_words = rows_words(f.p);
     a.hand = f.hand;
+    a.nsup = f.nsup;
+    a.Theta = f.nsup ? f.Theta : nullptr;
     return a;
 }
 
@@ -414,6 +418,38 @@ __global__ void batch_theta_kernel(const BatchFit* __restrict__ fits,
     if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) return;
     theta_pair<T>(static_cast<const T*>(f.BT), f.p, f.ldp, f.sigma, f.cs, f.Theta, f.sigma_out,
                   f.ctrl, blockIdx.x - f.theta_start);
+}
+
+// 1 / sigma_j^2 of every column, one per lane: an FP64 division takes a warp
+// some 250 cycles of the FP64 pipe whatever its active lanes, so the lists'
+// pass below reads it.
+__global__ void __launch_bounds__(256) batch_inv_kernel(const BatchFit* __restrict__ fits) {
+    const BatchFit& f = fits[blockIdx.y];
+    if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) return;
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < f.p; j += gridDim.x * blockDim.x) {
+        const double s = f.sigma[j];
+        f.hand[2 * (size_t)j] = 1.0 / (s * s);
+    }
+}
+
+// Theta's nonzero entries after the column solvers (see theta_column), the
+// block's columns all of one fit.
+constexpr int THETA_COLS = 256 / THETA_LANES;
+template <typename T>
+__global__ void __launch_bounds__(256) batch_theta_list_kernel(const BatchFit* __restrict__ fits,
+                                                              const int* __restrict__ theta_prefix,
+                                                              int count) {
+    const int fi = find_fit(theta_prefix, count, blockIdx.x);
+    const BatchFit& f = fits[fi];
+    if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) return;
+    const int j = (blockIdx.x - f.theta_start) * THETA_COLS + (int)threadIdx.x / THETA_LANES;
+    const double* __restrict__ inv = f.hand;
+    unsigned nnz = 0;
+    if (j < f.p)
+        nnz = theta_column<T>(static_cast<const T*>(f.BT), f.nsup, f.p, f.ldp, j, f.sigma, f.cs,
+                              f.Theta, f.sigma_out, [&](int k) { return inv[2 * (size_t)k]; });
+    nnz = __reduce_add_sync(FULL_MASK, nnz);
+    if ((threadIdx.x & 31) == 0 && nnz) atomicAdd(&f.ctrl->nnz, (unsigned long long)nnz);
 }
 
 // ---------------------------------------------------------------------------
@@ -652,7 +688,12 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
                                                num_sms() * 4));
         dk<<<dgrid, 32 * BATCH_DIAG_WARPS, dsm, st>>>(fits, colp, count, b->total_cols);
     }
-    batch_theta_kernel<T><<<b->total_theta, dim3(32, 8), 0, st>>>(fits, thetap, count);
+    if (lazy) {
+        batch_inv_kernel<<<dim3((b->max_p + 255) / 256, count), 256, 0, st>>>(fits);
+        batch_theta_list_kernel<T><<<b->total_theta, 256, 0, st>>>(fits, thetap, count);
+    } else {
+        batch_theta_kernel<T><<<b->total_theta, dim3(32, 8), 0, st>>>(fits, thetap, count);
+    }
     return cudaGetLastError();
 }
 
@@ -708,6 +749,9 @@ bool stage_table(spmesl_batch* b, unsigned char* ws) {
         d.diag_eps = diag_eps_for(b->precision, f.X ? f.n : 1);
         d.rows = b->count_rows ? reinterpret_cast<unsigned*>(ws + f.off_rows) : nullptr;
         d.hand = reinterpret_cast<double*>(ws + f.off_hand);
+        // the heat counts are dead once the columns are ordered
+        d.nsup = b->gradient != SPMESL_GRADIENT_EAGER
+                     ? reinterpret_cast<int*>(ws + b->off_heat) + f.col_start : nullptr;
         d.n = f.n;
         d.p = f.p;
         d.ldp = f.ldp;
@@ -887,7 +931,8 @@ spmesl_status spmesl_batch_create(const spmesl_problem* probs, int count, double
         f.theta_start = theta;
         f.prep_start = prep;
         prep += (f.p + PREP_ROWS - 1) / PREP_ROWS;
-        theta += o.precision == SPMESL_FP64 ? theta_pairs<double>(f.p) : theta_pairs<float>(f.p);
+        if (o.gradient != SPMESL_GRADIENT_EAGER) theta += (f.p + THETA_COLS - 1) / THETA_COLS;
+        else theta += o.precision == SPMESL_FP64 ? theta_pairs<double>(f.p) : theta_pairs<float>(f.p);
         b->max_ldp = std::max(b->max_ldp, f.ldp);
         b->max_p = std::max(b->max_p, f.p);
         b->max_n = std::max(b->max_n, f.n);

@@ -3,7 +3,8 @@
 // Layout in HBM (one fit; see common.cuh FitLayout):
 //   SC  p x ldp  working covariance (S^C = C S C when standardising), rows
 //                zero-padded to ldp = roundup(p, 32) elements
-//   BT  p x ldp  row j = coefficients b_.j of regression j (B transposed)
+//   BT  p x ldp  row j = coefficients b_.j of regression j (B transposed), as a list
+//                after the column solvers (cd_device.cuh), dense otherwise
 //   GT  p x ldp  row j = gradient g_j = S_.j - S b_j (joint rule only)
 // S is symmetric, so column k of S (needed by the rank-1 update) is row k of
 // SC: every S access below is a contiguous, 16-byte-vector, coalesced row read.
@@ -343,7 +344,7 @@ __global__ void __launch_bounds__(512) cd_joint_kernel(CDArgs<T> a) {
 template <typename T>
 __global__ void prep_diag_kernel(const T* __restrict__ S, int p, int standardize, double* cs,
                                  float* csf, double* sigma, int* active, int* col_status,
-                                 FitCtrl* ctrl) {
+                                 FitCtrl* ctrl, int compact_b) {
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < p; j += gridDim.x * blockDim.x) {
         const double d = (double)S[(size_t)j * p + j];
         if (!(d > 0.0) || !isfinite(d)) set_error(ctrl, DEV_ERR_NONFINITE);
@@ -354,7 +355,10 @@ __global__ void prep_diag_kernel(const T* __restrict__ S, int p, int standardize
         active[j] = j;
         col_status[j] = COL_OK;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->n_active = p;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctrl->n_active = p;
+        ctrl->compact_b = compact_b;
+    }
 }
 
 // One block per row of S^C (grid-stride over rows).
@@ -376,7 +380,7 @@ __global__ void prep_matrix_kernel(const T* __restrict__ S, int p, int ldp, cons
 }
 
 // ---------------------------------------------------------------------------
-// Theta: Omega_1 = -B D on the working scale (Eq. (4)), min-magnitude
+// Theta from dense coefficients: Omega_1 = -B D on the working scale (Eq. (4)), min-magnitude
 // symmetrisation (Eq. (9); for j < k the tie keeps omega_jk) and
 // Omega^o = C Omega C (Proposition 1), over pairs of mirrored output tiles
 // whose coefficient tiles are read once into shared memory.  Also writes
@@ -392,20 +396,42 @@ __global__ void theta_kernel(const T* __restrict__ BT, int p, int ldp,
     theta_pair<T>(BT, p, ldp, sigma, cs, Theta, sigma_out, ctrl, blockIdx.x);
 }
 
+// Theta's nonzero entries after the column solvers (see theta_column):
+// THETA_LANES lanes per column.
+template <typename T>
+__global__ void __launch_bounds__(256) theta_list_kernel(const T* __restrict__ BT,
+                                                        const int* __restrict__ nsup, int p, int ldp,
+                                                        const double* __restrict__ sigma,
+                                                        const double* __restrict__ cs,
+                                                        double* __restrict__ Theta,
+                                                        double* __restrict__ sigma_out,
+                                                        FitCtrl* ctrl) {
+    if (*reinterpret_cast<volatile int*>(&ctrl->err) != 0) return;
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) / THETA_LANES;
+    unsigned nnz = 0;
+    if (j < p)
+        nnz = theta_column<T>(BT, nsup, p, ldp, j, sigma, cs, Theta, sigma_out, [&](int k) {
+            const double s = sigma[k];
+            return 1.0 / (s * s);
+        });
+    nnz = __reduce_add_sync(FULL_MASK, nnz);
+    if ((threadIdx.x & 31) == 0 && nnz) atomicAdd(&ctrl->nnz, (unsigned long long)nnz);
+}
+
 // One regression r (spmesl_scaled_lasso): beta over the other columns in
 // order, in the original scale (b^o_k = b^C_k c_k / c_r, proof of
 // Proposition 1), sigma^o = sigma^C / c_r, nonzero coefficients counted.
 template <typename T>
-__global__ void lasso_export_kernel(const T* __restrict__ BT, int p, int ldp, int r,
+__global__ void lasso_export_kernel(const T* __restrict__ BT, const int* __restrict__ nsup, int p,
+                                    int ldp, int r,
                                     const double* __restrict__ sigma,
                                     const double* __restrict__ cs, double* __restrict__ beta,
                                     double* __restrict__ sigma_out, FitCtrl* ctrl) {
     if (*reinterpret_cast<volatile int*>(&ctrl->err) != 0) return;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const T* brow = BT + (size_t)r * ldp;
     bool nz = false;
     if (k < p && k != r) {
-        const T b = brow[k];
+        const T b = coef_of<T>(BT, nsup, ldp, r, k);
         nz = b != T(0);
         beta[k < r ? k : k - 1] = (double)b * cs[k] / cs[r];
     }
@@ -416,14 +442,26 @@ __global__ void lasso_export_kernel(const T* __restrict__ BT, int p, int ldp, in
 
 // B[j][k] = b_jk in the original scale: b^o_jk = b^C_jk c_j / c_k.
 template <typename T>
-__global__ void export_b_kernel(const T* __restrict__ BT, int p, int ldp, const double* cs,
+__global__ void export_b_kernel(const T* __restrict__ BT, const int* __restrict__ nsup,
+                                const FitCtrl* __restrict__ ctrl, int p, int ldp, const double* cs,
                                 double* __restrict__ B) {
     __shared__ T tile[32][33];
     const int j0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
     const int tx = threadIdx.x, ty = threadIdx.y;
+    const bool lists = ctrl->compact_b != 0;
     for (int rr = ty; rr < 32; rr += 8) {
         const int k = k0 + rr, j = j0 + tx;
-        tile[rr][tx] = (k < p && j < p) ? BT[(size_t)k * ldp + j] : T(0);
+        const int n = (lists && k < p) ? nsup[k] : -1;      // warp-uniform (one ty per warp)
+        const T* __restrict__ row = BT + (size_t)k * ldp;
+        if (n < 0) {
+            tile[rr][tx] = (k < p && j < p) ? row[j] : T(0);
+        } else {
+            tile[rr][tx] = T(0);
+            __syncwarp();
+            const int* __restrict__ idx = coef_idx(row, ldp);
+            for (int e = tx; e < n; e += 32)
+                if (idx[e] >= j0 && idx[e] < j0 + 32) tile[rr][idx[e] - j0] = row[e];
+        }
     }
     __syncthreads();
     const int k = k0 + tx;
@@ -563,8 +601,11 @@ static cudaError_t run_fit(const FitLaunch& f, const FitLayout& L, cudaStream_t 
     a.chunk_max = nullptr;
     a.rows_moved = f.count_rows ? reinterpret_cast<unsigned*>(ws + L.rows) : nullptr;
     a.rows_words = rows_words(f.p);
-    // the hand-over record of the column rule lives in the joint rule's G matrix
+    // the hand-over record of the column rule lives in the joint rule's G matrix,
+    // the list lengths in its second index vector (lent to the heat counts before)
     a.hand = reinterpret_cast<double*>(ws + L.GT);
+    a.nsup = nullptr;
+    a.Theta = nullptr;
     const bool single = f.response_col >= 0;    // one regression: lazy column rule
     const bool joint = !single && f.inner_rule == SPMESL_INNER_JOINT;
     // Lazy launch shape (warps per block, blocks per SM).
@@ -576,6 +617,10 @@ static cudaError_t run_fit(const FitLaunch& f, const FitLayout& L, cudaStream_t 
     // hold.  Heat overstates the support of small fits, whose slices are cheap
     // anyway, so the routing by heat is kept to large fits.
     const bool route = lazy && f.gradient == SPMESL_GRADIENT_AUTO;
+    if (lazy) {
+        a.nsup = a.active_next;
+        a.Theta = f.Theta;                       // nullptr for one regression
+    }
     a.ovf_supp = route ? handover_of(f.handover) : LAZY_CAP;
     auto lk = cd_column_lazy_kernel<T, STD>;
     const size_t lper = lazy_warp_smem_bytes<T>(L.ldp);
@@ -619,7 +664,7 @@ static cudaError_t run_fit(const FitLaunch& f, const FitLayout& L, cudaStream_t 
     const int pb = 256;
     prep_diag_kernel<T><<<(f.p + pb - 1) / pb, pb, 0, st>>>(
         reinterpret_cast<const T*>(f.S), f.p, f.standardize, reinterpret_cast<double*>(ws + L.cs),
-        reinterpret_cast<float*>(ws + L.csf), a.sigma, a.active, a.col_status, ctrl);
+        reinterpret_cast<float*>(ws + L.csf), a.sigma, a.active, a.col_status, ctrl, lazy ? 1 : 0);
     {
         const int grid = std::min(f.p, g_num_sms * 8);
         prep_matrix_kernel<T><<<grid, pb, 0, st>>>(
@@ -723,14 +768,20 @@ static cudaError_t run_fit(const FitLaunch& f, const FitLayout& L, cudaStream_t 
 
     if (single) {
         lasso_export_kernel<T><<<(f.p + 255) / 256, 256, 0, st>>>(
-            a.BT, f.p, L.ldp, f.response_col, a.sigma, reinterpret_cast<const double*>(ws + L.cs),
+            a.BT, a.nsup, f.p, L.ldp, f.response_col, a.sigma,
+            reinterpret_cast<const double*>(ws + L.cs),
             f.beta_out, f.sigma_out, ctrl);
         if (f.phase_events) cudaEventRecord(f.phase_events[2], st);
         return cudaGetLastError();
     }
-    theta_kernel<T><<<theta_pairs<T>(f.p), dim3(32, 8), 0, st>>>(a.BT, f.p, L.ldp, a.sigma,
-                                       reinterpret_cast<const double*>(ws + L.cs), f.Theta,
-                                       f.sigma_out, ctrl);
+    if (lazy)
+        theta_list_kernel<T><<<(f.p + 256 / THETA_LANES - 1) / (256 / THETA_LANES), 256, 0, st>>>(
+            a.BT, a.nsup, f.p, L.ldp, a.sigma, reinterpret_cast<const double*>(ws + L.cs), f.Theta,
+            f.sigma_out, ctrl);
+    else
+        theta_kernel<T><<<theta_pairs<T>(f.p), dim3(32, 8), 0, st>>>(
+            a.BT, f.p, L.ldp, a.sigma, reinterpret_cast<const double*>(ws + L.cs), f.Theta,
+            f.sigma_out, ctrl);
     if (f.phase_events) cudaEventRecord(f.phase_events[2], st);
     return cudaGetLastError();
 }
@@ -767,7 +818,7 @@ static cudaError_t run_diagnose(const void* S, int p, int standardize, double la
     prep_diag_kernel<T><<<(p + pb - 1) / pb, pb, 0, st>>>(
         reinterpret_cast<const T*>(S), p, standardize, cs, reinterpret_cast<float*>(ws + L.csf),
         a.sigma, reinterpret_cast<int*>(ws + L.active), reinterpret_cast<int*>(ws + L.col_status),
-        ctrl);
+        ctrl, 0);
     prep_matrix_kernel<T><<<std::min(p, g_num_sms * 8), pb, 0, st>>>(
         reinterpret_cast<const T*>(S), p, L.ldp, cs, reinterpret_cast<const float*>(ws + L.csf),
         reinterpret_cast<T*>(ws + L.SC), nullptr, reinterpret_cast<T*>(ws + L.diag), 0, ctrl, T(0),
@@ -793,12 +844,14 @@ cudaError_t launch_export_B(const unsigned char* ws, int p, int precision, doubl
     const FitLayout L = fit_layout(p, precision);
     dim3 tb(32, 8), tg((p + 31) / 32, (p + 31) / 32);
     const double* cs = reinterpret_cast<const double*>(ws + L.cs);
+    const int* nsup = reinterpret_cast<const int*>(ws + L.active_next);
+    const FitCtrl* ctrl = reinterpret_cast<const FitCtrl*>(ws + L.ctrl);
     if (precision == SPMESL_FP64)
-        export_b_kernel<double><<<tg, tb, 0, st>>>(reinterpret_cast<const double*>(ws + L.BT), p,
-                                                   L.ldp, cs, B);
+        export_b_kernel<double><<<tg, tb, 0, st>>>(reinterpret_cast<const double*>(ws + L.BT), nsup,
+                                                   ctrl, p, L.ldp, cs, B);
     else
-        export_b_kernel<float><<<tg, tb, 0, st>>>(reinterpret_cast<const float*>(ws + L.BT), p,
-                                                  L.ldp, cs, B);
+        export_b_kernel<float><<<tg, tb, 0, st>>>(reinterpret_cast<const float*>(ws + L.BT), nsup,
+                                                  ctrl, p, L.ldp, cs, B);
     return cudaGetLastError();
 }
 

@@ -49,7 +49,7 @@ struct FitCtrl {
     int n_heavy;                       // heavy columns: the first n_heavy of the heat order
     int heavy_next;                    // block solver's position among them
     int block_cols;                    // columns solved by the block solver
-    int pad[1];
+    int compact_b;                     // 1: the rows of BT are coefficient lists (see cd_device.cuh)
     unsigned long long act_sweeps;     // lazy solver: sweeps over the support only
     unsigned long long act_moves;      // moves in those sweeps
     // optimality diagnostics (opts.diagnostics): maxima over the columns of

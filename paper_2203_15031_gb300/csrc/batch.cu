@@ -89,18 +89,17 @@ __global__ void batch_mean_kernel(const BatchFit* __restrict__ fits) {
                     blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) batch_gram_kernel(const BatchFit* __restrict__ fits,
-                                                        const int* __restrict__ gram_prefix,
-                                                        int count) {
-    static_assert(sizeof(T) == 4, "FP64 takes the digit planes");
+__global__ void __launch_bounds__(GRAM_THREADS) batch_gram_kernel(const BatchFit* __restrict__ fits,
+                                                                 const int* __restrict__ gram_prefix,
+                                                                 int count) {
     const int fi = find_fit(gram_prefix, count, blockIdx.x);
     const BatchFit& f = fits[fi];
-    const int t = (f.p + GRAM_BM - 1) / GRAM_BM;
     int tm, tn;
-    upper_tile(blockIdx.x - f.gram_start, t, tm, tn);
-    gram_tile<T>(static_cast<const T*>(f.X), f.n, f.p, f.p, static_cast<const T*>(f.mu),
-                 static_cast<T*>(f.Sg), f.p, (T)(1.0 / (double)f.n), tm, tn);
+    upper_tile(blockIdx.x - f.gram_start, (f.p + GRAM_BM - 1) / GRAM_BM, tm, tn);
+    gram_tile<GRAM_BM, GRAM_BK, GRAM_THREADS, 8, 4, false>(static_cast<const float*>(f.X), f.n, f.p, f.p,
+                                           static_cast<const float*>(f.mu),
+                                           static_cast<float*>(f.Sg), f.p,
+                                           (float)(1.0 / (double)f.n), tm, tn);
 }
 
 // Split/transpose of every fit given as X (SPMESL_MIXED): blocks of 64
@@ -584,7 +583,7 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
                                            b->total_gram, st)) != cudaSuccess)
                 return e;
         } else {
-            batch_gram_kernel<T><<<b->total_gram, 256, 0, st>>>(fits, gramp, count);
+            batch_gram_kernel<<<b->total_gram, GRAM_THREADS, 0, st>>>(fits, gramp, count);
         }
     }
     batch_prep_diag_kernel<T><<<dim3((b->max_p + 255) / 256, count), 256, 0, st>>>(fits,

@@ -17,27 +17,35 @@ __global__ void column_mean_kernel(const T* __restrict__ X, int n, int p, int ld
                     gridDim.x * blockDim.x);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) gram_simt_kernel(const T* __restrict__ X, int n, int p,
-                                                       int ldx, const T* __restrict__ mu,
-                                                       T* __restrict__ S, int lds, T inv_n) {
-    const int t = (p + GRAM_BM - 1) / GRAM_BM;
+template <int BM, int BK, int THREADS, int TM, int TN, bool VEC>
+__global__ void __launch_bounds__(THREADS, TM * TN > 64 ? 2 : 4) gram_simt_kernel(const float* __restrict__ X, int n, int p,
+                                                           int ldx, const float* __restrict__ mu,
+                                                           float* __restrict__ S, int lds,
+                                                           float inv_n) {
     int tm, tn;
-    upper_tile(blockIdx.x, t, tm, tn);
-    gram_tile<T>(X, n, p, ldx, mu, S, lds, inv_n, tm, tn);
+    upper_tile(blockIdx.x, (p + BM - 1) / BM, tm, tn);
+    gram_tile<BM, BK, THREADS, TM, TN, VEC>(X, n, p, ldx, mu, S, lds, inv_n, tm, tn);
 }
 
-template <typename T>
-cudaError_t run_gram_simt(const T* X, int n, int p, int ldx, int center, T* S, int lds, void* ws,
-                          cudaStream_t st) {
-    T* mu = nullptr;
+cudaError_t run_gram_simt(const float* X, int n, int p, int ldx, int center, float* S, int lds,
+                          void* ws, cudaStream_t st) {
+    float* mu = nullptr;
     if (center) {
-        mu = reinterpret_cast<T*>(ws);
-        column_mean_kernel<T><<<(p + 255) / 256, 256, 0, st>>>(X, n, p, ldx, mu);
+        mu = reinterpret_cast<float*>(ws);
+        column_mean_kernel<float><<<(p + 255) / 256, 256, 0, st>>>(X, n, p, ldx, mu);
     }
-    const int t = (p + GRAM_BM - 1) / GRAM_BM;
-    gram_simt_kernel<T><<<t * (t + 1) / 2, 256, 0, st>>>(X, n, p, ldx, mu, S, lds,
-                                                        (T)(1.0 / (double)n));
+    const float inv_n = (float)(1.0 / (double)n);
+    const int tw = (p + GRAM_WIDE - 1) / GRAM_WIDE, t = (p + GRAM_BM - 1) / GRAM_BM;
+    const bool vec = ((p | ldx) & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    if (tw * (tw + 1) / 2 >= GRAM_WIDE_TILES) {
+        auto k = vec ? gram_simt_kernel<GRAM_WIDE, GRAM_WIDE_BK, GRAM_WIDE_THREADS, 8, 16, true>
+                     : gram_simt_kernel<GRAM_WIDE, GRAM_WIDE_BK, GRAM_WIDE_THREADS, 8, 16, false>;
+        k<<<tw * (tw + 1) / 2, GRAM_WIDE_THREADS, 0, st>>>(X, n, p, ldx, mu, S, lds, inv_n);
+    } else {
+        auto k = vec ? gram_simt_kernel<GRAM_BM, GRAM_BK, GRAM_THREADS, 8, 4, true>
+                     : gram_simt_kernel<GRAM_BM, GRAM_BK, GRAM_THREADS, 8, 4, false>;
+        k<<<t * (t + 1) / 2, GRAM_THREADS, 0, st>>>(X, n, p, ldx, mu, S, lds, inv_n);
+    }
     return cudaGetLastError();
 }
 
@@ -64,8 +72,8 @@ cudaError_t launch_gram(const void* X, int n, int p, int ldx, int precision, int
         return launch_gram_f64(static_cast<const double*>(X), n, p, ldx, center,
                                static_cast<double*>(S), lds, ws, st);
     if (precision == SPMESL_FP32)
-        return run_gram_simt<float>(static_cast<const float*>(X), n, p, ldx, center,
-                                    static_cast<float*>(S), lds, ws, st);
+        return run_gram_simt(static_cast<const float*>(X), n, p, ldx, center,
+                             static_cast<float*>(S), lds, ws, st);
     return launch_gram_tc(static_cast<const float*>(X), n, p, ldx, center, static_cast<float*>(S),
                           lds, ws, st);
 }

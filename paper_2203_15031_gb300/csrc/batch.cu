@@ -229,8 +229,8 @@ __global__ void __launch_bounds__(32 * PREP_ROWS) batch_prep_matrix_kernel(
 }
 
 template <typename T>
-__device__ __forceinline__ CDArgs<T> column_args(const BatchFit& f, double tol, int maxit,
-                                                 int ovf_supp = LAZY_CAP) {
+__device__ __forceinline__ CDArgs<T> column_args(const BatchFit& f, double tol, float tolf,
+                                                 int maxit, int ovf_supp = LAZY_CAP) {
     CDArgs<T> a;
     a.SC = static_cast<const T*>(f.SC);
     a.BT = static_cast<T*>(f.BT);
@@ -245,6 +245,7 @@ __device__ __forceinline__ CDArgs<T> column_args(const BatchFit& f, double tol, 
     a.maxit = maxit;
     a.lambda0 = f.lambda0;
     a.tol = tol;
+    a.tolf = tolf;
     a.ovf_list = nullptr;
     a.ovf_count = nullptr;
     a.order = nullptr;
@@ -272,7 +273,7 @@ template <typename T, bool STD>
 __global__ void __launch_bounds__(512) batch_cd_kernel(const BatchFit* __restrict__ fits,
                                                        const int* __restrict__ col_prefix,
                                                        int count, int total_cols, int max_ldp,
-                                                       double tol, int maxit,
+                                                       double tol, float tolf, int maxit,
                                                        BatchHeader* hdr, const int* ovf_list,
                                                        int from_queue) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(512) batch_cd_kernel(const BatchFit* __restric
         const int fi = find_fit(col_prefix, count, gc);
         const BatchFit& f = fits[fi];
         if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) continue;
-        const CDArgs<T> a = column_args<T>(f, tol, maxit);
+        const CDArgs<T> a = column_args<T>(f, tol, tolf, maxit);
         T* b = g + f.ldp;
         int* list = reinterpret_cast<int*>(b + f.ldp);
         ColCounters cnt;
@@ -317,7 +318,7 @@ template <typename T, bool STD>
 __global__ void __launch_bounds__(32 * LAZY_MAX_WARPS, 3) batch_cd_lazy_kernel(const BatchFit* __restrict__ fits,
                                                             const int* __restrict__ col_prefix,
                                                             int count, int total_cols, int max_ldp,
-                                                            double tol, int maxit,
+                                                            double tol, float tolf, int maxit,
                                                             BatchHeader* hdr, int* ovf_list,
                                                             const int* __restrict__ order,
                                                             int ovf_supp) {
@@ -344,7 +345,7 @@ __global__ void __launch_bounds__(32 * LAZY_MAX_WARPS, 3) batch_cd_lazy_kernel(c
         const int fi = find_fit(prefix, count, gc);
         const BatchFit& f = fits[fi];
         if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) continue;
-        const CDArgs<T> a = column_args<T>(f, tol, maxit, ovf_supp);
+        const CDArgs<T> a = column_args<T>(f, tol, tolf, maxit, ovf_supp);
         ColCounters cnt;
         if (!solve_column_lazy<T, STD>(gc - f.col_start, wsm, a, cnt) && lane == 0)
             ovf_list[atomicAdd(&hdr->ovf_count, 1)] = gc;
@@ -359,7 +360,7 @@ __global__ void __launch_bounds__(32 * LAZY_MAX_WARPS, 3) batch_cd_lazy_kernel(c
 template <typename T, bool STD>
 __global__ void __launch_bounds__(BLK_THREADS, 1) batch_cd_block_kernel(const BatchFit* __restrict__ fits,
                                                                      const int* __restrict__ col_prefix,
-                                                                     int count, double tol, int maxit,
+                                                                     int count, double tol, float tolf, int maxit,
                                                                      BatchHeader* hdr,
                                                                      const int* __restrict__ queue,
                                                                      int from_overflow) {
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(BLK_THREADS, 1) batch_cd_block_kernel(const Ba
         const int fi = find_fit(col_prefix, count, gc);
         const BatchFit& f = fits[fi];
         if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) continue;
-        const CDArgs<T> a = column_args<T>(f, tol, maxit);
+        const CDArgs<T> a = column_args<T>(f, tol, tolf, maxit);
         ColCounters cnt;
         solve_column_block<T, STD>(gc - f.col_start, smem_raw, a, cnt, sc);
         flush_counters_block(f.ctrl, cnt);
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(32 * BATCH_DIAG_WARPS) batch_diag_kernel(
         const int fi = find_fit(col_prefix, count, gc);
         const BatchFit& f = fits[fi];
         if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) continue;
-        const CDArgs<T> a = column_args<T>(f, 0.0, 1);
+        const CDArgs<T> a = column_args<T>(f, 0.0, 0.f, 1);
         DiagMax d;
         diagnose_column<T>(gc - f.col_start, wsm, a, f.diag_eps, d);
         flush_diag(f.ctrl, d);
@@ -608,6 +609,7 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
         heat_scatter_kernel<<<ORDER_BLOCKS, 256, 0, st>>>(heat, b->total_cols, hist, order);
     }
 
+    const float tolf = float_at_least(b->tol);
     const size_t budget = (size_t)max_smem_block() - 1024;
     const bool lazy = b->gradient != SPMESL_GRADIENT_EAGER;
     int* ovf = reinterpret_cast<int*>(ws + b->off_ovf);
@@ -631,7 +633,7 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
             if ((e = cudaEventRecord(b->fork2, st)) != cudaSuccess ||
                 (e = cudaStreamWaitEvent(b->side2, b->fork2, 0)) != cudaSuccess)
                 return e;
-            bk<<<bgrid, BLK_THREADS, bsm, b->side2>>>(fits, colp, count, b->tol, b->maxit, hdr,
+            bk<<<bgrid, BLK_THREADS, bsm, b->side2>>>(fits, colp, count, b->tol, tolf, b->maxit, hdr,
                                                       order, 0);
             if ((e = cudaEventRecord(b->join2, b->side2)) != cudaSuccess) return e;
         }
@@ -649,11 +651,11 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
             return e;
         lper_sm = std::max(lper_sm, 1);
         const int lgrid = std::min((b->total_cols + LW - 1) / LW, num_sms() * lper_sm);
-        lk<<<lgrid, 32 * LW, lsm, st>>>(fits, colp, count, b->total_cols, b->max_ldp, b->tol,
+        lk<<<lgrid, 32 * LW, lsm, st>>>(fits, colp, count, b->total_cols, b->max_ldp, b->tol, tolf,
                                         b->maxit, hdr, ovf, lazy_order ? order : nullptr,
                                         route ? handover_of(b->handover) : LAZY_CAP);
         // the columns the lazy launch handed over
-        bk<<<bgrid, BLK_THREADS, bsm, st>>>(fits, colp, count, b->tol, b->maxit, hdr, ovf, 1);
+        bk<<<bgrid, BLK_THREADS, bsm, st>>>(fits, colp, count, b->tol, tolf, b->maxit, hdr, ovf, 1);
         if (heavy && (e = cudaStreamWaitEvent(st, b->join2, 0)) != cudaSuccess) return e;
     } else {
         // eager gradient for every column
@@ -672,7 +674,7 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
             return e;
         per_sm = std::max(per_sm, 1);
         const int grid = std::min((b->total_cols + EW - 1) / EW, num_sms() * per_sm);
-        kern<<<grid, 32 * EW, smem, st>>>(fits, colp, count, b->total_cols, b->max_ldp, b->tol,
+        kern<<<grid, 32 * EW, smem, st>>>(fits, colp, count, b->total_cols, b->max_ldp, b->tol, tolf,
                                           b->maxit, hdr, ovf, 0);
     }
     if (timed) cudaEventRecord(b->ev[1], st);

@@ -594,6 +594,7 @@ static cudaError_t run_fit(const FitLaunch& f, const FitLayout& L, cudaStream_t 
     a.maxit = f.maxit;
     a.lambda0 = f.lambda0;
     a.tol = f.tol;
+    a.tolf = float_at_least(f.tol);
     a.ovf_list = a.flag;            // the column rule does not use the flag array
     a.ovf_count = &ctrl->ovf_count;
     a.order = nullptr;

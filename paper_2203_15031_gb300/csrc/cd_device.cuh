@@ -23,6 +23,7 @@ struct CDArgs {
     FitCtrl* ctrl;
     int p, ldp, maxit;
     double lambda0, tol;
+    float tolf;          // the smallest float not below tol (see float_at_least)
     int* ovf_list;       // columns handed from the lazy solver to the block (or eager) solver
     int* ovf_count;
     const int* order;    // queue order of the lazy solver (nullptr: 0..p-1)
@@ -197,19 +198,23 @@ __device__ __forceinline__ unsigned abs_key(float x) { return __float_as_uint(fa
 __device__ __forceinline__ unsigned abs_key(double x) {
     return (unsigned)(__double_as_longlong(x) >> 32) & 0x7fffffffu;
 }
-// The largest key of the warp as a float bound (non-negative floats and the
-// upper words of non-negative doubles order as unsigned integers).
+// The value that a key stands for, as a float bound.
 template <typename T>
-__device__ __forceinline__ float warp_max_key(unsigned key) {
-    const unsigned m = __reduce_max_sync(0xffffffffu, key);
+__device__ __forceinline__ float key_bound(unsigned m) {
     if constexpr (sizeof(T) == 4) return __uint_as_float(m);
     else return m == 0u ? 0.0f : __double2float_ru(__hiloint2double((int)(m + 1u), 0));
+}
+// The largest key of the warp (non-negative floats and the upper words of
+// non-negative doubles order as unsigned integers).
+template <typename T>
+__device__ __forceinline__ float warp_max_key(unsigned key) {
+    return key_bound<T>(__reduce_max_sync(0xffffffffu, key));
 }
 
 // The smallest float f >= x.  For a float m, m < x exactly when m < f, so a
 // stop test of a float iterate against the FP64 tolerance needs no FP64
 // arithmetic per test.
-__device__ __forceinline__ float float_at_least(double x) {
+inline float float_at_least(double x) {
     float f = (float)x;
     if ((double)f < x) f = nextafterf(f, INFINITY);
     return f;
@@ -367,6 +372,14 @@ __device__ __forceinline__ float warp_sum_f(float v) {
     return v;
 }
 
+// An upper bound of the warp's sum of |x| (one hardware reduction): each |x|
+// rounded up to a multiple of 2^-20; infinite when the sum reaches 64.
+__device__ __forceinline__ float warp_l1_bound(float x) {
+    const unsigned q = __float2uint_ru(fminf(fabsf(x), 64.0f) * 0x1p20f);
+    const unsigned t = __reduce_add_sync(FULL_MASK, q);
+    return t >= (1u << 26) ? INFINITY : __uint2float_ru(t) * 0x1p-20f;
+}
+
 template <typename T, bool STD>
 __device__ T sweep_column(int j, T* __restrict__ g, T* __restrict__ b, const CDArgs<T>& a, T lam,
                           unsigned long long& moves, ColScan& cs, int sweep_idx = -1) {
@@ -462,6 +475,7 @@ __device__ T sweep_column(int j, T* __restrict__ g, T* __restrict__ b, const CDA
 // Mark every chunk "must scan" (maxabs = infinity fails every skip test).
 __device__ __forceinline__ void reset_chunks(ColScan& cs, int ldp) {
     const int nc = (ldp + CHUNK - 1) / CHUNK;
+#pragma unroll 1
     for (int c = threadIdx.x & 31; c < nc; c += 32) cs.ci[c] = ChunkInfo{INFINITY, 0.f, 0u, 1};
     cs.dsum = 0.f;
     cs.nmoves = 0u;
@@ -704,9 +718,10 @@ __device__ __forceinline__ double sigma_step(double s0, double f0, double s1, do
 // y <- y + (q - y^2) / (2 y) from the FP32 root: the FP32 root's relative
 // error (at most 2^-23) is squared, so the result is within a few FP64 units
 // of the root, with five FP64 operations.  Outside the FP32 range, sqrt.
+static __device__ __noinline__ double sqrt_far(double q) { return sqrt(q); }
 __device__ __forceinline__ double sqrt_heron(double q) {
     const float yf = sqrtf((float)q);
-    if (!(yf > 1e-18f && yf < 1e18f)) return sqrt(q);
+    if (!(yf > 1e-18f && yf < 1e18f)) return sqrt_far(q);
     const double y0 = (double)yf;
     return fma(fma(-y0, y0, q), (double)(0.5f / yf), y0);
 }
@@ -794,8 +809,13 @@ __device__ void solve_column(int j, T* __restrict__ g, T* __restrict__ b, int* _
 // This is the covariance form of c = S_kj - sum_{l != k} S_kl b_l.  With about
 // 5 KB of shared memory per column instead of two p-vectors, many more columns
 // stay resident per SM.
-// If the support outgrows the list, the column is handed to the eager solver
-// (solve_column) through a queue and solved again from the start.
+// If the support outgrows the phase or the list, the column is handed to the
+// block solver (solve_column_block) through a queue.
+// Many warps run this code at different points of it, and its size is what they
+// wait for most after S: the 256-fit batch went from 2.55 to 2.19 ms when its
+// cold loops were no longer unrolled, the hand-over was written once and the
+// integer divisions left it, and to 2.08 ms without the FP64 square root and the
+// tolerance's rounding.  Keep cold loops at "unroll 1".
 // ===========================================================================
 constexpr int LAZY_CAP = 256;
 
@@ -810,14 +830,28 @@ struct Support {
     int n;         // warp-uniform count
 };
 
+// The support's entries of S kept in a lazy-solver warp's shared memory, for
+// the support `list` (n coordinates; n = -1: none yet): the block S_AA (column k
+// at saa + k ACT_MAX), S_jA and S_Aj (the standardised S is rounded by rows and
+// then columns, so the two differ in their last bits), and the links and
+// coefficients of the FP32 phase.
+template <typename T>
+struct SupportBlock {
+    T* saa;
+    T* row;            // S_{j A_m}
+    T* col;            // S_{A_m j}
+    int* list;
+    float2* tb;
+    int n;
+};
+
 // Shared memory of one lazy-solver warp: the support list, the chunk
-// summaries, the support's block of S, the last sigma step (sigma,
-// F(sigma)) for the secant step (kept out of registers) and the support the
-// block of S was gathered for, the links and coefficients of the FP32 phase.
+// summaries, the last sigma step (sigma, F(sigma)) for the secant step (kept
+// out of registers) and S_jj, and the support's block of S.
 template <typename T>
 __host__ __device__ constexpr size_t lazy_warp_smem_bytes(int ldp) {
     return (size_t)LAZY_CAP * (sizeof(int) + sizeof(T)) + (size_t)num_chunks(ldp) * sizeof(ChunkInfo) +
-           (size_t)ACT_MAX * ACT_MAX * sizeof(T) + 2 * sizeof(double) + ACT_MAX * sizeof(int) +
+           4 * sizeof(double) + (size_t)ACT_MAX * (ACT_MAX + 2) * sizeof(T) + ACT_MAX * sizeof(int) +
            (sizeof(T) == 4 ? ACT_MAX * sizeof(float2) : 0);
 }
 
@@ -838,6 +872,7 @@ __device__ bool support_set(Support<T>& s, int pos, int k, T v) {
     const int from = exists ? pos + 1 : pos;        // entries [from, n) move by `shift`
     const int cnt = s.n - from;
     // move in register-sized rounds; the direction keeps every read ahead of its write
+#pragma unroll 1
     for (int base = 0; base < cnt; base += 32) {
         const int t = shift > 0 ? cnt - 1 - (base + lane) : base + lane;
         int ix = 0;
@@ -891,11 +926,92 @@ __device__ __forceinline__ unsigned chunks_to_scan(const ColScan& cs, int from, 
     return __ballot_sync(FULL_MASK, need);
 }
 
+// The slices of up to scan_group() chunks at once, for a sweep that holds the support
+// (at most 32 coordinates, my = this lane's or -1): forms them as the sweep does,
+// writes the summaries of the leading chunks in which no coordinate at zero
+// passes lambda (there the sweep moves nothing) and returns their number.  In a
+// certifying sweep that is nearly always all of them, and the chunks' loads
+// are in flight together: a slice alone is one or a few dependent round trips
+// to L2 (2250 cycles at a mean support of 1.4, p = 2000).
+template <typename T>
+__host__ __device__ constexpr int scan_group() { return sizeof(T) == 4 ? 2 : 1; }
+template <typename T, bool STD, int U>
+__device__ __forceinline__ int scan_quiet_chunks(int j, const Support<T>& s, int my,
+                                                 const CDArgs<T>& a, T lam, ColScan& cs,
+                                                 const int (&ci)[scan_group<T>()], int cnt) {
+    constexpr int SCAN_G = scan_group<T>();
+    const int lane = threadIdx.x & 31;
+    const int ldp = a.ldp;
+    const T* __restrict__ Sj = a.SC + (size_t)j * ldp;
+    T acc[SCAN_G][SCAN_V];
+#pragma unroll
+    for (int g = 0; g < SCAN_G; ++g) {
+#pragma unroll
+        for (int t = 0; t < SCAN_V; ++t) acc[g][t] = T(0);
+        const int k0 = ci[g] * CHUNK + lane * SCAN_V;
+        if (g < cnt && k0 < ldp) load4g<T>(Sj + k0, acc[g]);
+    }
+#pragma unroll U
+    for (int e = 0; e < s.n; ++e) {
+        const T* __restrict__ row = a.SC + (size_t)s.idx[e] * ldp;
+        const T v = s.val[e];
+        T r[SCAN_G][SCAN_V];
+#pragma unroll
+        for (int g = 0; g < SCAN_G; ++g) {
+            const int k0 = ci[g] * CHUNK + lane * SCAN_V;
+            if (g < cnt && k0 < ldp) load4g<T>(row + k0, r[g]);
+        }
+#pragma unroll
+        for (int g = 0; g < SCAN_G; ++g) {
+            const int k0 = ci[g] * CHUNK + lane * SCAN_V;
+            if (g < cnt && k0 < ldp)
+#pragma unroll
+                for (int t = 0; t < SCAN_V; ++t) acc[g][t] = fma(-v, r[g][t], acc[g][t]);
+        }
+    }
+    int quiet = 0;
+    bool open = true;
+#pragma unroll
+    for (int g = 0; g < SCAN_G; ++g) {
+        if (g < cnt && open) {
+            const int k0 = ci[g] * CHUNK + lane * SCAN_V;
+            // coordinate j and the support's are not tested
+            unsigned held = __ballot_sync(FULL_MASK, my >= 0 && my / CHUNK == ci[g]);
+            const int nsupp = __popc(held);
+            int skip = j;
+            for (;;) {
+                const int d = skip - k0;
+#pragma unroll
+                for (int t = 0; t < SCAN_V; ++t)
+                    if (d == t) acc[g][t] = T(0);
+                if (held == 0u) break;
+                skip = __shfl_sync(FULL_MASK, my, __ffs(held) - 1);
+                held &= held - 1u;
+            }
+            unsigned key = 0u;
+#pragma unroll
+            for (int t = 0; t < SCAN_V; ++t) key = max(key, abs_key(acc[g][t]));
+            const unsigned top = __reduce_max_sync(FULL_MASK, key);
+            // FP64 keys are upper words: equal ones go to the exact test too
+            open = sizeof(T) == 4 ? top <= abs_key(lam) : top < abs_key(lam);
+            if (open) {
+                if constexpr (STD) {
+                    if (lane == 0)
+                        cs.ci[ci[g]] = ChunkInfo{key_bound<T>(top), cs.dsum, cs.nmoves, nsupp};
+                }
+                quiet = g + 1;
+            }
+        }
+    }
+    __syncwarp();
+    return quiet;
+}
+
 // One sweep; returns max |delta b|.  Sets `overflow` and stops early if the
 // support list is full.  With `frozen` the coordinates in the support keep
 // their values and only the others are updated (a coordinate that enters is
 // not revisited in the same sweep).
-template <typename T, bool STD>
+template <typename T, bool STD, int U>
 __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
                                unsigned long long& moves, ColScan& cs, bool& overflow,
                                bool frozen, int sweep_idx) {
@@ -909,8 +1025,9 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
     int mbase = 0;
     if constexpr (STD) {
         float l1 = 0.f;
+#pragma unroll 1
         for (int e = lane; e < s.n; e += 32) l1 += fabsf((float)s.val[e]);
-        cs.bl1 = warp_sum_f(l1) * (1.0f + 0x1p-16f);
+        cs.bl1 = warp_l1_bound(l1) * (1.0f + 0x1p-16f);
     }
     unsigned mask = chunks_to_scan<STD>(cs, 0, nch, (float)lam, frozen);
     for (;;) {
@@ -920,11 +1037,30 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
             mask = chunks_to_scan<STD>(cs, mbase, nch, (float)lam, frozen);
             continue;
         }
+        if (frozen && s.n <= 32) {
+            constexpr int SCAN_G = scan_group<T>();
+            const int cnt = min(SCAN_G, __popc(mask));
+            int g_ci[SCAN_G];
+            unsigned left = mask;
+#pragma unroll
+            for (int g = 0; g < SCAN_G; ++g) {
+                g_ci[g] = mbase + __ffs(left) - 1;
+                left &= left - 1u;
+            }
+            const int quiet = scan_quiet_chunks<T, STD, U>(j, s, lane < s.n ? s.idx[lane] : -1, a, lam,
+                                                           cs, g_ci, cnt);
+#pragma unroll
+            for (int g = 0; g < SCAN_G; ++g)
+                if (g < quiet) mask &= mask - 1u;
+            if (quiet == cnt) continue;
+        }
         const int ci = mbase + __ffs(mask) - 1;
         mask &= mask - 1u;
         const int cb = ci * CHUNK;
+#pragma unroll 1
         while (e0 < s.n && s.idx[e0] < cb) ++e0;
         int e1 = e0;
+#pragma unroll 1
         while (e1 < s.n && s.idx[e1] < cb + CHUNK) ++e1;
         const int k0 = cb + lane * SCAN_V;
         const bool in = k0 < ldp;                 // the whole quad is inside the padded row
@@ -946,6 +1082,7 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
         }
         // current b of this lane's coordinates (support entries of the chunk)
         T bv[SCAN_V] = {T(0), T(0), T(0), T(0)};
+#pragma unroll 1
         for (int e = e0; e < e1; ++e) {
             const int t = s.idx[e] - k0;
             if (t >= 0 && t < SCAN_V) {
@@ -987,6 +1124,7 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
             const T delta = nbs - __shfl_sync(FULL_MASK, b_sel, f);
             const int ks = cb + f * SCAN_V + tf;
             int pos = e0;
+#pragma unroll 1
             while (pos < e1 && s.idx[pos] < ks) ++pos;
             const int n_before = s.n;
             if (!support_set<T>(s, pos, ks, nbs)) {
@@ -1108,9 +1246,9 @@ __device__ __forceinline__ int phase_sweeps(const float* __restrict__ saa, float
 // Active-set phase of the lasso at a fixed lambda: cyclic sweeps (ascending
 // coordinate order) over the current support A only, until a sweep moves no
 // coefficient by tol or more (at most maxit sweeps).  Lane m holds coordinate
-// A_m: its b and g_m = S_jm - sum_{l in A} S_ml b_l; the block S_AA is
-// gathered into shared memory (column k at saa + k ACT_MAX), and kept from
-// the column's last phase when A is the same (saa_list, saa_n).  The phase's
+// A_m: its b and g_m = S_jm - sum_{l in A} S_ml b_l; the support's entries of S
+// are gathered into shared memory (SupportBlock), and kept from the column's
+// last phase when A is the same.  The phase's
 // net change of b enters the column's running sums as one change, so the
 // chunk skip test stays exact for the coordinates outside A.  Coordinates
 // that reach zero leave the support and mark their chunk for a rescan.  One
@@ -1122,8 +1260,7 @@ __device__ __forceinline__ int phase_sweeps(const float* __restrict__ saa, float
 // empty or larger than ACT_MAX); `conv` tells whether the last sweep moved
 // nothing by tol (true for an empty A, false when A is too large).
 template <typename T, bool STD>
-__device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, T* __restrict__ saa,
-                            int* __restrict__ saa_list, float2* __restrict__ tb, int& saa_n,
+__device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, SupportBlock<T>& sb,
                             unsigned long long& moves, ColScan& cs, bool& conv) {
     const int lane = threadIdx.x & 31;
     const int n = s.n;
@@ -1131,9 +1268,15 @@ __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, T* 
     if (n == 0 || n > ACT_MAX) return 0;
     conv = false;
     const int ldp = a.ldp;
+    T* __restrict__ saa = sb.saa;
+    float2* __restrict__ tb = sb.tb;
     const int my = lane < n ? s.idx[lane] : 0;
-    if (!(saa_n == n && __all_sync(FULL_MASK, lane >= n || saa_list[lane] == my))) {
-        // lane m reads S_{A_m A_k} for four k at a time (independent loads)
+    if (!(sb.n == n && __all_sync(FULL_MASK, lane >= n || sb.list[lane] == my))) {
+        // lane m reads S_{j A_m}, S_{A_m j} and S_{A_m A_k} for four k at a time
+        // (independent loads)
+        const T rv = lane < n ? a.SC[(size_t)j * ldp + my] : T(0);
+        const T cv = lane < n ? a.SC[(size_t)my * ldp + j] : T(0);
+#pragma unroll 1
         for (int k0 = 0; k0 < n; k0 += 4) {
             T v[4];
 #pragma unroll
@@ -1145,22 +1288,25 @@ __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, T* 
             for (int u = 0; u < 4; ++u)
                 if (k0 + u < n) saa[(k0 + u) * ACT_MAX + lane] = v[u];
         }
-        saa_list[lane] = my;
-        saa_n = n;
+        sb.row[lane] = rv;
+        sb.col[lane] = cv;
+        sb.list[lane] = my;
+        sb.n = n;
     }
     T b = lane < n ? s.val[lane] : T(0);
     const T b_start = b;
-    T g = lane < n ? a.SC[(size_t)j * ldp + my] : T(0);
+    T g = sb.row[lane];
     T skk = T(1);
     if constexpr (!STD) skk = lane < n ? a.diag[my] : T(1);
     __syncwarp();
+#pragma unroll 2
     for (int l = 0; l < n; ++l) {
         const T bl = __shfl_sync(FULL_MASK, b, l);
         if (lane < n) g = fma(-saa[l * ACT_MAX + lane], bl, g);
     }
     int sw = 0;
     unsigned mv = 0;
-    const float tf = float_at_least(a.tol);
+    const float tf = a.tolf;
     if constexpr (STD && sizeof(T) == 4) {
         const float2 first = phase_links<ACT_MAX>(saa, tb, n, b, T(0));
         sw = phase_sweeps<ACT_MAX>(saa, tb, n, lam, a.maxit, tf, first, g, g, mv, conv);
@@ -1192,7 +1338,7 @@ __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, T* 
     }
     moves += mv;
     // the phase enters the running sums as one change: its net l1 size
-    const float net = warp_sum_f(lane < n ? fabsf((float)(b - b_start)) : 0.f);
+    const float net = warp_l1_bound(lane < n ? (float)(b - b_start) : 0.f);
     cs.dsum += net * (1.0f + 0x1p-16f);
     ++cs.nmoves;
     // write back, dropping coordinates at zero (the list stays sorted)
@@ -1218,25 +1364,38 @@ __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, T* 
 // the n terms of b'S_.j are spread over the lanes (pair indices stepped by
 // 32 without a divide per pair), each lane adds b_u b_v S_uv and -2 b_u S_uj
 // into one FP64 partial, and one FP64 warp sum ends it.
+// The entries of S come from the phase's SupportBlock when it was gathered for
+// this support (the same values; a sigma step then reads nothing from L2),
+// otherwise from S.
 template <typename T>
-__device__ double residual_quadratic_form_list(int j, const Support<T>& s, const CDArgs<T>& a) {
+__device__ double residual_quadratic_form_list(int j, const Support<T>& s, const CDArgs<T>& a,
+                                               const SupportBlock<T>& sb, double sjj) {
     const int lane = threadIdx.x & 31;
     const int n = s.n;
     const int ldp = a.ldp;
+    if (n == 0) return sjj;
+    const bool held = sb.n == n && n <= ACT_MAX &&
+                      __all_sync(FULL_MASK, lane >= n || sb.list[lane] == s.idx[lane]);
     double acc = 0.0;
-    if (lane < n) {
-        // -2 b_u S_uj for u = lane, lane + 32, ... (-2 b_u is exact in the data precision)
-        for (int u = lane; u < n; u += 32)
-            acc = fma((double)(T(-2) * s.val[u]), (double)a.SC[(size_t)s.idx[u] * ldp + j], acc);
+    // -2 b_u S_uj for u = lane, lane + 32, ... (-2 b_u is exact in the data precision)
+#pragma unroll 1
+    for (int u = lane; u < n; u += 32) {
+        const T suj = held ? sb.col[u] : a.SC[(size_t)s.idx[u] * ldp + j];
+        acc = fma((double)(T(-2) * s.val[u]), (double)suj, acc);
     }
     const int np = n * n;
     if (lane < np) {
         // pair t = u n + v for t = lane, lane + 32, ...: (u, v) advance by (q, r)
-        int u = lane / n, v = lane - (lane / n) * n;
-        const int q = 32 / n, r = 32 - (32 / n) * n;
+        // (quotients of small integers by a reciprocal: half a unit from an integer
+        // is far above its rounding)
+        const float rn = __frcp_rn((float)n);
+        int u = (int)(((float)lane + 0.5f) * rn), v = lane - u * n;
+        const int q = (int)(32.5f * rn), r = 32 - q * n;
+#pragma unroll 1
         for (int t = lane; t < np; t += 32) {
             const double bb = (double)s.val[u] * (double)s.val[v];
-            acc = fma(bb, (double)a.SC[(size_t)s.idx[u] * ldp + s.idx[v]], acc);
+            const T suv = held ? sb.saa[v * ACT_MAX + u] : a.SC[(size_t)s.idx[u] * ldp + s.idx[v]];
+            acc = fma(bb, (double)suv, acc);
             u += q;
             v += r;
             if (v >= n) {
@@ -1246,7 +1405,7 @@ __device__ double residual_quadratic_form_list(int j, const Support<T>& s, const
         }
     }
     acc = warp_sum(acc);
-    return (double)a.SC[(size_t)j * ldp + j] + acc;
+    return sjj + acc;
 }
 
 // b_j as the whole dense row j of BT, zeros included (16-byte stores; ldp is a
@@ -1257,8 +1416,10 @@ __device__ __forceinline__ void store_row_lazy(int j, const Support<T>& s, const
     T* brow = a.BT + (size_t)j * a.ldp;
     uint4* q = reinterpret_cast<uint4*>(brow);
     const int nq = a.ldp * (int)sizeof(T) / 16;
+#pragma unroll 1
     for (int i = lane; i < nq; i += 32) q[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
+#pragma unroll 1
     for (int t = lane; t < s.n; t += 32) brow[s.idx[t]] = s.val[t];
 }
 
@@ -1274,6 +1435,7 @@ __device__ __forceinline__ void store_solved_lazy(int j, const Support<T>& s, co
     }
     T* row = a.BT + (size_t)j * a.ldp;
     int* idx = coef_idx(row, a.ldp);
+#pragma unroll 1
     for (int t = lane; t < s.n; t += 32) {
         row[t] = s.val[t];
         idx[t] = s.idx[t];
@@ -1306,7 +1468,7 @@ __device__ __forceinline__ void hand_over_lazy(int j, const Support<T>& s, const
 // support outgrew the list (nothing written; the caller queues the column
 // for the eager solver).  HS keeps the last sigma step in the warp's shared
 // memory instead of registers (for kernels at a tight register cap).
-template <typename T, bool STD, bool HS = false>
+template <typename T, bool STD, bool HS = false, int U = 1>
 __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a, ColCounters& cnt) {
     const int lane = threadIdx.x & 31;
     Support<T> s;
@@ -1314,11 +1476,15 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
     s.val = reinterpret_cast<T*>(wsm + LAZY_CAP * sizeof(int));
     s.n = 0;
     ColScan cs{reinterpret_cast<ChunkInfo*>(wsm + LAZY_CAP * (sizeof(int) + sizeof(T))), 0.f, 0u};
-    T* saa = reinterpret_cast<T*>(cs.ci + num_chunks(a.ldp));
-    double* prev = reinterpret_cast<double*>(saa + ACT_MAX * ACT_MAX);   // HS: (sigma, F(sigma))
-    int* saa_list = reinterpret_cast<int*>(prev + 2);    // the support S_AA was gathered for
-    float2* tb = reinterpret_cast<float2*>(saa_list + ACT_MAX);   // the FP32 phase's links and b
-    int saa_n = -1;
+    double* prev = reinterpret_cast<double*>(cs.ci + num_chunks(a.ldp));   // HS: (sigma, F(sigma)); S_jj
+    SupportBlock<T> sb;
+    sb.saa = reinterpret_cast<T*>(prev + 4);
+    sb.row = sb.saa + ACT_MAX * ACT_MAX;
+    sb.col = sb.row + ACT_MAX;
+    sb.tb = reinterpret_cast<float2*>(sb.col + ACT_MAX);
+    sb.list = reinterpret_cast<int*>(sb.tb + (sizeof(T) == 4 ? ACT_MAX : 0));
+    sb.n = -1;
+    if (lane == 0) prev[2] = (double)a.SC[(size_t)j * a.ldp + j];
     reset_chunks(cs, a.ldp);
     if constexpr (STD) {
         // b = 0: the gradient is row j of S^C, whose chunk maxima the
@@ -1326,6 +1492,7 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
         if (a.chunk_max) {
             const int nch = num_chunks(a.ldp);
             const float* __restrict__ cm = a.chunk_max + (size_t)j * nch;
+#pragma unroll 1
             for (int c = lane; c < nch; c += 32) cs.ci[c] = ChunkInfo{cm[c], 0.f, 0u, 0};
         }
     }
@@ -1334,9 +1501,8 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
     double sigma = 1.0;                                  // sigma^(0) = 1, b = 0
     double s_prev = 0.0, f_prev = 0.0;                   // last (sigma, F(sigma))
     const unsigned long long sweeps0 = cnt.sweeps;
-    const double floor2 = 1e-12 * (double)a.SC[(size_t)j * a.ldp + j];
     int status = COL_OK;
-    bool overflow = false;
+    bool overflow = false;           // the column goes to the block solver
     int r;
     for (r = 0; r < a.maxit; ++r) {
         const T lam = (T)(sigma * a.lambda0);
@@ -1349,28 +1515,28 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
             // by tol.  Otherwise a full sweep of every coordinate decides (the
             // stop rule of Algorithm 1).
             bool conv;
-            if (s.n > a.ovf_supp) {                       // a heavy column: the block solver
-                hand_over_lazy<T, HS>(j, s, a, sigma, HS ? prev[0] : s_prev, HS ? prev[1] : f_prev,
-                                      r, status);
-                return false;
+            if (s.n > a.ovf_supp) {
+                overflow = true;
+                break;
             }
-            cnt.act_sweeps += active_phase<T, STD>(j, s, a, lam, saa, saa_list, tb, saa_n,
-                                                  cnt.act_moves, cs, conv);
-            const T md = sweep_column_lazy<T, STD>(j, s, a, lam, cnt.moves, cs, overflow, conv,
+            cnt.act_sweeps += active_phase<T, STD>(j, s, a, lam, sb, cnt.act_moves, cs, conv);
+            const T md = sweep_column_lazy<T, STD, U>(j, s, a, lam, cnt.moves, cs, overflow, conv,
                                                    (int)(cnt.sweeps - sweeps0));
             ++cnt.sweeps;
-            if (overflow) {
-                hand_over_lazy<T, HS>(j, s, a, sigma, HS ? prev[0] : s_prev, HS ? prev[1] : f_prev,
-                                      r, status);
-                return false;
-            }
-            if ((double)md < a.tol) {
+            if (overflow) break;
+            if (below_tol<T>(md, a.tol, a.tolf)) {
                 inner_ok = true;
                 break;
             }
         }
+        if (overflow) {
+            hand_over_lazy<T, HS>(j, s, a, sigma, HS ? prev[0] : s_prev, HS ? prev[1] : f_prev, r,
+                                  status);
+            return false;
+        }
         if (!inner_ok) status |= COL_NOT_CONVERGED;
-        double q = residual_quadratic_form_list<T>(j, s, a);
+        double q = residual_quadratic_form_list<T>(j, s, a, sb, prev[2]);
+        const double floor2 = 1e-12 * prev[2];
         if (q <= floor2) {
             q = floor2;
             status |= COL_DEGENERATE;
@@ -2011,7 +2177,7 @@ __device__ int block_active_phase(int j, T* __restrict__ b, const int* __restric
     conv = false;
     int sw = 0;
     unsigned mv = 0;
-    const float tf = float_at_least(a.tol);
+    const float tf = a.tolf;
     if constexpr (STD && sizeof(T) == 4) {
         const float2 first = phase_links<BLK_AMAX>(saa, tb, n, b0, b1);
         sw = phase_sweeps<BLK_AMAX>(saa, tb, n, lam, a.maxit, tf, first, g0, g1, mv, conv);

@@ -311,11 +311,18 @@ constexpr int PREFIX_SMEM = 1024;
 // Lazy gradient over all columns of all fits; overflowing columns are queued
 // for the block solver, and the first n_heavy columns of the heat order
 // belong to it from the start.
-// At most 8 warps a block and 3 blocks an SM: the kernel then keeps its
-// working set in registers instead of spilling inside the sweep.
+// At most 8 warps a block; MINB blocks an SM.  Three (80 registers) carry most
+// columns a second; two (128 registers) solve one column sooner, with more of its
+// loads in flight and no spills, which decides while the longest columns do:
+// up to LAZY_WIDE_COLS columns per resident warp of the two-block form (20:
+// 48640 columns on 152 SMs), and in FP64, where 80 registers spill most.
+// 256 fits (133 k columns) 2.04 ms with three, 2.18 with two; 128 (62 k) 1.30
+// and 1.17; 96 (44 k) 1.17 and 1.03; ten p = 2000 fits (20 k) 0.42 and 0.38, twenty
+// (40 k) 0.64 and 0.68, forty (80 k) 1.24 and 1.32; FP64 study (25 k) 1.33 and 1.26.
 constexpr int LAZY_MAX_WARPS = 8;
-template <typename T, bool STD>
-__global__ void __launch_bounds__(32 * LAZY_MAX_WARPS, 3) batch_cd_lazy_kernel(const BatchFit* __restrict__ fits,
+constexpr int LAZY_WIDE_COLS = 20;
+template <typename T, bool STD, int MINB>
+__global__ void __launch_bounds__(32 * LAZY_MAX_WARPS, MINB) batch_cd_lazy_kernel(const BatchFit* __restrict__ fits,
                                                             const int* __restrict__ col_prefix,
                                                             int count, int total_cols, int max_ldp,
                                                             double tol, float tolf, int maxit,
@@ -641,7 +648,10 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
         const size_t lper = lazy_warp_smem_bytes<T>(b->max_ldp);
         const int LW = std::max(1, std::min({W, LAZY_MAX_WARPS, (int)(budget / lper)}));
         const size_t lsm = lper * LW;
-        auto lk = b->standardize ? batch_cd_lazy_kernel<T, true> : batch_cd_lazy_kernel<T, false>;
+        auto lk = b->standardize ? batch_cd_lazy_kernel<T, true, 2> : batch_cd_lazy_kernel<T, false, 2>;
+        if constexpr (sizeof(T) == 4)
+            if (b->total_cols > LAZY_WIDE_COLS * num_sms() * 2 * LAZY_MAX_WARPS)
+                lk = b->standardize ? batch_cd_lazy_kernel<T, true, 3> : batch_cd_lazy_kernel<T, false, 3>;
         if ((e = cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)lsm)) != cudaSuccess)
             return e;

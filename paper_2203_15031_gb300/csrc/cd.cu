@@ -63,10 +63,16 @@ __global__ void __launch_bounds__(512) cd_column_kernel(CDArgs<T> a, int from_qu
 }
 
 // Lazy gradient (sorted support in shared memory); columns whose support
-// outgrows the list go to the queue for cd_column_kernel.
+// outgrows the phase or the list go to the queue for the block solver.  A
+// single fit rarely fills the SMs, and its time is its longest column's
+// chain: two blocks an SM (128 registers) and four chunks of a quiet scan at
+// once, with four support rows of each in flight (p = 2000 fit 234 -> 203 us,
+// p = 2000 regression 443 -> 292 us against the batch's three blocks and two
+// chunks; p = 10000 the same).
 template <typename T, bool STD>
-__global__ void __launch_bounds__(256, 3) cd_column_lazy_kernel(CDArgs<T> a) {
+__global__ void __launch_bounds__(256, 2) cd_column_lazy_kernel(CDArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr bool F32 = sizeof(T) == 4;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     unsigned char* wsm = smem_raw + (size_t)warp * lazy_warp_smem_bytes<T>(a.ldp);
@@ -83,7 +89,7 @@ __global__ void __launch_bounds__(256, 3) cd_column_lazy_kernel(CDArgs<T> a) {
         }
         j = __shfl_sync(FULL_MASK, j, 0);
         if (j >= a.p) break;
-        if (!solve_column_lazy<T, STD, true>(j, wsm, a, cnt) && lane == 0)
+        if (!solve_column_lazy<T, STD, true, F32 ? 4 : 2, F32 ? 4 : 1>(j, wsm, a, cnt) && lane == 0)
             a.ovf_list[atomicAdd(a.ovf_count, 1)] = j;
         __syncwarp();
     }

@@ -929,17 +929,19 @@ __device__ __forceinline__ unsigned chunks_to_scan(const ColScan& cs, int from, 
 // The slices of up to scan_group() chunks at once, for a sweep that holds the support
 // (at most 32 coordinates, my = this lane's or -1): forms them as the sweep does,
 // writes the summaries of the leading chunks in which no coordinate at zero
-// passes lambda (there the sweep moves nothing) and returns their number.  In a
+// passes lambda (there the sweep moves nothing) and returns their number; the
+// next chunk's slice, if there is one, is left in `slice` (zero at coordinate j
+// and at the support's, which that sweep does not read).  In a
 // certifying sweep that is nearly always all of them, and the chunks' loads
 // are in flight together: a slice alone is one or a few dependent round trips
 // to L2 (2250 cycles at a mean support of 1.4, p = 2000).
 template <typename T>
 __host__ __device__ constexpr int scan_group() { return sizeof(T) == 4 ? 2 : 1; }
-template <typename T, bool STD, int U>
+template <typename T, bool STD, int U, int SCAN_G>
 __device__ __forceinline__ int scan_quiet_chunks(int j, const Support<T>& s, int my,
                                                  const CDArgs<T>& a, T lam, ColScan& cs,
-                                                 const int (&ci)[scan_group<T>()], int cnt) {
-    constexpr int SCAN_G = scan_group<T>();
+                                                 const int (&ci)[SCAN_G], int cnt,
+                                                 T (&slice)[SCAN_V]) {
     const int lane = threadIdx.x & 31;
     const int ldp = a.ldp;
     const T* __restrict__ Sj = a.SC + (size_t)j * ldp;
@@ -1000,6 +1002,9 @@ __device__ __forceinline__ int scan_quiet_chunks(int j, const Support<T>& s, int
                         cs.ci[ci[g]] = ChunkInfo{key_bound<T>(top), cs.dsum, cs.nmoves, nsupp};
                 }
                 quiet = g + 1;
+            } else {
+#pragma unroll
+                for (int t = 0; t < SCAN_V; ++t) slice[t] = acc[g][t];
             }
         }
     }
@@ -1011,7 +1016,7 @@ __device__ __forceinline__ int scan_quiet_chunks(int j, const Support<T>& s, int
 // support list is full.  With `frozen` the coordinates in the support keep
 // their values and only the others are updated (a coordinate that enters is
 // not revisited in the same sweep).
-template <typename T, bool STD, int U>
+template <typename T, bool STD, int U, int SCAN_G>
 __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
                                unsigned long long& moves, ColScan& cs, bool& overflow,
                                bool frozen, int sweep_idx) {
@@ -1037,8 +1042,9 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
             mask = chunks_to_scan<STD>(cs, mbase, nch, (float)lam, frozen);
             continue;
         }
-        if (frozen && s.n <= 32) {
-            constexpr int SCAN_G = scan_group<T>();
+        T acc[SCAN_V] = {T(0), T(0), T(0), T(0)};
+        const bool grouped = frozen && s.n <= 32;
+        if (grouped) {
             const int cnt = min(SCAN_G, __popc(mask));
             int g_ci[SCAN_G];
             unsigned left = mask;
@@ -1047,8 +1053,8 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
                 g_ci[g] = mbase + __ffs(left) - 1;
                 left &= left - 1u;
             }
-            const int quiet = scan_quiet_chunks<T, STD, U>(j, s, lane < s.n ? s.idx[lane] : -1, a, lam,
-                                                           cs, g_ci, cnt);
+            const int quiet = scan_quiet_chunks<T, STD, U, SCAN_G>(j, s, lane < s.n ? s.idx[lane] : -1, a, lam,
+                                                           cs, g_ci, cnt, acc);
 #pragma unroll
             for (int g = 0; g < SCAN_G; ++g)
                 if (g < quiet) mask &= mask - 1u;
@@ -1066,18 +1072,19 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
         const bool in = k0 < ldp;                 // the whole quad is inside the padded row
         // slice of g: S_jk - sum_{l in support} S_lk b_l (four rows in flight;
         // an L1 prefetch of all the support rows first was measured slower)
-        const T* __restrict__ col = a.SC + k0;    // column k0 of S; row l at col + l ldp
-        T acc[SCAN_V] = {T(0), T(0), T(0), T(0)};
-        if (in) load4g<T>(Sj + k0, acc);
+        if (!grouped) {
+            const T* __restrict__ col = a.SC + k0;    // column k0 of S; row l at col + l ldp
+            if (in) load4g<T>(Sj + k0, acc);
 #pragma unroll 4
-        for (int e = 0; e < s.n; ++e) {
-            const int l = s.idx[e];
-            const T v = s.val[e];
-            if (in) {
-                T r[SCAN_V];
-                load4g<T>(col + (size_t)l * ldp, r);
+            for (int e = 0; e < s.n; ++e) {
+                const int l = s.idx[e];
+                const T v = s.val[e];
+                if (in) {
+                    T r[SCAN_V];
+                    load4g<T>(col + (size_t)l * ldp, r);
 #pragma unroll
-                for (int t = 0; t < SCAN_V; ++t) acc[t] = fma(-v, r[t], acc[t]);
+                    for (int t = 0; t < SCAN_V; ++t) acc[t] = fma(-v, r[t], acc[t]);
+                }
             }
         }
         // current b of this lane's coordinates (support entries of the chunk)
@@ -1198,17 +1205,22 @@ __device__ __forceinline__ float2 phase_links(const float* __restrict__ saa, flo
     return tb[0];
 }
 
+// b0, b1: this lane's coefficients, updated once a sweep from tb; they also
+// count the moves (a move changes its coefficient), off the chain.
 template <int LD>
 __device__ __forceinline__ int phase_sweeps(const float* __restrict__ saa, float2* __restrict__ tb,
                                             int n, float lam, int maxit, float tf, float2 q, float& g0,
-                                            float& g1, unsigned& mv, bool& conv) {
-    const float* __restrict__ col = saa + (threadIdx.x & 31);
+                                            float& g1, float& b0, float& b1, unsigned& mv,
+                                            bool& conv) {
+    const int lane = threadIdx.x & 31;
+    const float* __restrict__ col = saa + lane;
     float c0 = col[0], c1 = LD > 32 ? col[32] : 0.f;
     float gk = __shfl_sync(FULL_MASK, g0, 0), dp = 0.f;
     float md;
+    unsigned moved = 0;
     // move k; kn is the next one, gs the slot of its gradient
     auto move = [&](int k, int kn, const float& gs) {
-        const float gn = __shfl_sync(FULL_MASK, gs, kn & 31);
+        const float gn = __shfl_sync(FULL_MASK, gs, kn);        // (lane kn mod 32)
         float2 qn = tb[kn];
         const float n0 = col[kn * LD], n1 = LD > 32 ? col[kn * LD + 32] : 0.f;
         gk = fmaf(-q.x, dp, gk);
@@ -1219,13 +1231,14 @@ __device__ __forceinline__ int phase_sweeps(const float* __restrict__ saa, float
         g0 = fmaf(-c0, dp, g0);
         if (LD > 32) g1 = fmaf(-c1, dp, g1);
         md = max_abs(md, dp);
-        mv += is_move(dp);
         c0 = n0;
         c1 = n1;
         q = qn;
         gk = gn;
     };
-    for (int sw = 1; sw <= maxit; ++sw) {
+    int sw = 0;
+    while (sw < maxit) {
+        ++sw;
         md = 0.f;
         const int n_lo = LD > 32 ? min(n, 32) : n;
 #pragma unroll 4
@@ -1235,12 +1248,23 @@ __device__ __forceinline__ int phase_sweeps(const float* __restrict__ saa, float
             for (int k = 31; k < n - 1; ++k) move(k, k + 1, g1);
         }
         move(n - 1, 0, g0);
+        if (lane < n) {
+            const float x = tb[lane].y;
+            moved += x != b0;
+            b0 = x;
+        }
+        if (LD > 32 && lane + 32 < n) {
+            const float x = tb[lane + 32].y;
+            moved += x != b1;
+            b1 = x;
+        }
         if (md < tf) {
             conv = true;
-            return sw;
+            break;
         }
     }
-    return maxit;
+    mv = __reduce_add_sync(FULL_MASK, moved);
+    return sw;
 }
 
 // Active-set phase of the lasso at a fixed lambda: cyclic sweeps (ascending
@@ -1309,9 +1333,7 @@ __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, Sup
     const float tf = a.tolf;
     if constexpr (STD && sizeof(T) == 4) {
         const float2 first = phase_links<ACT_MAX>(saa, tb, n, b, T(0));
-        sw = phase_sweeps<ACT_MAX>(saa, tb, n, lam, a.maxit, tf, first, g, g, mv, conv);
-        __syncwarp();
-        if (lane < n) b = tb[lane].y;
+        sw = phase_sweeps<ACT_MAX>(saa, tb, n, lam, a.maxit, tf, first, g, g, b, b, mv, conv);
     } else {
         while (sw < a.maxit) {
             ++sw;
@@ -1468,7 +1490,7 @@ __device__ __forceinline__ void hand_over_lazy(int j, const Support<T>& s, const
 // support outgrew the list (nothing written; the caller queues the column
 // for the eager solver).  HS keeps the last sigma step in the warp's shared
 // memory instead of registers (for kernels at a tight register cap).
-template <typename T, bool STD, bool HS = false, int U = 1>
+template <typename T, bool STD, bool HS = false, int U = 2, int SCAN_G = scan_group<T>()>
 __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a, ColCounters& cnt) {
     const int lane = threadIdx.x & 31;
     Support<T> s;
@@ -1520,7 +1542,7 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
                 break;
             }
             cnt.act_sweeps += active_phase<T, STD>(j, s, a, lam, sb, cnt.act_moves, cs, conv);
-            const T md = sweep_column_lazy<T, STD, U>(j, s, a, lam, cnt.moves, cs, overflow, conv,
+            const T md = sweep_column_lazy<T, STD, U, SCAN_G>(j, s, a, lam, cnt.moves, cs, overflow, conv,
                                                    (int)(cnt.sweeps - sweeps0));
             ++cnt.sweeps;
             if (overflow) break;
@@ -2180,10 +2202,7 @@ __device__ int block_active_phase(int j, T* __restrict__ b, const int* __restric
     const float tf = a.tolf;
     if constexpr (STD && sizeof(T) == 4) {
         const float2 first = phase_links<BLK_AMAX>(saa, tb, n, b0, b1);
-        sw = phase_sweeps<BLK_AMAX>(saa, tb, n, lam, a.maxit, tf, first, g0, g1, mv, conv);
-        __syncwarp();
-        if (h0) b0 = tb[m0].y;
-        if (h1) b1 = tb[m1].y;
+        sw = phase_sweeps<BLK_AMAX>(saa, tb, n, lam, a.maxit, tf, first, g0, g1, b0, b1, mv, conv);
     } else {
         while (sw < a.maxit) {
             ++sw;

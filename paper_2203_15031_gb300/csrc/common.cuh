@@ -114,7 +114,8 @@ inline FitLayout fit_layout(int p, int precision) {
 
 // Byte offsets of the residual-form workspace (spmesl_fit_residual): the
 // control block first (spmesl_fit_result reads it there), then the per-column
-// vectors, the scaled data W (ldn x ldp) and its transpose Wt (p x ldn), and
+// vectors (mu and wscale, dead once the scaled data are built, then hold the
+// chunk maxima of |w_k' w_l|), the scaled data W (ldn x ldp) and its transpose Wt (p x ldn), and
 // the coefficients BT (p x ldp).
 struct ResLayout {
     int ldn, ldp;

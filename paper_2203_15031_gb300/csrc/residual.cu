@@ -30,9 +30,12 @@
 //
 // What bounds it: the longest column's chain of slices and moves (one warp).
 // Chunks whose coordinates at zero provably stay there have only their support
-// coordinates formed, one n-term dot each.  Erdos-Renyi p = 2000, n = 200,
-// FP32: 4.4 ms a fit, against 16.5 ms with a whole slice formed per visit and
-// per move; the same iterates bit for bit.
+// coordinates formed, one n-term dot each, over a row that the warp loads ahead;
+// a slice is formed once, not after each of its moves.  Erdos-Renyi p = 2000,
+// n = 200, FP32, a fit: 16.9 ms with a whole slice formed per visit and per move;
+// 4.3 ms with quiet chunks; 3.5 ms with the growth bounded per chunk; 1.77 ms
+// with rows staged through shared memory (a visit 3800 -> under 1000 cycles)
+// and single coordinates formed after a move.  The same iterates bit for bit.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -51,12 +54,32 @@ struct ResArgs {
     const T* Wt;
     T* BT;
     const T* diag;       // ||w_k||^2 (unstandardised update)
+    const unsigned char *cmax0, *cmax1;   // bounds of |w_k' w_l| (see chunk_bound)
+    int cm_chunks;       // 128-coordinate chunks per byte of them
+    int stage;           // 1: support rows go through shared memory (n <= RES_ROW * 32)
     double* sigma;       // working-scale sigma
     int* col_status;
     FitCtrl* ctrl;
     int n, ldn, p, ldp, maxit;
     double lambda0, tol;
 };
+
+// A bound of |w_k' w_l| over the coordinates l != k of chunk c (standardised
+// data): sixteen bytes per column, each for cm_chunks chunks (one up to
+// p = 2048), in units of 1/254.  They take the place of the column means and
+// scales once the scaled data are built, so the workspace is O(n p) as before.
+constexpr int CM_GROUPS = 16;
+template <typename T>
+__device__ __forceinline__ float chunk_bound(const ResArgs<T>& a, int k, int c) {
+    const int g = a.cm_chunks == 1 ? c : c / a.cm_chunks;
+    const unsigned char* t = g < 8 ? a.cmax0 + g : a.cmax1 + (g - 8);
+    return (float)t[8 * (size_t)k] * ((1.0f + 0x1p-20f) / 254.0f);
+}
+
+// Samples of a support row that the warp holds in registers (32 per register).
+constexpr int RES_ROW = 16;
+// Coordinates of a chunk that are formed one by one after a move.
+constexpr int RES_OPEN = 12;
 
 // Upper bounds on ||r_j|| (warp-uniform): rb now, rmax over the solve so far.
 struct ResNorm {
@@ -114,15 +137,16 @@ __device__ __forceinline__ void slice_dot(const T* __restrict__ W, int ldp, int 
 // The same sum for one coordinate from its row of Wt (Wt[k][i] = W[i][k]):
 // the products and their order are those of slice_dot, so the result is the
 // value that the chunk's slice holds at coordinate k.  Every lane forms it
-// (uniform reads: the row from L1, r from shared memory).
-template <typename T>
+// (uniform reads of r and of the row, which is staged in shared memory).
+template <typename T, bool SMEM>
 __device__ __forceinline__ T column_dot(const T* __restrict__ wk, int n4, const T* __restrict__ r) {
     T a0 = T(0), a1 = T(0);
 #pragma unroll(sizeof(T) == 4 ? 8 : 4)
     for (int i = 0; i < n4; i += 4) {
         T rv[4], z[4];
         lds4<T>(r + i, rv);
-        load4g<T>(wk + i, z);
+        if constexpr (SMEM) lds4<T>(wk + i, z);
+        else load4g<T>(wk + i, z);
         a0 = fma(z[0], rv[0], a0);
         a1 = fma(z[1], rv[1], a1);
         a0 = fma(z[2], rv[2], a0);
@@ -131,25 +155,61 @@ __device__ __forceinline__ T column_dot(const T* __restrict__ wk, int n4, const 
     return a0 + a1;
 }
 
-// Bring a row of n entries into L1 (one 128-byte line per lane and step).
+// Row k of Wt in the warp's registers (entry lane + 32 i in v[i]; n <= RES_ROW * 32).
 template <typename T>
-__device__ __forceinline__ void prefetch_row(const T* __restrict__ row, int n) {
-    constexpr int LINE = 128 / (int)sizeof(T);
-    for (int i = (int)(threadIdx.x & 31) * LINE; i < n; i += 32 * LINE)
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(row + i));
+__device__ __forceinline__ void load_row(const ResArgs<T>& a, int k, T (&v)[RES_ROW]) {
+    const T* __restrict__ wk = a.Wt + (size_t)k * a.ldn + (threadIdx.x & 31);
+#pragma unroll
+    for (int i = 0; i < RES_ROW; ++i)
+        if (32 * i < a.n) v[i] = __ldg(wk + 32 * i);
 }
+
+// The gradient of one coordinate k at the current residual: its row through the
+// stage buffer (from registers when the caller has loaded it), or from global
+// memory when n is beyond it.
+template <typename T>
+__device__ __forceinline__ T coordinate_dot(const ResArgs<T>& a, int k, const T (&v)[RES_ROW],
+                                            T* __restrict__ stage, const T* __restrict__ r) {
+    const int n4 = (a.n + 3) & ~3;
+    if (!a.stage) return column_dot<T, false>(a.Wt + (size_t)k * a.ldn, n4, r);
+    __syncwarp();                       // the last row's readers are done
+#pragma unroll
+    for (int i = 0; i < RES_ROW; ++i)
+        if (32 * i < a.n) stage[32 * i + (threadIdx.x & 31)] = v[i];
+    __syncwarp();
+    return column_dot<T, true>(stage, n4, r);
+}
+
+// Per-chunk summary of the residual form: after the chunk was last scanned, the
+// largest |g_k| over its coordinates with b_k = 0, a bound of how far any of them
+// has moved since, the move count at that moment, and whether it holds support.
+struct ResChunk {
+    float maxabs, grow;
+    unsigned moves_at;
+    int nsupp;
+};
+static_assert(sizeof(ResChunk) == sizeof(ChunkInfo), "res_warp_smem_bytes counts ChunkInfo");
+
+// Scan state of one column (warp-uniform).
+struct ResScan {
+    ResChunk* ci;
+    unsigned nmoves;
+};
 
 // Chunks of [from, from + 32) that the sweep must visit (standardised data),
 // and in `full` those of them whose slice must be formed.
 // A chunk is quiet when none of its coordinates at zero can reach
 // the threshold.  Since the chunk was scanned, each move delta_m changed the
-// exact dot w_k' r by at most |delta_m| ||w_k|| ||w_m|| <= |delta_m| (1 + 2^-21)
-// plus the rounding of the r update (2^-24 ||r||), and each residual
-// recomputation was entered as a move of size ||r_new - r_old||; each of the
+// exact dot w_k' r by |delta_m w_k' w_m| <= |delta_m| cmax[m][chunk] (the bound
+// is a quarter of the Cauchy-Schwarz one at p = 2000, n = 200, and most of a
+// column's slices were formed for the difference), plus the rounding of the r
+// update (2^-24 ||r||), and each residual
+// recomputation was entered as a move of size ||r_new - r_old|| in every chunk; each of the
 // two computed dots (then and now) is within n 2^-24 ||r|| of the exact one
 // (Cauchy-Schwarz, ||w_k|| <= 1 + 2^-22).  With rmax bounding ||r|| over the
-// solve, the margins below cover these terms, the rounding of the running
-// sum (as in chunk_skippable) and of the bound itself.  A coordinate at zero
+// solve, the margins below cover these terms, the rounding of the growth's
+// sum (each of the dm additions is off by at most 2^-24 of it) and of the bound
+// itself.  A coordinate at zero
 // in a quiet chunk would therefore have computed |g_k| < lambda and not moved:
 // a quiet chunk without support is skipped, and in one with support only the
 // support coordinates are formed and tested, in their order, so the sweep is
@@ -157,19 +217,18 @@ __device__ __forceinline__ void prefetch_row(const T* __restrict__ row, int n) {
 // when the chunk was scanned; one that has come to zero since marks its chunk,
 // maxabs = infinity.)
 template <bool STD>
-__device__ __forceinline__ unsigned res_chunks_to_visit(const ColScan& cs, int from, int nch,
+__device__ __forceinline__ unsigned res_chunks_to_visit(const ResScan& cs, int from, int nch,
                                                         float lam, float rmax, int n,
                                                         unsigned& full) {
     const int ci = from + (int)(threadIdx.x & 31);
     bool scan = ci < nch, visit = scan;
     if constexpr (STD) {
         if (scan) {
-            const ChunkInfo c = cs.ci[ci];
+            const ResChunk c = cs.ci[ci];
             const unsigned dm = cs.nmoves - c.moves_at;
             if (dm <= 4096u) {
-                const float bound = c.maxabs * (1.0f + 0x1p-22f) +
-                                    (cs.dsum - c.dsum_at) * (1.0f + 0x1p-10f) +
-                                    cs.dsum * (float)(dm + 2u) * 0x1p-23f +
+                const float bound = c.maxabs * (1.0f + 0x1p-22f) + c.grow * (1.0f + 0x1p-10f) +
+                                    c.grow * (float)(dm + 2u) * 0x1p-23f +
                                     rmax * (float)(n + (int)dm + 2) * 0x1p-22f + lam * 0x1p-20f;
                 scan = !(bound < lam);
                 visit = scan || c.nsupp != 0;
@@ -181,23 +240,38 @@ __device__ __forceinline__ unsigned res_chunks_to_visit(const ColScan& cs, int f
 }
 
 // A move of coordinate k by delta: Proposition 2's r_j -= w_k delta (row k of
-// Wt) and the running sums of the skip test.
-template <typename T>
-__device__ __forceinline__ void note_residual_move(T* __restrict__ r, const T* __restrict__ wk, int n,
-                                                   T delta, ColScan& cs, ResNorm& rn) {
-    cs.dsum += fabsf((float)delta);
+// Wt, in v with the stage buffer) and the chunks' growth.
+template <typename T, bool STD>
+__device__ __forceinline__ void note_residual_move(T* __restrict__ r, int k, const ResArgs<T>& a,
+                                                   const T (&v)[RES_ROW], T delta, ResScan& cs,
+                                                   ResNorm& rn) {
+    const int n = a.n, lane = threadIdx.x & 31;
     ++cs.nmoves;
+    if constexpr (STD) {
+        const int nch = num_chunks(a.ldp);
+        for (int c = lane; c < nch; c += 32)
+            cs.ci[c].grow += fabsf((float)delta) * chunk_bound(a, k, c);
+    }
     rn.rb = (rn.rb + fabsf((float)delta)) * (1.0f + 0x1p-19f);
     rn.rmax = fmaxf(rn.rmax, rn.rb);
-    for (int i = (int)(threadIdx.x & 31); i < n; i += 32) r[i] = fma(-delta, wk[i], r[i]);
+    __syncwarp();                       // every lane has read r
+    if (a.stage) {
+#pragma unroll
+        for (int i = 0; i < RES_ROW; ++i)
+            if (32 * i + lane < n) r[32 * i + lane] = fma(-delta, v[i], r[32 * i + lane]);
+    } else {
+        const T* __restrict__ wk = a.Wt + (size_t)k * a.ldn;
+        for (int i = lane; i < n; i += 32) r[i] = fma(-delta, wk[i], r[i]);
+    }
     __syncwarp();
 }
 
 // One sweep over all coordinates of column j; returns max |delta b|.  Sets
 // `overflow` and stops if the support list is full (the move is not applied).
 template <typename T, bool STD>
-__device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, const ResArgs<T>& a, T lam,
-                            unsigned long long& moves, ColScan& cs, ResNorm& rn, bool& overflow) {
+__device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restrict__ stage,
+                            const ResArgs<T>& a, T lam,
+                            unsigned long long& moves, ResScan& cs, ResNorm& rn, bool& overflow) {
     const int lane = threadIdx.x & 31;
     const int p = a.p, ldp = a.ldp;
     const int n4 = (a.n + 3) & ~3;
@@ -225,21 +299,25 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, const ResAr
         if constexpr (STD) {
             if (!((full >> bit) & 1u)) {
                 // a quiet chunk: its support coordinates in turn.  One costs a
-                // chain of n/2 fused multiply-adds over a row held in L1; the
-                // whole slice it replaces read n rows of 512 bytes from L2.
-                if (e0 < e1) prefetch_row<T>(a.Wt + (size_t)s.idx[e0] * a.ldn, a.n);
+                // chain of n/2 fused multiply-adds over its row, which is loaded
+                // under the chain before it; the whole slice it replaces read
+                // n rows of 512 bytes from L2.
+                T nx[RES_ROW];
+                if (a.stage && e0 < e1) load_row<T>(a, s.idx[e0], nx);
                 for (int e = e0; e < e1;) {
                     const int k = s.idx[e];
                     const T bk = s.val[e];
-                    if (e + 1 < s.n) prefetch_row<T>(a.Wt + (size_t)s.idx[e + 1] * a.ldn, a.n);
-                    const T* __restrict__ wk = a.Wt + (size_t)k * a.ldn;
-                    const T nb = soft<T>(column_dot<T>(wk, n4, r) + bk, lam);  // ||w_k||^2 = 1
+                    T v[RES_ROW];
+#pragma unroll
+                    for (int i = 0; i < RES_ROW; ++i) v[i] = nx[i];
+                    if (a.stage && e + 1 < e1) load_row<T>(a, s.idx[e + 1], nx);
+                    const T nb = soft<T>(coordinate_dot<T>(a, k, v, stage, r) + bk, lam);  // ||w_k||^2 = 1
                     if (nb == bk) {
                         ++e;
                         continue;
                     }
                     const T delta = nb - bk;
-                    __syncwarp();                 // every lane has read r and the list
+                    __syncwarp();                 // every lane has read the list
                     support_set<T>(s, e, k, nb);
                     if (nb == T(0)) {
                         --e1;
@@ -248,7 +326,7 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, const ResAr
                         ++e;
                     }
                     maxd = fmax(maxd, fabs(delta));
-                    note_residual_move<T>(r, wk, a.n, delta, cs, rn);
+                    note_residual_move<T, STD>(r, k, a, v, delta, cs, rn);
                     ++moves;
                 }
                 if (lane == 0) cs.ci[ci].nsupp = e1 - e0;
@@ -274,8 +352,19 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, const ResAr
                     if (u == t) bv[u] = s.val[e];
             }
         }
+        // The slice is exact until the chunk's first move.  After it only the
+        // coordinates that can still move are formed again, one at a time: the
+        // support's and those at zero that the growth since may have carried to
+        // the threshold.  More than RES_OPEN of them (about what a slice costs),
+        // and every move without standardisation, form the slice again.
+        bool fresh = true, gone = false;
+        float grow = 0.f;
+        unsigned formed_at = cs.nmoves;
         int cursor = cb;
         for (;;) {
+            const float reach = (float)lam - (grow * (1.0f + 0x1p-10f) +
+                                              rn.rmax * (float)(a.n + 64) * 0x1p-21f +
+                                              (float)lam * 0x1p-20f);
             T nbv[SCAN_V];
             unsigned mvmask = 0u;
 #pragma unroll
@@ -283,28 +372,57 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, const ResAr
                 const int k = k0 + t;
                 nbv[t] = bv[t];
                 if (k >= cursor && k < p && k != j) {
-                    T nb;
-                    if constexpr (STD) {
-                        nb = soft<T>(acc[t] + bv[t], lam);                 // ||w_k||^2 = 1
-                    } else {
-                        const T dk = a.diag[k];
-                        nb = soft<T>(acc[t] + dk * bv[t], lam) / dk;       // Soft(c, lambda)/S_kk
+                    if (fresh) {
+                        T nb;
+                        if constexpr (STD) {
+                            nb = soft<T>(acc[t] + bv[t], lam);                 // ||w_k||^2 = 1
+                        } else {
+                            const T dk = a.diag[k];
+                            nb = soft<T>(acc[t] + dk * bv[t], lam) / dk;       // Soft(c, lambda)/S_kk
+                        }
+                        nbv[t] = nb;
+                        if (nb != bv[t]) mvmask |= 1u << t;
+                    } else if (!STD || bv[t] != T(0) ||
+                               !(fabsf((float)acc[t]) * (1.0f + 0x1p-22f) < reach)) {
+                        mvmask |= 1u << t;
                     }
-                    nbv[t] = nb;
-                    if (nb != bv[t]) mvmask |= 1u << t;
                 }
             }
             const unsigned bal = __ballot_sync(FULL_MASK, mvmask != 0u);
             if (bal == 0u) break;
+            if (!fresh && (!STD || __reduce_add_sync(FULL_MASK, __popc(mvmask)) > RES_OPEN)) {
+                if (in) slice_dot<T>(a.W, ldp, n4, k0, r, acc);
+                fresh = true;
+                grow = 0.f;
+                formed_at = cs.nmoves;
+                continue;
+            }
             const int f = __ffs(bal) - 1;
             const int tf = __ffs(__shfl_sync(FULL_MASK, mvmask, f)) - 1;
             T nb_sel = nbv[0], b_sel = bv[0];
 #pragma unroll
             for (int t = 1; t < SCAN_V; ++t)
                 if (t == tf) { nb_sel = nbv[t]; b_sel = bv[t]; }
-            const T nbs = __shfl_sync(FULL_MASK, nb_sel, f);
-            const T delta = nbs - __shfl_sync(FULL_MASK, b_sel, f);
+            T nbs = __shfl_sync(FULL_MASK, nb_sel, f);
+            const T bs = __shfl_sync(FULL_MASK, b_sel, f);
             const int ks = cb + f * SCAN_V + tf;
+            cursor = ks + 1;
+            T v[RES_ROW];
+            if (a.stage) load_row<T>(a, ks, v);
+            if (!fresh) {
+                const T gk = coordinate_dot<T>(a, ks, v, stage, r);
+                if constexpr (STD) {
+                    nbs = soft<T>(gk + bs, lam);
+                } else {
+                    const T dk = a.diag[ks];
+                    nbs = soft<T>(gk + dk * bs, lam) / dk;
+                }
+                if (nbs == bs) {
+                    if (cursor >= cb + CHUNK) break;
+                    continue;
+                }
+            }
+            const T delta = nbs - bs;
             int pos = e0;
             while (pos < e1 && s.idx[pos] < ks) ++pos;
             const int n_before = s.n;
@@ -320,18 +438,16 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, const ResAr
             }
             maxd = fmax(maxd, fabs(delta));
             ++moves;
-            note_residual_move<T>(r, a.Wt + (size_t)ks * a.ldn, a.n, delta, cs, rn);
-            cursor = ks + 1;
+            note_residual_move<T, STD>(r, ks, a, v, delta, cs, rn);
+            fresh = false;
+            gone |= nbs == T(0);
+            if constexpr (STD) grow += fabsf((float)delta) * chunk_bound(a, ks, ci);
             if (cursor >= cb + CHUNK) break;
-            // the slice again from the new residual (every lane, so that the
-            // chunk summary below refers to one residual)
-            if (in) slice_dot<T>(a.W, ldp, n4, k0, r, acc);
         }
         if constexpr (STD) {
-            // the summary must describe the residual after the chunk's last
-            // move: a move at the chunk's end left the slice one move behind
-            if (cursor >= cb + CHUNK && cs.nmoves != nmoves0 && in)
-                slice_dot<T>(a.W, ldp, n4, k0, r, acc);
+            // the summary: the slice as it was formed, and the growth since.  A
+            // coordinate that came to zero here moved its own gradient by more
+            // than the growth: it marks the chunk.
             float mx = 0.f;
 #pragma unroll
             for (int t = 0; t < SCAN_V; ++t) {
@@ -340,7 +456,7 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, const ResAr
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL_MASK, mx, o));
-            if (lane == 0) cs.ci[ci] = ChunkInfo{mx, cs.dsum, cs.nmoves, e1 - e0};
+            if (lane == 0) cs.ci[ci] = ResChunk{gone ? INFINITY : mx, grow, formed_at, e1 - e0};
             __syncwarp();
             if (cs.nmoves != nmoves0) {
                 mbase = ci + 1;
@@ -391,8 +507,14 @@ __device__ void solve_column_residual(int j, unsigned char* wsm, const ResArgs<T
     s.idx = reinterpret_cast<int*>(wsm + (size_t)a.ldn * sizeof(T));
     s.val = reinterpret_cast<T*>(s.idx + LAZY_CAP);
     s.n = 0;
-    ColScan cs{reinterpret_cast<ChunkInfo*>(s.val + LAZY_CAP), 0.f, 0u};
-    reset_chunks(cs, a.ldp);
+    ResScan cs{reinterpret_cast<ResChunk*>(s.val + LAZY_CAP), 0u};
+    {
+        // b = 0: g_k = w_k' w_j, bounded per chunk by the table
+        const int nch = num_chunks(a.ldp);
+        for (int c = lane; c < nch; c += 32)
+            cs.ci[c] = ResChunk{STD ? chunk_bound(a, j, c) : INFINITY, 0.f, 0u, 0};
+    }
+    T* stage = reinterpret_cast<T*>(cs.ci + num_chunks(a.ldp));
     // r_j = w_j (b = 0); rows of Wt are zero past n
     const T* wj = a.Wt + (size_t)j * a.ldn;
     double q0 = 0.0;
@@ -417,7 +539,7 @@ __device__ void solve_column_residual(int j, unsigned char* wsm, const ResArgs<T
         const T lam = (T)(sigma * a.lambda0);
         bool inner_ok = false;
         for (int m = 0; m < a.maxit; ++m) {
-            const T md = sweep_residual<T, STD>(j, s, r, a, lam, cnt.moves, cs, rn, overflow);
+            const T md = sweep_residual<T, STD>(j, s, r, stage, a, lam, cnt.moves, cs, rn, overflow);
             ++cnt.sweeps;
             if (overflow) break;
             if ((double)md < a.tol) {
@@ -434,8 +556,10 @@ __device__ void solve_column_residual(int j, unsigned char* wsm, const ResArgs<T
         double q = residual_reset<T>(j, s, r, a, dr);
         // the recomputed residual moved r by dr: one move of that size for the
         // skip bound
-        cs.dsum += (float)dr * (1.0f + 0x1p-8f);
+        for (int c = lane; c < num_chunks(a.ldp); c += 32)
+            cs.ci[c].grow += (float)dr * (1.0f + 0x1p-8f);
         ++cs.nmoves;
+        __syncwarp();
         rn.rb = (float)sqrt(q) * (1.0f + 0x1p-20f);
         rn.rmax = fmaxf(rn.rmax, rn.rb);
         if (q <= floor2) {
@@ -469,7 +593,8 @@ __global__ void __launch_bounds__(256) cd_residual_kernel(ResArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    unsigned char* wsm = smem_raw + (size_t)warp * res_warp_smem_bytes<T>(a.ldn, a.ldp);
+    unsigned char* wsm = smem_raw + (size_t)warp * (res_warp_smem_bytes<T>(a.ldn, a.ldp) +
+                                                    (a.stage ? a.ldn * sizeof(T) : 0));
     FitCtrl* ctrl = a.ctrl;
     if (*reinterpret_cast<volatile int*>(&ctrl->err) != 0) return;
     ColCounters cnt;
@@ -552,6 +677,84 @@ __global__ void res_build_kernel(const T* __restrict__ X, int n, int p, int ldx,
     }
 }
 
+// The bounds of chunk_bound: one block of 128 threads forms 64 columns j against
+// the chunks of one byte in FP32, 8 x 8 products a thread, and keeps only the
+// row maxima; n 2^-23 covers the rounding of the dots (and of W to FP32).
+// Bound by the FP32 pipe: p = 2000, n = 200 0.05 ms.
+constexpr int CM_BJ = 64, CM_BK = 16, CM_THREADS = 128;
+template <typename T>
+__global__ void __launch_bounds__(CM_THREADS) res_cmax_kernel(const T* __restrict__ W, int n, int p,
+                                                             int ldp, int cm_chunks,
+                                                             unsigned char* __restrict__ cmax0,
+                                                             unsigned char* __restrict__ cmax1,
+                                                             FitCtrl* ctrl) {
+    if (*reinterpret_cast<volatile int*>(&ctrl->err) != 0) return;
+    __shared__ __align__(16) float As[CM_BK][CM_BJ], Bs[CM_BK][CHUNK];
+    const int g = blockIdx.x, j0 = blockIdx.y * CM_BJ;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;     // 16 x 8
+    const int c_end = min((g + 1) * cm_chunks, num_chunks(ldp));
+    float m[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) m[u] = 0.f;
+    for (int c = g * cm_chunks; c < c_end; ++c) {
+        const int k0 = c * CHUNK;
+        float acc[8][8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int v = 0; v < 8; ++v) acc[u][v] = 0.f;
+        for (int i0 = 0; i0 < n; i0 += CM_BK) {
+#pragma unroll
+            for (int q = 0; q < CM_BK * CM_BJ / CM_THREADS; ++q) {
+                const int e = threadIdx.x + q * CM_THREADS, i = i0 + e / CM_BJ, col = j0 + e % CM_BJ;
+                As[e / CM_BJ][e % CM_BJ] = (i < n && col < ldp) ? (float)W[(size_t)i * ldp + col] : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < CM_BK; ++q) {
+                const int i = i0 + q, col = k0 + threadIdx.x;
+                Bs[q][threadIdx.x] = (i < n && col < ldp) ? (float)W[(size_t)i * ldp + col] : 0.f;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int kk = 0; kk < CM_BK; ++kk) {
+                float a[8], b[8];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    *reinterpret_cast<float4*>(a + 4 * h) =
+                        *reinterpret_cast<const float4*>(&As[kk][32 * h + 4 * ty]);
+                    *reinterpret_cast<float4*>(b + 4 * h) =
+                        *reinterpret_cast<const float4*>(&Bs[kk][64 * h + 4 * tx]);
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+#pragma unroll
+                    for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int j = j0 + 32 * (u >> 2) + 4 * ty + (u & 3);
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                const int k = k0 + 64 * (v >> 2) + 4 * tx + (v & 3);
+                if (k != j) m[u] = fmaxf(m[u], fabsf(acc[u][v]));
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int j = j0 + 32 * (u >> 2) + 4 * ty + (u & 3);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) m[u] = fmaxf(m[u], __shfl_xor_sync(FULL_MASK, m[u], o));
+        if (tx == 0 && j < p) {
+            const float b = m[u] * (1.0f + 0x1p-20f) + (float)(n + 4) * 0x1p-23f;   // at most 1.003
+            (g < 8 ? cmax0 + g : cmax1 + (g - 8))[8 * (size_t)j] =
+                (unsigned char)fminf(ceilf(b * 254.0f), 255.0f);
+        }
+    }
+}
+
 template <typename T>
 __global__ void res_theta_kernel(const T* __restrict__ BT, int p, int ldp,
                                  const double* __restrict__ sigma, const double* __restrict__ cs,
@@ -575,6 +778,9 @@ cudaError_t run_residual(const ResLaunch& f, const ResLayout& L, cudaStream_t st
     a.Wt = reinterpret_cast<const T*>(ws + L.Wt);
     a.BT = reinterpret_cast<T*>(ws + L.BT);
     a.diag = reinterpret_cast<const T*>(ws + L.diag);
+    a.cmax0 = ws + L.mu;
+    a.cmax1 = ws + L.wscale;
+    a.cm_chunks = (num_chunks(L.ldp) + CM_GROUPS - 1) / CM_GROUPS;
     a.sigma = reinterpret_cast<double*>(ws + L.sigma);
     a.col_status = reinterpret_cast<int*>(ws + L.col_status);
     a.ctrl = ctrl;
@@ -587,9 +793,11 @@ cudaError_t run_residual(const ResLaunch& f, const ResLayout& L, cudaStream_t st
     a.tol = f.tol;
     double* cs = reinterpret_cast<double*>(ws + L.cs);
 
-    const size_t per = res_warp_smem_bytes<T>(L.ldn, L.ldp);
+    size_t per = res_warp_smem_bytes<T>(L.ldn, L.ldp);
     const size_t budget = (size_t)smem_optin - 1024;
     if (per > budget) return cudaErrorInvalidValue;
+    a.stage = f.n <= 32 * RES_ROW && per + L.ldn * sizeof(T) <= budget;
+    if (a.stage) per += L.ldn * sizeof(T);
     int LW = f.warps_per_block > 0 ? f.warps_per_block : 8;
     LW = std::max(1, std::min({LW, 8, (int)(budget / per)}));
     const size_t smem = per * LW;
@@ -618,6 +826,10 @@ cudaError_t run_residual(const ResLaunch& f, const ResLayout& L, cudaStream_t st
             reinterpret_cast<const double*>(ws + L.wscale), reinterpret_cast<T*>(ws + L.W), L.ldp,
             reinterpret_cast<T*>(ws + L.Wt), L.ldn, ctrl);
     }
+    if (STD)
+        res_cmax_kernel<T><<<dim3((num_chunks(L.ldp) + a.cm_chunks - 1) / a.cm_chunks,
+                                  (f.p + CM_BJ - 1) / CM_BJ), CM_THREADS, 0, st>>>(
+            a.W, f.n, f.p, L.ldp, a.cm_chunks, ws + L.mu, ws + L.wscale, ctrl);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (f.phase_events) cudaEventRecord(f.phase_events[0], st);
     const int grid = std::min((f.p + LW - 1) / LW, nsm * per_sm);

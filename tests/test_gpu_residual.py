@@ -159,3 +159,23 @@ def test_quiet_chunks_at_the_edges(p, n):
     S, ref = _oracle(prob.X, prob.lambda0, 1e-10)
     res = compare_theta(T, ref["Theta"], ref["B"], ref["sigma"], rel=1e-7)
     assert res["ok"], res
+
+
+@pytest.mark.parametrize("p,n,prec,rel", [
+    (2100, 60, "fp32", 1e-4),     # more than 16 chunks: two chunks per bound
+    (130, 512, "fp64", 1e-7),     # the longest row kept in registers
+    (130, 513, "fp64", 1e-7),     # one beyond it
+    (300, 700, "fp32", 1e-4),
+])
+@pytest.mark.parametrize("standardize", [True, False])
+def test_rows_and_bounds_at_their_limits(p, n, prec, rel, standardize):
+    """The chunk bounds' groups and the rows held in registers or not, at the
+    bars of the oracle comparison above."""
+    prob = synth.make_problem("hub_scaled" if p < 2000 else "er", p, n, 7,
+                              dtype=np.float64 if prec == "fp64" else np.float32)
+    lam = prob.lambda0 * (1.0 if standardize else 1.2)
+    T, sig, st = _res(prob.X, lam, 1e-10 if prec == "fp64" else 1e-6, prec, standardize=standardize)
+    assert st["status"] == sp.SPMESL_OK
+    S, ref = _oracle(prob.X, lam, 1e-10, standardize=standardize)
+    res = compare_theta(T, ref["Theta"], ref["B"], ref["sigma"], rel=rel)
+    assert res["ok"], res

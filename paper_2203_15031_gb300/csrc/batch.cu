@@ -85,8 +85,9 @@ template <typename T>
 __global__ void batch_mean_kernel(const BatchFit* __restrict__ fits) {
     const BatchFit& f = fits[blockIdx.y];
     if (!f.X || !f.mu) return;
+    if ((int)blockIdx.x * 32 >= f.p) return;
     column_means<T>(static_cast<const T*>(f.X), f.n, f.p, f.p, static_cast<T*>(f.mu),
-                    blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+                    blockIdx.x * 32);
 }
 
 __global__ void __launch_bounds__(GRAM_THREADS) batch_gram_kernel(const BatchFit* __restrict__ fits,
@@ -396,24 +397,21 @@ __global__ void __launch_bounds__(BLK_THREADS, 1) batch_cd_block_kernel(const Ba
 }
 
 // Optimality diagnostics of every column of every fit (opts.diagnostics):
-// one warp per column, 4 warps a block, grid-stride over the columns.
-constexpr int BATCH_DIAG_WARPS = 4;
+// one block per column, grid-stride over the columns.
 template <typename T>
-__global__ void __launch_bounds__(32 * BATCH_DIAG_WARPS) batch_diag_kernel(
+__global__ void __launch_bounds__(32 * DIAG_WARPS) batch_diag_kernel(
     const BatchFit* __restrict__ fits, const int* __restrict__ col_prefix, int count,
     int total_cols) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int warp = threadIdx.x >> 5;
-    unsigned char* wsm = smem_raw + (size_t)warp * diag_warp_smem_bytes();
-    for (int gc = blockIdx.x * BATCH_DIAG_WARPS + warp; gc < total_cols;
-         gc += gridDim.x * BATCH_DIAG_WARPS) {
+    __shared__ DiagShared sh;
+    for (int gc = blockIdx.x; gc < total_cols; gc += gridDim.x) {
         const int fi = find_fit(col_prefix, count, gc);
         const BatchFit& f = fits[fi];
-        if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) continue;
+        if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) continue;   // block-uniform
         const CDArgs<T> a = column_args<T>(f, 0.0, 0.f, 1);
         DiagMax d;
-        diagnose_column<T>(gc - f.col_start, wsm, a, f.diag_eps, d);
+        diagnose_column<T>(gc - f.col_start, sh, a, f.diag_eps, d);
         flush_diag(f.ctrl, d);
+        __syncthreads();
     }
 }
 
@@ -575,7 +573,8 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
     const int count = b->count;
     if (b->any_x) {
         if (b->center)
-            batch_mean_kernel<T><<<dim3((b->max_p + 255) / 256, count), 256, 0, st>>>(fits);
+            batch_mean_kernel<T><<<dim3((b->max_p + 31) / 32, count), dim3(32, MEAN_GROUPS), 0, st>>>(
+                fits);
         if (b->precision == SPMESL_MIXED) {
             batch_split_kernel<<<b->total_split, dim3(32, 8), 0, st>>>(
                 fits, reinterpret_cast<const int*>(ws + b->off_splitp), count);
@@ -690,14 +689,8 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
     if (timed) cudaEventRecord(b->ev[1], st);
     if (b->count_rows) batch_rows_count_kernel<<<count, 256, 0, st>>>(fits);
     if (b->diagnostics) {
-        const size_t dsm = diag_warp_smem_bytes() * BATCH_DIAG_WARPS;
-        auto dk = batch_diag_kernel<T>;
-        if ((e = cudaFuncSetAttribute(dk, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)dsm)) != cudaSuccess)
-            return e;
-        const int dgrid = std::max(1, std::min((b->total_cols + BATCH_DIAG_WARPS - 1) / BATCH_DIAG_WARPS,
-                                               num_sms() * 4));
-        dk<<<dgrid, 32 * BATCH_DIAG_WARPS, dsm, st>>>(fits, colp, count, b->total_cols);
+        const int dgrid = std::max(1, std::min(b->total_cols, num_sms() * 16));
+        batch_diag_kernel<T><<<dgrid, 32 * DIAG_WARPS, 0, st>>>(fits, colp, count, b->total_cols);
     }
     if (lazy) {
         batch_inv_kernel<<<dim3((b->max_p + 255) / 256, count), 256, 0, st>>>(fits);

@@ -130,19 +130,18 @@ __global__ void rows_count_kernel(const unsigned* __restrict__ bits, size_t nwor
                      (size_t)gridDim.x * blockDim.x);
 }
 
-// Optimality diagnostics of columns [j0, j1): one warp per column
-// (diagnose_column), 4 warps a block, grid-stride over the columns.
-constexpr int DIAG_WARPS = 4;
+// Optimality diagnostics of columns [j0, j1): one block per column
+// (diagnose_column), grid-stride over the columns.
 template <typename T>
 __global__ void __launch_bounds__(32 * DIAG_WARPS) cd_diag_kernel(CDArgs<T> a, double eps, int j0,
                                                                   int j1) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int warp = threadIdx.x >> 5;
-    unsigned char* wsm = smem_raw + (size_t)warp * diag_warp_smem_bytes();
+    __shared__ DiagShared sh;
     if (*reinterpret_cast<volatile int*>(&a.ctrl->err) != 0) return;
     DiagMax d;
-    for (int j = j0 + blockIdx.x * DIAG_WARPS + warp; j < j1; j += gridDim.x * DIAG_WARPS)
-        diagnose_column<T>(j, wsm, a, eps, d);
+    for (int j = j0 + blockIdx.x; j < j1; j += gridDim.x) {
+        diagnose_column<T>(j, sh, a, eps, d);
+        __syncthreads();
+    }
     flush_diag(a.ctrl, d);
 }
 
@@ -568,13 +567,8 @@ static cudaError_t block_launch_shape(int ldp, size_t& smem, int& grid) {
 
 template <typename T>
 static cudaError_t launch_diag(const CDArgs<T>& a, double eps, int j0, int j1, cudaStream_t st) {
-    const size_t sm = diag_warp_smem_bytes() * DIAG_WARPS;
-    auto k = cd_diag_kernel<T>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    const int cols = j1 - j0;
-    const int grid = std::max(1, std::min((cols + DIAG_WARPS - 1) / DIAG_WARPS, g_num_sms * 4));
-    k<<<grid, 32 * DIAG_WARPS, sm, st>>>(a, eps, j0, j1);
+    const int grid = std::max(1, std::min(j1 - j0, g_num_sms * 16));
+    cd_diag_kernel<T><<<grid, 32 * DIAG_WARPS, 0, st>>>(a, eps, j0, j1);
     return cudaGetLastError();
 }
 

@@ -660,9 +660,9 @@ __device__ __forceinline__ bool standardize_row(const T* __restrict__ S, int p, 
                 }
             }
             if (cmax) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL_MASK, mx, o));
-                if (lane == 0) cmax[(size_t)r * nch + ch] = mx;
+                // non-negative floats order as unsigned integers (a NaN has ended the fit)
+                const unsigned top = __reduce_max_sync(FULL_MASK, __float_as_uint(mx));
+                if (lane == 0) cmax[(size_t)r * nch + ch] = __uint_as_float(top);
             }
         }
     }
@@ -1608,7 +1608,7 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
 // when the lasso subgradient conditions hold at lambda = lambda0 sigma_j
 // (Section 2.1): with g = S_.j - S b_j,
 //   g_k = lambda sign(b_k) where b_k != 0,   |g_k| <= lambda where b_k = 0,
-// and sigma_j is the fixed point of Eq. (14).  One warp per column forms the
+// and sigma_j is the fixed point of Eq. (14).  One block per column forms the
 // whole gradient in FP64 from the working matrix (row j and the support rows,
 // the lazy solver's slices accumulated in FP64) and reports
 //  - the largest violation of those conditions relative to lambda;
@@ -1626,12 +1626,19 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
 //    and 2 lambda |A| kkt from a solve that is not exactly optimal.  Then
 //    Theta_kj = -b_kj / sigma_j^2, Theta_jj = 1 / sigma_j^2 differentiated.
 // ===========================================================================
-constexpr int DIAG_CAP = 1024;         // support list of one warp
+constexpr int DIAG_CAP = 1024;         // support list of a column
+constexpr int DIAG_WARPS = 4;          // warps of a block: the column's chunks in turn.  (One warp
+                                       // a column took 92 us for p = 1003, the chain of its
+                                       // longest column; four 56.)
 static_assert(COEF_CAP <= DIAG_CAP, "a stored list must fit the diagnostics' list");
 
-__host__ __device__ constexpr size_t diag_warp_smem_bytes() {
-    return (size_t)DIAG_CAP * (sizeof(int) + sizeof(double));
-}
+// Shared memory of a diagnostics block.
+struct DiagShared {
+    int idx[DIAG_CAP];
+    double val[DIAG_CAP];
+    double kkt[DIAG_WARPS], gmax[DIAG_WARPS], bg[DIAG_WARPS];
+    int ns;
+};
 
 // Per-warp maxima of the diagnostics (non-negative doubles), flushed with
 // atomicMax on their bits.
@@ -1639,8 +1646,9 @@ struct DiagMax {
     double kkt = 0.0, gap = 0.0, err = 0.0, thmax = 0.0;
 };
 
+// (warp 0 of a diagnostics block holds the maxima)
 __device__ __forceinline__ void flush_diag(FitCtrl* ctrl, const DiagMax& d) {
-    if ((threadIdx.x & 31) == 0) {
+    if (threadIdx.x == 0) {
         atomicMax(&ctrl->diag_kkt, dbits(d.kkt));
         atomicMax(&ctrl->diag_gap, dbits(d.gap));
         atomicMax(&ctrl->diag_err, dbits(d.err));
@@ -1649,45 +1657,49 @@ __device__ __forceinline__ void flush_diag(FitCtrl* ctrl, const DiagMax& d) {
     }
 }
 
+// By a block of DIAG_WARPS warps; the maxima go to warp 0's `out`.
 template <typename T>
-__device__ void diagnose_column(int j, unsigned char* wsm, const CDArgs<T>& a, double eps_s,
+__device__ void diagnose_column(int j, DiagShared& sh, const CDArgs<T>& a, double eps_s,
                                 DiagMax& out) {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int p = a.p, ldp = a.ldp;
-    int* idx = reinterpret_cast<int*>(wsm);
-    double* val = reinterpret_cast<double*>(wsm + DIAG_CAP * sizeof(int));
+    int* __restrict__ idx = sh.idx;
+    double* __restrict__ val = sh.val;
     const T* __restrict__ brow = a.BT + (size_t)j * ldp;
     // support of b_j in ascending order: its list, or collected from a dense row
-    int ns = a.nsup ? a.nsup[j] : -1;
-    const bool dense = ns < 0;
+    const int nl = a.nsup ? a.nsup[j] : -1;
+    const bool dense = nl < 0;
     if (!dense) {
         const int* __restrict__ src = coef_idx(brow, ldp);
-        for (int e = lane; e < ns; e += 32) {
+        for (int e = threadIdx.x; e < nl; e += 32 * DIAG_WARPS) {
             idx[e] = src[e];
             val[e] = (double)brow[e];
         }
-    } else {
-        ns = 0;
+        if (threadIdx.x == 0) sh.ns = nl;
+    } else if (warp == 0) {
+        int c = 0;
         for (int c0 = 0; c0 < p; c0 += 32) {
             const int k = c0 + lane;
             const T bk = k < p ? brow[k] : T(0);
             const unsigned bal = __ballot_sync(FULL_MASK, bk != T(0));
-            const int pos = ns + __popc(bal & ((1u << lane) - 1u));
+            const int pos = c + __popc(bal & ((1u << lane) - 1u));
             if (bk != T(0) && pos < DIAG_CAP) {
                 idx[pos] = k;
                 val[pos] = (double)bk;
             }
-            ns += __popc(bal);
+            c += __popc(bal);
         }
+        if (lane == 0) sh.ns = c;
     }
-    __syncwarp();
-    int e0 = 0;                                       // list: first entry of the chunk
+    __syncthreads();
+    const int ns = sh.ns;
     const bool listed = ns <= DIAG_CAP;
+    int e0 = 0;                                       // list: first entry of the chunk
     const double sig = a.sigma[j];
     const double lam = a.lambda0 * sig;
     const T* __restrict__ Sj = a.SC + (size_t)j * ldp;
     double kkt = 0.0, gmax = 0.0, bg = 0.0;
-    for (int cb = 0; cb < p; cb += CHUNK) {
+    for (int cb = warp * CHUNK; cb < p; cb += DIAG_WARPS * CHUNK) {
         const int k0 = cb + lane * SCAN_V;
         const bool in = k0 < ldp;
         double acc[SCAN_V] = {0.0, 0.0, 0.0, 0.0};
@@ -1727,6 +1739,7 @@ __device__ void diagnose_column(int j, unsigned char* wsm, const CDArgs<T>& a, d
 #pragma unroll
                 for (int t = 0; t < SCAN_V; ++t) bq[t] = (double)r[t];
             } else {
+                while (e0 < ns && idx[e0] < cb) ++e0;
                 for (int e = e0; e < ns && idx[e] < cb + CHUNK; ++e) {
                     const int u = idx[e] - k0;
 #pragma unroll
@@ -1745,8 +1758,22 @@ __device__ void diagnose_column(int j, unsigned char* wsm, const CDArgs<T>& a, d
                 if (bk != 0.0) bg = fma(bk, g, bg);
             }
         }
-        if (!dense)
-            while (e0 < ns && idx[e0] < cb + CHUNK) ++e0;
+    }
+    kkt = warp_max(kkt);
+    gmax = warp_max(gmax);
+    bg = warp_sum(bg);
+    if (lane == 0) {
+        sh.kkt[warp] = kkt;
+        sh.gmax[warp] = gmax;
+        sh.bg[warp] = bg;
+    }
+    __syncthreads();
+    if (warp != 0) return;                            // (the caller's barrier follows)
+#pragma unroll
+    for (int w = 1; w < DIAG_WARPS; ++w) {
+        kkt = fmax(kkt, sh.kkt[w]);
+        gmax = fmax(gmax, sh.gmax[w]);
+        bg += sh.bg[w];
     }
     double bS = 0.0, l1 = 0.0, l2 = 0.0, bmax = 0.0;
     if (listed) {
@@ -1765,10 +1792,7 @@ __device__ void diagnose_column(int j, unsigned char* wsm, const CDArgs<T>& a, d
             bmax = fmax(bmax, fabs(v));
         }
     }
-    kkt = warp_max(kkt);
-    gmax = warp_max(gmax);
     bmax = warp_max(bmax);
-    bg = warp_sum(bg);
     bS = warp_sum(bS);
     l1 = warp_sum(l1);
     l2 = sqrt(warp_sum(l2));
@@ -1789,7 +1813,6 @@ __device__ void diagnose_column(int j, unsigned char* wsm, const CDArgs<T>& a, d
     out.gap = fmax(out.gap, gap);
     out.err = fmax(out.err, eth);
     out.thmax = fmax(out.thmax, 1.0 / s2);
-    __syncwarp();
 }
 
 // ===========================================================================

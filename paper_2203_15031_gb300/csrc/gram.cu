@@ -13,8 +13,7 @@ namespace {
 
 template <typename T>
 __global__ void column_mean_kernel(const T* __restrict__ X, int n, int p, int ldx, T* mu) {
-    column_means<T>(X, n, p, ldx, mu, blockIdx.x * blockDim.x + threadIdx.x,
-                    gridDim.x * blockDim.x);
+    column_means<T>(X, n, p, ldx, mu, blockIdx.x * 32);
 }
 
 template <int BM, int BK, int THREADS, int TM, int TN, bool VEC>
@@ -32,7 +31,7 @@ cudaError_t run_gram_simt(const float* X, int n, int p, int ldx, int center, flo
     float* mu = nullptr;
     if (center) {
         mu = reinterpret_cast<float*>(ws);
-        column_mean_kernel<float><<<(p + 255) / 256, 256, 0, st>>>(X, n, p, ldx, mu);
+        column_mean_kernel<float><<<(p + 31) / 32, dim3(32, MEAN_GROUPS), 0, st>>>(X, n, p, ldx, mu);
     }
     const float inv_n = (float)(1.0 / (double)n);
     const int tw = (p + GRAM_WIDE - 1) / GRAM_WIDE, t = (p + GRAM_BM - 1) / GRAM_BM;

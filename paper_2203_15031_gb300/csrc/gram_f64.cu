@@ -395,8 +395,7 @@ __global__ void __launch_bounds__(256) f64_digits_kernel(const double* __restric
 }
 
 __global__ void f64_mean_kernel(const double* __restrict__ X, int n, int p, int ldx, double* mu) {
-    column_means<double>(X, n, p, ldx, mu, blockIdx.x * blockDim.x + threadIdx.x,
-                         gridDim.x * blockDim.x);
+    column_means<double>(X, n, p, ldx, mu, blockIdx.x * 32);
 }
 
 template <class Src>
@@ -456,7 +455,7 @@ cudaError_t launch_gram_f64(const double* X, int n, int p, int ldx, int center, 
     F64One one;
     if (!f64_encode_fit(one.f, X, n, p, ldx, mu, expo, D, S, lds, 0)) return cudaErrorInvalidValue;
     one.n_tiles = one.f.g.count();
-    if (center) f64_mean_kernel<<<(p + 255) / 256, 256, 0, st>>>(X, n, p, ldx, mu);
+    if (center) f64_mean_kernel<<<(p + 31) / 32, dim3(32, MEAN_GROUPS), 0, st>>>(X, n, p, ldx, mu);
     f64_digits_kernel<<<(p + 31) / 32, dim3(32, 8), 0, st>>>(X, n, p, ldx, mu, expo, D, one.f.n_pad);
     return launch_tiles(one, one.n_tiles, st);
 }

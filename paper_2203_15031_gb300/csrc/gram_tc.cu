@@ -103,8 +103,7 @@ __global__ void split_transpose_kernel(const float* __restrict__ X, int n, int p
 }
 
 __global__ void tc_mean_kernel(const float* __restrict__ X, int n, int p, int ldx, float* mu) {
-    column_means<float>(X, n, p, ldx, mu, blockIdx.x * blockDim.x + threadIdx.x,
-                        gridDim.x * blockDim.x);
+    column_means<float>(X, n, p, ldx, mu, blockIdx.x * 32);
 }
 
 // Where one tile's operands and output are.
@@ -493,7 +492,7 @@ cudaError_t launch_gram_tc(const float* X, int n, int p, int ldx, int center, fl
     __nv_bfloat16* XhT = reinterpret_cast<__nv_bfloat16*>(base + align_up((size_t)p * 4, 256));
     __nv_bfloat16* XlT = reinterpret_cast<__nv_bfloat16*>(
         reinterpret_cast<unsigned char*>(XhT) + align_up((size_t)p * n_pad * 2, 256));
-    if (center) tc_mean_kernel<<<(p + 255) / 256, 256, 0, st>>>(X, n, p, ldx, mu);
+    if (center) tc_mean_kernel<<<(p + 31) / 32, dim3(32, MEAN_GROUPS), 0, st>>>(X, n, p, ldx, mu);
     split_transpose_kernel<<<dim3(n_pad / 32, (p + 31) / 32), dim3(32, 8), 0, st>>>(
         X, n, p, ldx, center ? mu : nullptr, XhT, XlT, n_pad);
     // 128 x 256 tiles cut the operand traffic per flop by a quarter against

@@ -42,6 +42,7 @@
 #include <algorithm>
 
 #include "cd_device.cuh"
+#include "gram_device.cuh"
 
 namespace spmesl {
 namespace {
@@ -608,7 +609,8 @@ __global__ void __launch_bounds__(256) cd_residual_kernel(ResArgs<T> a) {
     flush_counters(ctrl, cnt);
 }
 
-// Per column k (one thread): mu_k (0 without centring), s_kk = ||x_k - mu_k||^2 / n
+// Per column k (32 columns a 32 x 8 block, see column_means): mu_k (0 without
+// centring), s_kk = ||x_k - mu_k||^2 / n
 // in FP64, c_k = s_kk^-1/2 when standardising (else 1), the factor
 // c_k / sqrt(n) that makes w_k, the working diagonal ||w_k||^2 = c_k^2 s_kk,
 // and the starting sigma = 1.  Non-finite data or s_kk <= 0 sets
@@ -619,18 +621,30 @@ __global__ void res_stats_kernel(const T* __restrict__ X, int n, int p, int ldx,
                                  double* __restrict__ mu, double* __restrict__ wscale,
                                  T* __restrict__ diag, double* __restrict__ sigma,
                                  int* __restrict__ col_status, FitCtrl* ctrl) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= p) return;
+    __shared__ double part[MEAN_GROUPS][33];
+    __shared__ double mean[32];
+    const int k = blockIdx.x * 32 + threadIdx.x;
     double m = 0.0;
     if (center) {
-        for (int i = 0; i < n; ++i) m += (double)X[(size_t)i * ldx + k];
-        m /= (double)n;
+        if (k < p) {
+#pragma unroll 8
+            for (int i = threadIdx.y; i < n; i += MEAN_GROUPS) m += (double)X[(size_t)i * ldx + k];
+        }
+        m = group_sum(m, part) / (double)n;
+        if (threadIdx.y == 0) mean[threadIdx.x] = m;
+        __syncthreads();
+        m = mean[threadIdx.x];
     }
     double ss = 0.0;
-    for (int i = 0; i < n; ++i) {
-        const double d = (double)X[(size_t)i * ldx + k] - m;
-        ss = fma(d, d, ss);
+    if (k < p) {
+#pragma unroll 8
+        for (int i = threadIdx.y; i < n; i += MEAN_GROUPS) {
+            const double d = (double)X[(size_t)i * ldx + k] - m;
+            ss = fma(d, d, ss);
+        }
     }
+    ss = group_sum(ss, part);
+    if (threadIdx.y != 0 || k >= p) return;
     const double skk = ss / (double)n;
     if (!(skk > 0.0) || !isfinite(skk) || !isfinite(m)) set_error(ctrl, DEV_ERR_NONFINITE);
     const double c = standardize ? 1.0 / sqrt(skk) : 1.0;
@@ -815,7 +829,7 @@ cudaError_t run_residual(const ResLaunch& f, const ResLayout& L, cudaStream_t st
     if ((e = cudaMemsetAsync(ws + L.BT, 0, (size_t)f.p * L.ldp * sizeof(T), st)) != cudaSuccess)
         return e;
     const T* X = static_cast<const T*>(f.X);
-    res_stats_kernel<T><<<(f.p + 127) / 128, 128, 0, st>>>(
+    res_stats_kernel<T><<<(f.p + 31) / 32, dim3(32, MEAN_GROUPS), 0, st>>>(
         X, f.n, f.p, f.ldx, f.center, f.standardize, cs, reinterpret_cast<double*>(ws + L.mu),
         reinterpret_cast<double*>(ws + L.wscale), reinterpret_cast<T*>(ws + L.diag), a.sigma,
         a.col_status, ctrl);

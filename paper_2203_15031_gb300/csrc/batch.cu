@@ -218,10 +218,12 @@ __global__ void __launch_bounds__(32 * PREP_ROWS) batch_prep_matrix_kernel(
     const int r = (blockIdx.x - f.prep_start) * PREP_ROWS + (int)(threadIdx.x >> 5);
     if (r >= f.p) return;                      // warp-uniform
     int cnt = 0;
+    float top = 0.f;
     const bool bad = standardize_row<T>(static_cast<const T*>(f.S), f.p, f.ldp, r, f.cs, f.csf,
                                         static_cast<T*>(f.SC), nullptr, nullptr,
                                         static_cast<T*>(f.diag), lane, 32, (T)f.lambda0,
-                                        heat ? &cnt : nullptr, f.cmax);
+                                        heat ? &cnt : nullptr, f.cmax, &top);
+    if (f.cmax && lane == 0) static_cast<T*>(f.diag)[r] = (T)top;
     if (heat) {
         cnt = __reduce_add_sync(FULL_MASK, cnt);
         if (lane == 0) heat[f.col_start + r] = min(cnt, f.p >= heavy_min_p ? INT_MAX : heavy_heat);

@@ -373,13 +373,24 @@ template <typename T>
 __global__ void prep_matrix_kernel(const T* __restrict__ S, int p, int ldp, const double* cs,
                                    const float* csf, T* SC, T* GT, T* diag, int init_g,
                                    FitCtrl* ctrl, T heat_lam, int* heat, float* cmax) {
+    __shared__ float top[32];
     bool bad = false;
     for (int r = blockIdx.x; r < p; r += gridDim.x) {
         int cnt = 0;
+        float m = 0.f;
         bad |= standardize_row<T>(S, p, ldp, r, cs, csf, SC, init_g ? GT : nullptr, nullptr,
                                   diag, threadIdx.x, blockDim.x, heat_lam, heat ? &cnt : nullptr,
-                                  cmax);
+                                  cmax, &m);
         if (cnt) atomicAdd(&heat[r], cnt);
+        if (cmax) {
+            if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = m;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, top[w]);
+                diag[r] = (T)m;
+            }
+            __syncthreads();
+        }
     }
     if (bad) set_error(ctrl, DEV_ERR_NONFINITE);
 }

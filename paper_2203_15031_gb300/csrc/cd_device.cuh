@@ -14,7 +14,8 @@ struct CDArgs {
     const T* SC;
     T* BT;
     T* GT;
-    const T* diag;       // S_kk of the working matrix (unstandardised update)
+    const T* diag;       // S_kk of the working matrix (unstandardised update); with chunk_max
+                         // (standardised lazy solves) max_k |S^C_jk|, k != j, instead
     double* sigma;       // working-scale sigma
     int* col_status;
     int* active;
@@ -241,6 +242,18 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// (double)x without the FP64 pipe, where a conversion takes as long as an
+// addition: the exponent rebased and the fraction moved, by integer
+// instructions.  Exact for zero and normal x; a denormal FP32 value (below
+// 2^-126, 26 decades under any sigma^2 it could enter) gives zero.
+__device__ __forceinline__ double exact_double(float x) {
+    const unsigned u = __float_as_uint(x);
+    const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+    const bool normal = (u & 0x7f800000u) != 0u;
+    return __hiloint2double(normal ? (int)hi : 0, normal ? (int)(u << 29) : 0);
+}
+__device__ __forceinline__ double exact_double(double x) { return x; }
+
 // Ordered bits of a non-negative double (for atomicMax).
 __device__ __forceinline__ unsigned long long dbits(double x) {
     return (unsigned long long)__double_as_longlong(x);
@@ -331,21 +344,24 @@ struct ChunkInfo {
 // Scan state of one column solve (warp-uniform).
 struct ColScan {
     ChunkInfo* ci;
-    float dsum;          // running sum of the l1 size of every change of b_j so far: one
-                         // move's |delta|, or an active-set phase's net change
+    float dsum;          // running sum of the size of every change of b_j so far: one
+                         // move's |delta|, or an active-set phase's net change; in the lazy
+                         // solver each |delta_m| times max_k |S_mk|
     unsigned nmoves;     // number of those changes
-    float bl1;           // lazy solver: an upper bound of ||b_j||_1 (0 elsewhere)
+    float bl1;           // lazy solver: an upper bound of ||b_j||_1 so far (0 elsewhere)
 };
 
 // A chunk with no support can be skipped when no coordinate in it can reach
 // the threshold: each move delta_m at row m changes g_k by -S_km delta_m with
 // |S_km| <= 1 (standardised), so |g_k| <= maxabs + sum|delta| since the chunk
 // was scanned (and a change of several coefficients at once moves g_k by at
-// most its l1 size).  The lazy solver forms g_k afresh from S rows at every
+// most its l1 size).  The lazy solver counts each |delta_m| times the largest
+// off-diagonal |S_mk| of row m (an Erdos-Renyi column at p = 2000 forms 6.2
+// slices instead of 10.1, one of an AR(1) network at p = 1000 13.1 instead of
+// 16.8).  It forms g_k afresh from S rows at every
 // scan: each of the two computations (then and now) is off by at most
 // 384 * 2^-24 (1 + ||b||_1) (up to 256 support rows and 128 moves in a
-// chunk, |S| <= 1), the last term below with ||b_then||_1 <=
-// ||b_now||_1 + the change since.  The margins cover FP32 rounding of the standardised S
+// chunk, |S| <= 1), the last term below with bl1 bounding ||b||_1 then and now.  The margins cover FP32 rounding of the standardised S
 // (|S_km| <= 1 + 2^-22), of every g update (half an ulp of a value below
 // lambda) and of the running sum (each of the dm additions since the scan is
 // off by at most 2^-24 of the sum, which only grows); after 4096 moves the
@@ -569,8 +585,9 @@ __device__ double residual_quadratic_form(int j, const T* __restrict__ b, const 
 // nthr a multiple of 32).  Optional outputs: heat, this thread's count of
 // off-diagonal |SC_rc| > heat_lam; cmax, per chunk c of the row the largest
 // off-diagonal |SC_rk| (row r of a p x num_chunks(ldp) table; S^C is
-// symmetric, so it is also column r's first-sweep gradient bound).  Returns
-// true if a non-finite entry was seen.
+// symmetric, so it is also column r's first-sweep gradient bound); with it,
+// *rowmax takes the largest of the warp's chunks and diag is left to the
+// caller.  Returns true if a non-finite entry was seen.
 constexpr int STD_U = 4;
 template <typename T>
 __device__ __forceinline__ bool standardize_row(const T* __restrict__ S, int p, int ldp, int r,
@@ -579,7 +596,8 @@ __device__ __forceinline__ bool standardize_row(const T* __restrict__ S, int p, 
                                                 T* __restrict__ SC, T* __restrict__ GT,
                                                 T* __restrict__ BT, T* __restrict__ diag, int tid,
                                                 int nthr, T heat_lam = T(0), int* heat = nullptr,
-                                                float* __restrict__ cmax = nullptr) {
+                                                float* __restrict__ cmax = nullptr,
+                                                float* rowmax = nullptr) {
     bool bad = false;
     const int lane = tid & 31;
     const T cr = sizeof(T) == 4 ? (T)csf[r] : (T)cs[r];
@@ -633,7 +651,7 @@ __device__ __forceinline__ bool standardize_row(const T* __restrict__ S, int p, 
                     const T cc = sizeof(T) == 4 ? (T)csf[c] : (T)cs[c];
                     v[t] = sv[u][t] * cr * cc;
                     if (c == r) {
-                        diag[r] = v[t];
+                        if (!cmax) diag[r] = v[t];
                     } else {
                         mx = fmaxf(mx, (float)fabs(v[t]));
                         if (heat && fabs(v[t]) > heat_lam) ++*heat;
@@ -663,6 +681,7 @@ __device__ __forceinline__ bool standardize_row(const T* __restrict__ S, int p, 
                 // non-negative floats order as unsigned integers (a NaN has ended the fit)
                 const unsigned top = __reduce_max_sync(FULL_MASK, __float_as_uint(mx));
                 if (lane == 0) cmax[(size_t)r * nch + ch] = __uint_as_float(top);
+                *rowmax = fmaxf(*rowmax, __uint_as_float(top));
             }
         }
     }
@@ -703,15 +722,22 @@ __device__ __forceinline__ void flush_counters(FitCtrl* ctrl, ColCounters& c) {
 // so only the differences are taken in FP64 and the step itself (relative to
 // s1) is formed and safeguarded in FP32: FP64 arithmetic is scarce on this
 // part and every column takes this step a few times.
-__device__ __forceinline__ double sigma_step(double s0, double f0, double s1, double f1) {
-    const float g1 = (float)(f1 - s1), g0 = (float)(f0 - s0), ds = (float)(s1 - s0);
+// g0 and g1 are (float)(F(s0) - s0) and (float)(f1 - s1).
+__device__ __forceinline__ double sigma_step(double s0, float g0, double s1, double f1, float g1) {
+    const float ds = (float)(s1 - s0);
     const float den = g1 - g0;
     if (den == 0.0f) return f1;
     const float step = -g1 * (ds / den);                  // candidate - s1
     const float w = 4.0f * fabsf(g1);
     const float lo = fminf(0.0f, g1) - w, hi = fmaxf(0.0f, g1) + w;
-    const double cand = s1 + (double)step;
-    return (cand > 0.0 && step >= lo && step <= hi) ? cand : f1;
+    const double cand = s1 + exact_double(step);
+    // cand > 0, on the bits
+    return (__double_as_longlong(cand) > 0 && step >= lo && step <= hi) ? cand : f1;
+}
+
+// |d| < tol (tol > 0) on the bits of d.
+__device__ __forceinline__ bool below(double d, double tol) {
+    return abs_bits(d) < __double_as_longlong(tol);
 }
 
 // sqrt(q) for q > 0 in FP64 by one step of Newton's (Heron's) iteration
@@ -722,8 +748,8 @@ static __device__ __noinline__ double sqrt_far(double q) { return sqrt(q); }
 __device__ __forceinline__ double sqrt_heron(double q) {
     const float yf = sqrtf((float)q);
     if (!(yf > 1e-18f && yf < 1e18f)) return sqrt_far(q);
-    const double y0 = (double)yf;
-    return fma(fma(-y0, y0, q), (double)(0.5f / yf), y0);
+    const double y0 = exact_double(yf);
+    return fma(fma(-y0, y0, q), exact_double(0.5f / yf), y0);
 }
 
 // Algorithm 1 for response column j, by one warp: warm start from b = 0,
@@ -772,7 +798,7 @@ __device__ void solve_column(int j, T* __restrict__ g, T* __restrict__ b, int* _
         }
         double nxt = sn;
         if (have_prev && r + 1 < a.maxit && !(status & COL_DEGENERATE))
-            nxt = sigma_step(s_prev, f_prev, sigma, sn);
+            nxt = sigma_step(s_prev, (float)(f_prev - s_prev), sigma, sn, (float)(sn - sigma));
         s_prev = sigma;
         f_prev = sn;
         have_prev = true;
@@ -840,6 +866,7 @@ struct SupportBlock {
     T* saa;
     T* row;            // S_{j A_m}
     T* col;            // S_{A_m j}
+    float* top;        // max_k |S_{A_m k}|, k != A_m (standardised)
     int* list;
     float2* tb;
     int n;
@@ -851,7 +878,7 @@ struct SupportBlock {
 template <typename T>
 __host__ __device__ constexpr size_t lazy_warp_smem_bytes(int ldp) {
     return (size_t)LAZY_CAP * (sizeof(int) + sizeof(T)) + (size_t)num_chunks(ldp) * sizeof(ChunkInfo) +
-           4 * sizeof(double) + (size_t)ACT_MAX * (ACT_MAX + 2) * sizeof(T) + ACT_MAX * sizeof(int) +
+           4 * sizeof(double) + (size_t)ACT_MAX * (ACT_MAX + 2) * sizeof(T) + 2 * ACT_MAX * sizeof(int) +
            (sizeof(T) == 4 ? ACT_MAX * sizeof(float2) : 0);
 }
 
@@ -1032,7 +1059,7 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
         float l1 = 0.f;
 #pragma unroll 1
         for (int e = lane; e < s.n; e += 32) l1 += fabsf((float)s.val[e]);
-        cs.bl1 = warp_l1_bound(l1) * (1.0f + 0x1p-16f);
+        cs.bl1 = fmaxf(cs.bl1, warp_l1_bound(l1) * (1.0f + 0x1p-16f));
     }
     unsigned mask = chunks_to_scan<STD>(cs, 0, nch, (float)lam, frozen);
     for (;;) {
@@ -1147,9 +1174,10 @@ __device__ T sweep_column_lazy(int j, Support<T>& s, const CDArgs<T>& a, T lam,
             }
             maxd = fmax(maxd, fabs(delta));
             ++moves;
-            cs.dsum += fabsf((float)delta);
+            if constexpr (STD)
+                cs.dsum += fabsf((float)delta) * (float)a.diag[ks] * (1.0f + 0x1p-20f);
             ++cs.nmoves;
-            cs.bl1 += fabsf((float)delta);
+            cs.bl1 += fabsf((float)delta) * (1.0f + 0x1p-16f);
             // rank-1 update of the rest of this chunk's slice
             if (in) {
                 T r[SCAN_V];
@@ -1300,6 +1328,8 @@ __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, Sup
         // (independent loads)
         const T rv = lane < n ? a.SC[(size_t)j * ldp + my] : T(0);
         const T cv = lane < n ? a.SC[(size_t)my * ldp + j] : T(0);
+        float tv = 0.f;
+        if constexpr (STD) tv = lane < n ? (float)a.diag[my] : 0.f;
 #pragma unroll 1
         for (int k0 = 0; k0 < n; k0 += 4) {
             T v[4];
@@ -1314,6 +1344,7 @@ __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, Sup
         }
         sb.row[lane] = rv;
         sb.col[lane] = cv;
+        sb.top[lane] = tv;
         sb.list[lane] = my;
         sb.n = n;
     }
@@ -1360,7 +1391,7 @@ __device__ int active_phase(int j, Support<T>& s, const CDArgs<T>& a, T lam, Sup
     }
     moves += mv;
     // the phase enters the running sums as one change: its net l1 size
-    const float net = warp_l1_bound(lane < n ? (float)(b - b_start) : 0.f);
+    const float net = warp_l1_bound(lane < n ? (float)(b - b_start) * sb.top[lane] : 0.f);
     cs.dsum += net * (1.0f + 0x1p-16f);
     ++cs.nmoves;
     // write back, dropping coordinates at zero (the list stays sorted)
@@ -1403,7 +1434,7 @@ __device__ double residual_quadratic_form_list(int j, const Support<T>& s, const
 #pragma unroll 1
     for (int u = lane; u < n; u += 32) {
         const T suj = held ? sb.col[u] : a.SC[(size_t)s.idx[u] * ldp + j];
-        acc = fma((double)(T(-2) * s.val[u]), (double)suj, acc);
+        acc = fma(exact_double(T(-2) * s.val[u]), exact_double(suj), acc);
     }
     const int np = n * n;
     if (lane < np) {
@@ -1415,9 +1446,9 @@ __device__ double residual_quadratic_form_list(int j, const Support<T>& s, const
         const int q = (int)(32.5f * rn), r = 32 - q * n;
 #pragma unroll 1
         for (int t = lane; t < np; t += 32) {
-            const double bb = (double)s.val[u] * (double)s.val[v];
+            const double bb = exact_double(s.val[u]) * exact_double(s.val[v]);
             const T suv = held ? sb.saa[v * ACT_MAX + u] : a.SC[(size_t)s.idx[u] * ldp + s.idx[v]];
-            acc = fma(bb, (double)suv, acc);
+            acc = fma(bb, exact_double(suv), acc);
             u += q;
             v += r;
             if (v >= n) {
@@ -1426,8 +1457,12 @@ __device__ double residual_quadratic_form_list(int j, const Support<T>& s, const
             }
         }
     }
-    acc = warp_sum(acc);
-    return sjj + acc;
+    // the warp sum over the lanes that hold terms (n^2 of them, n >= 1): the
+    // others would add exact zeros
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        if (o < np) acc += __shfl_xor_sync(FULL_MASK, acc, o);
+    return sjj + __shfl_sync(FULL_MASK, acc, 0);
 }
 
 // b_j as the whole dense row j of BT, zeros included (16-byte stores; ldp is a
@@ -1505,8 +1540,9 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
     sb.col = sb.row + ACT_MAX;
     sb.tb = reinterpret_cast<float2*>(sb.col + ACT_MAX);
     sb.list = reinterpret_cast<int*>(sb.tb + (sizeof(T) == 4 ? ACT_MAX : 0));
+    sb.top = reinterpret_cast<float*>(sb.list + ACT_MAX);
     sb.n = -1;
-    if (lane == 0) prev[2] = (double)a.SC[(size_t)j * a.ldp + j];
+    if (lane == 0) prev[2] = exact_double(a.SC[(size_t)j * a.ldp + j]);
     reset_chunks(cs, a.ldp);
     if constexpr (STD) {
         // b = 0: the gradient is row j of S^C, whose chunk maxima the
@@ -1522,6 +1558,7 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
 
     double sigma = 1.0;                                  // sigma^(0) = 1, b = 0
     double s_prev = 0.0, f_prev = 0.0;                   // last (sigma, F(sigma))
+    float g_prev = 0.f;                                  // (float)(F(sigma) - sigma) of it
     const unsigned long long sweeps0 = cnt.sweeps;
     int status = COL_OK;
     bool overflow = false;           // the column goes to the block solver
@@ -1558,19 +1595,26 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
         }
         if (!inner_ok) status |= COL_NOT_CONVERGED;
         double q = residual_quadratic_form_list<T>(j, s, a, sb, prev[2]);
-        const double floor2 = 1e-12 * prev[2];
-        if (q <= floor2) {
-            q = floor2;
-            status |= COL_DEGENERATE;
+        // q <= 1e-12 S_jj, decided on the upper words where they decide it
+        const double sjj = prev[2];
+        if (__double2hiint(q) <= __double2hiint(sjj) - (39 << 20)) {   // q < 2^-38 S_jj (or negative)
+            const double floor2 = 1e-12 * sjj;
+            if (q <= floor2) {
+                q = floor2;
+                status |= COL_DEGENERATE;
+            }
         }
         const double sn = sqrt_heron(q);
-        if (fabs(sn - sigma) < a.tol) {
+        const double dg = sn - sigma;
+        if (below(dg, a.tol)) {
             sigma = sn;
             break;
         }
         double nxt = sn;
+        const float g1 = (float)dg;
         if (r > 0 && r + 1 < a.maxit && !(status & COL_DEGENERATE))
-            nxt = HS ? sigma_step(prev[0], prev[1], sigma, sn) : sigma_step(s_prev, f_prev, sigma, sn);
+            nxt = sigma_step(HS ? prev[0] : s_prev, g_prev, sigma, sn, g1);
+        g_prev = g1;
         if constexpr (HS) {
             __syncwarp();
             if (lane == 0) {
@@ -2401,16 +2445,27 @@ __device__ __noinline__ bool block_quadratic_form_saa(int j, const T* __restrict
     const int inA = __syncthreads_count(tid < na && b[saa_list[tid]] != T(0));
     if (inA != nsupp) return false;
     const int v0 = lane, v1 = lane + 32;
-    const double bv0 = v0 < na ? (double)b[saa_list[v0]] : 0.0;
-    const double bv1 = v1 < na ? (double)b[saa_list[v1]] : 0.0;
+    const double bv0 = v0 < na ? exact_double(b[saa_list[v0]]) : 0.0;
+    const double bv1 = v1 < na ? exact_double(b[saa_list[v1]]) : 0.0;
     double acc = 0.0;
-    for (int k = warp; k < na; k += BLK_WARPS) {
-        const int ak = saa_list[k];
-        const double bk = (double)b[ak];
-        double t = v0 < na ? bv0 * (double)saa[k * BLK_AMAX + v0] : 0.0;
-        if (v1 < na) t = fma(bv1, (double)saa[k * BLK_AMAX + v1], t);
-        acc = fma(bk, t, acc);                              // b_k sum_m S_km b_m
-        if (lane == 0) acc = fma(-2.0 * bk, (double)a.SC[(size_t)ak * a.ldp + j], acc);
+    // -2 b_k S_kj of this warp's rows, loaded together
+    T skj[BLK_AMAX / BLK_WARPS];
+#pragma unroll
+    for (int i = 0; i < BLK_AMAX / BLK_WARPS; ++i) {
+        const int k = warp + i * BLK_WARPS;
+        skj[i] = (k < na && lane == 0) ? a.SC[(size_t)saa_list[k] * a.ldp + j] : T(0);
+    }
+#pragma unroll
+    for (int i = 0; i < BLK_AMAX / BLK_WARPS; ++i) {
+        const int k = warp + i * BLK_WARPS;
+        if (k < na) {
+            const T bt = b[saa_list[k]];
+            const double bk = exact_double(bt);
+            double t = v0 < na ? bv0 * exact_double(saa[k * BLK_AMAX + v0]) : 0.0;
+            if (v1 < na) t = fma(bv1, exact_double(saa[k * BLK_AMAX + v1]), t);
+            acc = fma(bk, t, acc);                          // b_k sum_m S_km b_m
+            if (lane == 0) acc = fma(exact_double(T(-2) * bt), exact_double(skj[i]), acc);
+        }
     }
     acc = block_sum_d(acc, sc);
     q = (double)a.SC[(size_t)j * a.ldp + j] + acc;
@@ -2574,7 +2629,7 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
         }
         double nxt = sn;
         if (r > 0 && r + 1 < a.maxit && !(status & COL_DEGENERATE))
-            nxt = sigma_step(s_prev, f_prev, sigma, sn);
+            nxt = sigma_step(s_prev, (float)(f_prev - s_prev), sigma, sn, (float)(sn - sigma));
         s_prev = sigma;
         f_prev = sn;
         sigma = nxt;

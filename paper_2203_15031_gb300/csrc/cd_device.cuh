@@ -1910,8 +1910,9 @@ struct BlockScratch {
     int vred[BLK_WARPS];         // scan: coordinates that would move, per warp
     float mred[BLK_WARPS];       // scan: their largest candidate |move|, per warp
     int wcnt[2], wmax[2];        // refresh scan: count and largest |move| (float bits), by parity
-    int saa_n;                   // size of the support S_AA was last gathered for (warp 0's copy)
-    int nlist;
+    double sig[2];               // the sigma step's F(sigma) and next sigma (warp 0's)
+    int sigf;                    // its flags: 1 degenerate, 2 converged
+    float bl1;                   // an upper bound of ||b_j||_1 after any phase so far
     int col;
 };
 
@@ -1945,7 +1946,7 @@ __device__ __forceinline__ double block_sum_d(double v, BlockScratch& sc) {
 // Each thread counts the nonzeros of its own contiguous segment of b, a block
 // scan gives the segment offsets, and each thread writes its entries.
 template <typename T>
-__device__ int block_support_list(const T* __restrict__ b, int p, int* __restrict__ list,
+__device__ __noinline__ int block_support_list(const T* __restrict__ b, int p, int* __restrict__ list,
                                   BlockScratch& sc, int& par) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int seg = (p + BLK_THREADS - 1) / BLK_THREADS;
@@ -1974,6 +1975,29 @@ __device__ int block_support_list(const T* __restrict__ b, int p, int* __restric
     return total;
 }
 
+// The nonzero coordinates of src[0, n) (sorted, n <= BLK_AMAX, holding the whole
+// support) into list (src itself may be list); returns their number.  A pass over b
+// for the support took 12 % of a hub's regression at p = 10000 (5500 cycles each).
+template <typename T>
+__device__ __forceinline__ int block_filter_list(const T* __restrict__ b, const int* src, int n, int* list,
+                                 BlockScratch& sc, int& par) {
+    const int lane = threadIdx.x;
+    if (lane < 32) {
+        const int k0 = lane < n ? src[lane] : 0, k1 = lane + 32 < n ? src[lane + 32] : 0;
+        const bool s0 = lane < n && b[k0] != T(0), s1 = lane + 32 < n && b[k1] != T(0);
+        const unsigned m0 = __ballot_sync(FULL_MASK, s0), m1 = __ballot_sync(FULL_MASK, s1);
+        const unsigned below = (1u << lane) - 1u;
+        const int c0 = __popc(m0);
+        if (s0) list[__popc(m0 & below)] = k0;
+        if (s1) list[c0 + __popc(m1 & below)] = k1;
+        if (lane == 0) sc.red[par][0] = c0 + __popc(m1);
+    }
+    __syncthreads();
+    const int m = sc.red[par][0];
+    par ^= 1;
+    return m;
+}
+
 // The scan that certifies a converged support.  A coordinate k != j outside
 // the support (b_k = 0) would move in a sweep with the support held exactly
 // when its candidate Soft(g_k, lambda) (divided by S_kk without
@@ -1998,7 +2022,7 @@ __device__ __forceinline__ bool scan_member(int k, int j, const T* __restrict__ 
 }
 
 template <typename T, bool STD>
-__device__ int block_scan_list(int j, const T* __restrict__ g, const T* __restrict__ b,
+__device__ __noinline__ int block_scan_list(int j, const T* __restrict__ g, const T* __restrict__ b,
                                const CDArgs<T>& a, T lam, int* __restrict__ list, BlockScratch& sc,
                                int& par, int& nv, float& mv) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -2079,16 +2103,44 @@ struct RefreshScan {
     int wp;
 };
 
-// g = S_.j - sum_{l in A} S_.l b_l over the whole row (block-wide), A = list[0, n).
-// A thread takes QG of its quads at once and reads R support rows for each, so
+// Bounds of the gradient by chunk (standardised matrix), kept from one
+// refresh with a scan to the next: ub[c] >= |g_k| for every k != j of chunk c
+// that was neither j nor in the support at the last one, `prev[0, nprev)` holds that support's
+// list, and a phase leaves the change of each of its coordinates in dl.  With
+// |S^C_lk| <= cmax[l][c], chunk c grows by at most sum_l dl_l cmax[l][c]; while
+// that stays below lambda (with the margins of chunk_skippable) no coordinate at
+// zero in it would move, so the refresh leaves the chunk out: the scan finds the same
+// coordinates.  A coordinate that has reached zero since opens its chunk.  What reads all of g
+// (block_sweep, block_scan_list) has it formed whole first.  Of 79 chunks the
+// refreshes of a hub's regression (p = 10000, 49 coefficients) form 78, 78, 11, 79, 2,
+// 1, 2 and 0; a whole one takes 50 kcycles, rows from L2 and DRAM.  With the
+// support's list kept, S_AA gathered by the block and the sigma step's FP64 in one
+// warp, that fit takes 926 us instead of 989, and 256 mixed fits 1897 instead of 1935.
+struct ChunkBounds {
+    float* ub;
+    int* prev;
+    float* dl;
+    int nprev;
+    bool valid;
+};
+constexpr int BLK_MAX_CHUNKS = 1024;       // chunks the bounds have room for
+
+// g = S_.j - sum_{l in A} S_.l b_l (block-wide), A = list[0, n): over the whole row,
+// or over the chunks that `cb` cannot leave out.  Warp w takes chunks w, w + 16, ...,
+// QG at once, and reads R support rows for each, so
 // QG * R independent loads are in flight; the products are accumulated in
-// the order of the list.  With `scan` the refresh also scans (RefreshScan).
+// the order of the list.  With `scan` the refresh also scans (RefreshScan), and
+// with cb it leaves the bounds of the chunks that it forms; plist[0, np) are the
+// coordinates of the phase before it.
 template <typename T, bool STD>
-__device__ void block_form_gradient(int j, T* __restrict__ g, const T* __restrict__ b,
+__device__ __noinline__ void block_form_gradient(int j, T* __restrict__ g, const T* __restrict__ b,
                                     const int* __restrict__ list, int n, const CDArgs<T>& a,
-                                    bool scan, T lam, BlockScratch& sc, RefreshScan ws) {
+                                    bool scan, T lam, BlockScratch& sc, RefreshScan ws,
+                                    const ChunkBounds* cb, const int* __restrict__ plist, int np) {
+    static_assert(CHUNK == 128, "a warp's quads are one chunk");
     constexpr int QG = sizeof(T) == 4 ? 2 : 1, R = 4;
-    const int ldp = a.ldp;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ldp = a.ldp, nch = num_chunks(ldp);
     const T* __restrict__ Sj = a.SC + (size_t)j * ldp;
     if (scan) {
         if (threadIdx.x == 0) {
@@ -2096,75 +2148,123 @@ __device__ void block_form_gradient(int j, T* __restrict__ g, const T* __restric
             sc.wmax[ws.wp ^ 1] = 0;
         }
     }
-    for (int q0 = threadIdx.x; 4 * q0 < ldp; q0 += QG * BLK_THREADS) {
-        T acc[QG][4];
+    for (int base = warp; base < nch; base += 32 * BLK_WARPS) {
+        // the warp's chunks base + 16 i to be formed, i < 32
+        const int cnt = min(32, (nch - base + BLK_WARPS - 1) / BLK_WARPS);
+        unsigned open = cnt == 32 ? FULL_MASK : (1u << cnt) - 1u;
+        if (STD && cb && cb->valid) {
+            const float d0 = lane < np ? cb->dl[lane] : 0.f, d1 = lane + 32 < np ? cb->dl[lane + 32] : 0.f;
+            const float* r0 = a.chunk_max + (size_t)(lane < np ? plist[lane] : j) * nch + base;
+            const float* r1 = a.chunk_max + (size_t)(lane + 32 < np ? plist[lane + 32] : j) * nch + base;
+            const float top = (float)lam - (2.0f + 2.0f * sc.bl1) * 0x1p-14f;
+            unsigned keep = 0u;
+            for (int i0 = 0; i0 < cnt; i0 += 4) {
+                float x[4];
 #pragma unroll
-        for (int u = 0; u < QG; ++u) {
-            const int k0 = 4 * (q0 + u * BLK_THREADS);
-            if (k0 < ldp) load4g<T>(Sj + k0, acc[u]);
+                for (int i = 0; i < 4; ++i)
+                    x[i] = i0 + i < cnt ? d0 * r0[(i0 + i) * BLK_WARPS] + d1 * r1[(i0 + i) * BLK_WARPS]
+                                        : 0.f;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (i0 + i >= cnt) break;
+                    const int c = base + (i0 + i) * BLK_WARPS;
+                    const float u = (cb->ub[c] + warp_l1_bound(x[i]) * (1.0f + 0x1p-10f)) * (1.0f + 0x1p-20f);
+                    __syncwarp();
+                    if (u < top) {
+                        if (lane == 0) cb->ub[c] = u;
+                        keep |= 1u << (i0 + i);
+                    }
+                }
+            }
+            // chunks of coordinates that have reached zero
+            unsigned left = 0u;
+            for (int e = lane; e < cb->nprev; e += 32) {
+                const int k = cb->prev[e], i = k / CHUNK - base;
+                if (b[k] == T(0) && i >= 0 && i % BLK_WARPS == 0 && i / BLK_WARPS < cnt)
+                    left |= 1u << (i / BLK_WARPS);
+            }
+            keep &= ~__reduce_or_sync(FULL_MASK, left);
+            open &= ~keep;
         }
-        int e = 0;
-        for (; e + R <= n; e += R) {
-            T r[R][QG][4];
+        while (open) {
+            int k0[QG];
 #pragma unroll
-            for (int v = 0; v < R; ++v) {
-                const T* __restrict__ row = a.SC + (size_t)list[e + v] * ldp;
+            for (int u = 0; u < QG; ++u) {
+                k0[u] = ldp;                                   // no chunk: nothing is read
+                if (open) {
+                    k0[u] = (base + (__ffs(open) - 1) * BLK_WARPS) * CHUNK + 4 * lane;
+                    open &= open - 1u;
+                }
+            }
+            T acc[QG][4];
+#pragma unroll
+            for (int u = 0; u < QG; ++u)
+                if (k0[u] < ldp) load4g<T>(Sj + k0[u], acc[u]);
+            int e = 0;
+            for (; e + R <= n; e += R) {
+                T r[R][QG][4];
+#pragma unroll
+                for (int v = 0; v < R; ++v) {
+                    const T* __restrict__ row = a.SC + (size_t)list[e + v] * ldp;
+#pragma unroll
+                    for (int u = 0; u < QG; ++u)
+                        if (k0[u] < ldp) load4g<T>(row + k0[u], r[v][u]);
+                }
+#pragma unroll
+                for (int v = 0; v < R; ++v) {
+                    const T bv = b[list[e + v]];
+#pragma unroll
+                    for (int u = 0; u < QG; ++u)
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) acc[u][t] = fma(-bv, r[v][u][t], acc[u][t]);
+                }
+            }
+            for (; e < n; ++e) {
+                const T* __restrict__ row = a.SC + (size_t)list[e] * ldp;
+                const T bv = b[list[e]];
 #pragma unroll
                 for (int u = 0; u < QG; ++u) {
-                    const int k0 = 4 * (q0 + u * BLK_THREADS);
-                    if (k0 < ldp) load4g<T>(row + k0, r[v][u]);
+                    if (k0[u] < ldp) {
+                        T r[4];
+                        load4g<T>(row + k0[u], r);
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) acc[u][t] = fma(-bv, r[t], acc[u][t]);
+                    }
                 }
             }
 #pragma unroll
-            for (int v = 0; v < R; ++v) {
-                const T bv = b[list[e + v]];
-#pragma unroll
-                for (int u = 0; u < QG; ++u)
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) acc[u][t] = fma(-bv, r[v][u][t], acc[u][t]);
-            }
-        }
-        for (; e < n; ++e) {
-            const T* __restrict__ row = a.SC + (size_t)list[e] * ldp;
-            const T bv = b[list[e]];
-#pragma unroll
             for (int u = 0; u < QG; ++u) {
-                const int k0 = 4 * (q0 + u * BLK_THREADS);
-                if (k0 < ldp) {
-                    T r[4];
-                    load4g<T>(row + k0, r);
+                if (k0[u] < ldp)
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) acc[u][t] = fma(-bv, r[t], acc[u][t]);
-                }
+                    for (int t = 0; t < 4; ++t) g[k0[u] + t] = acc[u][t];
             }
-        }
+            if (scan) {
 #pragma unroll
-        for (int u = 0; u < QG; ++u) {
-            const int k0 = 4 * (q0 + u * BLK_THREADS);
-            if (k0 < ldp)
+                for (int u = 0; u < QG; ++u) {
+                    float top = 0.f;
+                    if (k0[u] < a.p) {
+                        T bq[4];
+                        load4<T>(b + k0[u], bq);
 #pragma unroll
-                for (int t = 0; t < 4; ++t) g[k0 + t] = acc[u][t];
-        }
-        if (scan) {
-#pragma unroll
-            for (int u = 0; u < QG; ++u) {
-                const int k0 = 4 * (q0 + u * BLK_THREADS);
-                if (k0 < a.p) {
-                    T bq[4];
-                    load4<T>(b + k0, bq);
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        const int k = k0 + t;
-                        if (k < a.p && k != j && bq[t] == T(0)) {
-                            T nb;
-                            if constexpr (STD) nb = soft<T>(acc[u][t] + bq[t], lam);     // S_kk = 1
-                            else nb = soft<T>(acc[u][t] + a.diag[k] * bq[t], lam) / a.diag[k];
-                            if (nb != T(0) && !list_contains(list, n, k)) {
-                                const int slot = atomicAdd(&sc.wcnt[ws.wp], 1);
-                                if (slot < ws.vcap) ws.vlist[slot] = k;
-                                atomicMax(&sc.wmax[ws.wp], __float_as_int(fabsf((float)nb)));
+                        for (int t = 0; t < 4; ++t) {
+                            const int k = k0[u] + t;
+                            if (k < a.p && k != j && bq[t] == T(0)) {
+                                T nb;
+                                if constexpr (STD) nb = soft<T>(acc[u][t] + bq[t], lam);     // S_kk = 1
+                                else nb = soft<T>(acc[u][t] + a.diag[k] * bq[t], lam) / a.diag[k];
+                                if (STD) top = fmaxf(top, fabsf((float)acc[u][t]));
+                                if (nb != T(0) && !list_contains(list, n, k)) {
+                                    const int slot = atomicAdd(&sc.wcnt[ws.wp], 1);
+                                    if (slot < ws.vcap) ws.vlist[slot] = k;
+                                    atomicMax(&sc.wmax[ws.wp], __float_as_int(fabsf((float)nb)));
+                                }
                             }
                         }
+                    }
+                    if (STD && cb) {
+                        // lane 0 holds the chunk's first coordinate, below ldp when there is a chunk
+                        const unsigned m = __reduce_max_sync(FULL_MASK, __float_as_uint(top));
+                        if (lane == 0 && k0[u] < ldp) cb->ub[k0[u] / CHUNK] = __uint_as_float(m);
                     }
                 }
             }
@@ -2204,6 +2304,39 @@ __device__ inline void warp_union(const int* __restrict__ list, int n, const int
     __syncwarp();
 }
 
+// S_AA of A = list[0, n), n <= BLK_AMAX, by the whole block: warp w gathers rows
+// w, w + 16, ... with all of its loads in flight (one warp alone took 67 of a
+// hub's 800 kcycles at p = 10000); zero outside the n x n block so the idle slots
+// stay finite.  Kept from the last phase when the support is the same
+// (saa_list, saa_n; the same in every thread).
+template <typename T>
+__device__ __forceinline__ void block_gather_saa(const int* __restrict__ list, int n, const CDArgs<T>& a,
+                                                 T* __restrict__ saa, int* __restrict__ saa_list,
+                                                 int& saa_n) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (__syncthreads_and(saa_n == n && (tid >= n || saa_list[tid] == list[tid]))) return;
+    constexpr int NR = BLK_AMAX / BLK_WARPS;
+    const int m0 = lane, m1 = lane + 32;
+    const int l0 = m0 < n ? list[m0] : 0, l1 = m1 < n ? list[m1] : 0;
+    T v0[NR], v1[NR];
+#pragma unroll
+    for (int u = 0; u < NR; ++u) {
+        const int k = warp + u * BLK_WARPS;
+        const T* __restrict__ row = a.SC + (size_t)(k < n ? list[k] : 0) * a.ldp;
+        v0[u] = (k < n && m0 < n) ? row[l0] : T(0);
+        v1[u] = (k < n && m1 < n) ? row[l1] : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < NR; ++u) {
+        const int k = warp + u * BLK_WARPS;
+        saa[k * BLK_AMAX + m0] = v0[u];
+        saa[k * BLK_AMAX + m1] = v1[u];
+    }
+    if (tid < n) saa_list[tid] = list[tid];
+    saa_n = n;
+    __syncthreads();
+}
+
 // Active-set phase of the block solver, run by warp 0 on A = list[0, n),
 // n <= BLK_AMAX: lane m holds coordinates A_m and A_{m+32}.  Reads and writes
 // b for the coordinates of A; g is formed afresh by the caller afterwards.
@@ -2215,43 +2348,17 @@ __device__ inline void warp_union(const int* __restrict__ list, int n, const int
 // on it.
 template <typename T, bool STD>
 __device__ int block_active_phase(int j, T* __restrict__ b, const int* __restrict__ list, int n,
-                                  const CDArgs<T>& a, T lam, T* __restrict__ saa,
-                                  int* __restrict__ saa_list, float2* __restrict__ tb, int& saa_n,
+                                  const CDArgs<T>& a, T lam, const T* __restrict__ saa,
+                                  float2* __restrict__ tb, float* __restrict__ dl, BlockScratch& sc,
                                   unsigned long long& moves, bool& conv) {
     const int lane = threadIdx.x & 31;
     const int ldp = a.ldp;
     const int m0 = lane, m1 = lane + 32;
-    // S_AA, zero outside the n x n block so the idle slots stay finite; kept
-    // from the last phase when the support is the same (saa_list, saa_n)
-    const bool same = saa_n == n &&
-                      __all_sync(FULL_MASK, (m0 >= n || saa_list[m0] == list[m0]) &&
-                                                (m1 >= n || saa_list[m1] == list[m1]));
-    if (!same) {
-        const int l0 = m0 < n ? list[m0] : 0, l1 = m1 < n ? list[m1] : 0;
-        for (int k0 = 0; k0 < BLK_AMAX; k0 += 8) {
-            T v0[8], v1[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int k = k0 + u;
-                const T* __restrict__ row = a.SC + (size_t)(k < n ? list[k] : 0) * ldp;
-                v0[u] = (k < n && m0 < n) ? row[l0] : T(0);
-                v1[u] = (k < n && m1 < n) ? row[l1] : T(0);
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                saa[(k0 + u) * BLK_AMAX + m0] = v0[u];
-                saa[(k0 + u) * BLK_AMAX + m1] = v1[u];
-            }
-        }
-        if (m0 < n) saa_list[m0] = list[m0];
-        if (m1 < n) saa_list[m1] = list[m1];
-        saa_n = n;
-        __syncwarp();
-    }
     const bool h0 = m0 < n, h1 = m1 < n;
     T b0 = h0 ? b[list[m0]] : T(0), b1 = h1 ? b[list[m1]] : T(0);
     T g0 = h0 ? a.SC[(size_t)j * ldp + list[m0]] : T(0);
     T g1 = h1 ? a.SC[(size_t)j * ldp + list[m1]] : T(0);
+    const T b0_start = b0, b1_start = b1;
     T s0 = T(1), s1 = T(1);
     if constexpr (!STD) {
         if (h0) s0 = a.diag[list[m0]];
@@ -2308,6 +2415,10 @@ __device__ int block_active_phase(int j, T* __restrict__ b, const int* __restric
     moves += mv;
     if (h0) b[list[m0]] = b0;
     if (h1) b[list[m1]] = b1;
+    dl[m0] = fabsf((float)(b0 - b0_start));                 // ChunkBounds
+    dl[m1] = fabsf((float)(b1 - b1_start));
+    const float l1 = warp_l1_bound((float)b0) + warp_l1_bound((float)b1);
+    if (lane == 0) sc.bl1 = fmaxf(sc.bl1, l1);
     return sw;
 }
 
@@ -2315,7 +2426,7 @@ __device__ int block_active_phase(int j, T* __restrict__ b, const int* __restric
 // coordinates of the support keep their values).  Returns max |delta b|.
 // cand holds the candidate moves (new b, delta) of every thread, two buffers.
 template <typename T, bool STD>
-__device__ T block_sweep(int j, T* __restrict__ g, T* __restrict__ b, const CDArgs<T>& a, T lam,
+__device__ __noinline__ T block_sweep(int j, T* __restrict__ g, T* __restrict__ b, const CDArgs<T>& a, T lam,
                          bool frozen, T* __restrict__ cand, unsigned long long& moves,
                          BlockScratch& sc, int& par, int sweep_idx) {
     const int tid = threadIdx.x;
@@ -2431,9 +2542,13 @@ __device__ __noinline__ double block_quadratic_form(int j, const T* __restrict__
 // S_AA in shared memory, when the support lies in the list A it was
 // gathered for (A = saa_list[0, na), sorted; saa[k BLK_AMAX + m] = S_{A_k A_m}):
 // b is zero on A outside the support, and the zero terms add nothing.
-// Returns false (nothing computed) when some support coordinate is not in A.
-// The products are formed in FP64, warp w taking the rows k = w, w + 16, ...
-// of S_AA and each lane two of its entries; one fixed-order block sum.
+// Returns false (nothing computed) when some support coordinate is not in A;
+// q is valid in warp 0.  The FP64 pipe (16 cycles a warp's instruction) bounds this, so
+// the products are formed by BLK_QWARPS warps, warp w taking the rows k = w,
+// w + 4, ... of S_AA and each lane two of its entries, only these warps' sums are
+// formed, and one warp adds them up: with all 16 warps in each of these steps
+// a sigma step took 12 of a hub's 850 kcycles (p = 10000, six steps).
+constexpr int BLK_QWARPS = 4;
 template <typename T>
 __device__ __noinline__ bool block_quadratic_form_saa(int j, const T* __restrict__ b, int nsupp,
                                          const int* __restrict__ saa_list, int na,
@@ -2442,33 +2557,45 @@ __device__ __noinline__ bool block_quadratic_form_saa(int j, const T* __restrict
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int tid = threadIdx.x;
     if (na <= 0 || na > BLK_AMAX || nsupp > na) return false;
+    const int v0 = lane, v1 = lane + 32;
+    // S_kj and S_jj (warp 0), on their way during the products
+    T s0 = T(0), s1 = T(0), sjj = T(0);
+    if (warp == 0) {
+        if (v0 < na) s0 = a.SC[(size_t)saa_list[v0] * a.ldp + j];
+        if (v1 < na) s1 = a.SC[(size_t)saa_list[v1] * a.ldp + j];
+        sjj = a.SC[(size_t)j * a.ldp + j];
+    }
     const int inA = __syncthreads_count(tid < na && b[saa_list[tid]] != T(0));
     if (inA != nsupp) return false;
-    const int v0 = lane, v1 = lane + 32;
-    const double bv0 = v0 < na ? exact_double(b[saa_list[v0]]) : 0.0;
-    const double bv1 = v1 < na ? exact_double(b[saa_list[v1]]) : 0.0;
-    double acc = 0.0;
-    // -2 b_k S_kj of this warp's rows, loaded together
-    T skj[BLK_AMAX / BLK_WARPS];
-#pragma unroll
-    for (int i = 0; i < BLK_AMAX / BLK_WARPS; ++i) {
-        const int k = warp + i * BLK_WARPS;
-        skj[i] = (k < na && lane == 0) ? a.SC[(size_t)saa_list[k] * a.ldp + j] : T(0);
-    }
-#pragma unroll
-    for (int i = 0; i < BLK_AMAX / BLK_WARPS; ++i) {
-        const int k = warp + i * BLK_WARPS;
-        if (k < na) {
-            const T bt = b[saa_list[k]];
-            const double bk = exact_double(bt);
-            double t = v0 < na ? bv0 * exact_double(saa[k * BLK_AMAX + v0]) : 0.0;
-            if (v1 < na) t = fma(bv1, exact_double(saa[k * BLK_AMAX + v1]), t);
-            acc = fma(bk, t, acc);                          // b_k sum_m S_km b_m
-            if (lane == 0) acc = fma(exact_double(T(-2) * bt), exact_double(skj[i]), acc);
+    if (warp < BLK_QWARPS) {
+        const T b0 = v0 < na ? b[saa_list[v0]] : T(0), b1 = v1 < na ? b[saa_list[v1]] : T(0);
+        const double bv0 = exact_double(b0), bv1 = exact_double(b1);
+        double acc = 0.0;
+        if (na <= 32) {
+#pragma unroll 4
+            for (int k = warp; k < na; k += BLK_QWARPS)     // b_k sum_m S_km b_m
+                acc = fma(exact_double(b[saa_list[k]]), bv0 * exact_double(saa[k * BLK_AMAX + v0]), acc);
+        } else {
+#pragma unroll 4
+            for (int k = warp; k < na; k += BLK_QWARPS)
+                acc = fma(exact_double(b[saa_list[k]]),
+                          fma(bv1, exact_double(saa[k * BLK_AMAX + v1]),
+                              bv0 * exact_double(saa[k * BLK_AMAX + v0])), acc);
         }
+        if (warp == 0) {                                    // -2 b_k S_kj
+            acc = fma(exact_double(T(-2) * b0), exact_double(s0), acc);
+            if (na > 32) acc = fma(exact_double(T(-2) * b1), exact_double(s1), acc);
+        }
+        acc = warp_sum(acc);
+        if (lane == 0) sc.dred[warp] = acc;
     }
-    acc = block_sum_d(acc, sc);
-    q = (double)a.SC[(size_t)j * a.ldp + j] + acc;
+    __syncthreads();
+    if (warp == 0) {
+        double t = exact_double(sjj);
+#pragma unroll
+        for (int w = 0; w < BLK_QWARPS; ++w) t += sc.dred[w];
+        q = t;
+    }
     return true;
 }
 
@@ -2492,7 +2619,19 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
     int* vlist = ubuf + BLK_AMAX;
     // the phase's links and coefficients too (2 KB of the buffers' 8 KB at most)
     float2* tb = reinterpret_cast<float2*>(vlist + BLK_AMAX);
-    int saa_n = -1;                                       // warp 0: no S_AA gathered yet
+    // and, between sweeps, the bounds of the gradient's chunks (5 KB)
+    ChunkBounds cb;
+    cb.prev = reinterpret_cast<int*>(tb) + 2048 / sizeof(int);
+    cb.dl = reinterpret_cast<float*>(cb.prev + BLK_AMAX);
+    cb.ub = cb.dl + BLK_AMAX;
+    static_assert(4 * BLK_AMAX * sizeof(int) + 2048 + BLK_MAX_CHUNKS * sizeof(float) <=
+                  2 * 2 * BLK_THREADS * sizeof(float), "the bounds share the candidate buffers");
+    cb.nprev = 0;
+    cb.valid = false;
+    const int nch = num_chunks(ldp);
+    const bool bounds = STD && a.chunk_max && nch <= BLK_MAX_CHUNKS;
+    bool gfull = true;                                    // every chunk of g is up to date
+    int saa_n = -1;                                       // no S_AA gathered yet
     int par = 0;
     int wp = 0;                                           // parity of the refresh scan's counters
     // a column the lazy solver handed over continues from its iterate
@@ -2508,7 +2647,11 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
         if (tid == 0) {
             sc.wcnt[0] = sc.wcnt[1] = 0;
             sc.wmax[0] = sc.wmax[1] = 0;
-            sc.saa_n = -1;
+            sc.bl1 = 0.f;
+        }
+        if (bounds && !warm) {                            // b = 0: the row's chunk maxima
+            for (int c = tid; c < nch; c += BLK_THREADS) cb.ub[c] = a.chunk_max[(size_t)j * nch + c];
+            cb.valid = true;
         }
     }
     __syncthreads();
@@ -2517,6 +2660,23 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
     int status = COL_OK;
     int r0 = 0;
     bool stale = false;                                   // g is not yet S_.j - S b
+    // list[0, nl) (or its first BLK_LIST) holds the support, and nothing else if `exact`;
+    // nl = -1 when that is not known
+    int nl = warm ? -1 : 0;
+    bool exact = true;
+    auto support = [&]() {
+        if (nl < 0) nl = block_support_list<T>(b, a.p, list, sc, par);
+        else if (!exact) nl = block_filter_list<T>(b, list, nl, list, sc, par);
+        exact = true;
+        return nl;
+    };
+    // the chunks that refreshes have left out (the support is then one of a phase)
+    auto form_all = [&]() {
+        block_form_gradient<T, STD>(j, g, b, list, nl, a, false, T(0), sc, RefreshScan{vlist, 0, wp},
+                                    nullptr, list, 0);
+        __syncthreads();
+        gfull = true;
+    };
     if (warm) {
         sigma = a.sigma[j];
         s_prev = a.hand[2 * (size_t)j];
@@ -2538,25 +2698,27 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
             // converge on the support first (when it fits the phase), then a
             // sweep with the support held decides; otherwise a full sweep
             // decides (Algorithm 1's stop), as in the lazy solver
-            int n = uni ? nu : block_support_list<T>(b, a.p, list, sc, par);
+            int n = uni ? nu : support();
             const int* plist = uni ? ubuf : list;
+            const int np = n;
             bool conv = n == 0;
             const bool phase = n > 0 && n <= BLK_AMAX;
             if (phase) {
                 int sw = 0;
                 bool c = false;
-                if (tid < 32) sw = block_active_phase<T, STD>(j, b, plist, n, a, lam, saa, saa_list,
-                                                              tb, saa_n, cnt.act_moves, c);
+                block_gather_saa<T>(plist, n, a, saa, saa_list, saa_n);
+                if (tid < 32) sw = block_active_phase<T, STD>(j, b, plist, n, a, lam, saa, tb, cb.dl, sc,
+                                                              cnt.act_moves, c);
                 if (tid == 0) {
                     sc.red[par][0] = sw;
                     sc.red[par][1] = c ? 1 : 0;
-                    sc.saa_n = saa_n;
                 }
                 __syncthreads();
                 sw = sc.red[par][0];
                 conv = sc.red[par][1] != 0;
                 par ^= 1;
                 cnt.act_sweeps += sw;
+                exact = false;                            // coordinates may have reached zero
             }
             // Working set: with the support converged, one scan of every
             // coordinate finds those that a sweep with the support held
@@ -2573,11 +2735,25 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
             float mv = 0.f;
             // a handed-over support (at most LAZY_CAP entries) fits the list
             if (phase || stale) {
-                if (uni) n = block_support_list<T>(b, a.p, list, sc, par);   // the support
+                if (uni) {                                // the support of the union
+                    n = nl = block_filter_list<T>(b, ubuf, np, list, sc, par);
+                    exact = true;
+                }
                 scanned = ws && n <= BLK_AMAX;
+                const bool keep = scanned && bounds;      // what the scan leaves bounds for
+                if (!scanned) cb.valid = false;
+                gfull = !cb.valid;
                 block_form_gradient<T, STD>(j, g, b, list, n, a, scanned, lam, sc,
-                                            RefreshScan{vlist, BLK_AMAX, wp});
+                                            RefreshScan{vlist, BLK_AMAX, wp}, keep ? &cb : nullptr,
+                                            plist, phase ? np : 0);
                 __syncthreads();
+                if (keep) {
+                    // by warp 0, which is also the one that changes the list
+                    if (tid < 32)
+                        for (int e = tid; e < n; e += 32) cb.prev[e] = list[e];
+                    cb.nprev = n;
+                    cb.valid = true;
+                }
                 if (scanned) {
                     nv = sc.wcnt[wp];
                     mv = __int_as_float(sc.wmax[wp]);
@@ -2588,6 +2764,7 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
             uni = false;
             if (ws && n <= BLK_AMAX) {
                 if (!scanned) {
+                    if (!gfull) form_all();
                     // no refresh (b = 0, g = S_.j): a scan of its own, the union into ubuf
                     nu = block_scan_list<T, STD>(j, g, b, a, lam, ubuf, sc, par, nv, mv);
                 }
@@ -2605,8 +2782,11 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
                     continue;
                 }
             }
+            if (!gfull) form_all();
             const T md = block_sweep<T, STD>(j, g, b, a, lam, conv, cand, cnt.moves, sc, par,
                                              (int)(cnt.sweeps - sweeps0));
+            nl = -1;
+            cb.valid = false;                             // the candidates have overwritten them
             ++cnt.sweeps;
             if ((double)md < a.tol) {
                 inner_ok = true;
@@ -2614,22 +2794,34 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
             }
         }
         if (!inner_ok) status |= COL_NOT_CONVERGED;
-        const int n = block_support_list<T>(b, a.p, list, sc, par);
+        const int n = support();
         double q;
-        if (!block_quadratic_form_saa<T>(j, b, n, saa_list, sc.saa_n, saa, a, sc, q))
+        if (!block_quadratic_form_saa<T>(j, b, n, saa_list, saa_n, saa, a, sc, q))
             q = block_quadratic_form<T>(j, b, list, n, a, sc);
-        if (q <= floor2) {
-            q = floor2;
-            status |= COL_DEGENERATE;
+        if (tid < 32) {                                   // one warp on the FP64 pipe
+            int f = (status & COL_DEGENERATE) ? 1 : 0;
+            if (q <= floor2) {
+                q = floor2;
+                f = 1;
+            }
+            const double sn = sqrt_heron(q);
+            double nxt = sn;
+            if (fabs(sn - sigma) < a.tol) f |= 2;
+            else if (r > 0 && r + 1 < a.maxit && !f)
+                nxt = sigma_step(s_prev, (float)(f_prev - s_prev), sigma, sn, (float)(sn - sigma));
+            if (tid == 0) {
+                sc.sig[0] = sn;
+                sc.sig[1] = nxt;
+                sc.sigf = f;
+            }
         }
-        const double sn = sqrt_heron(q);
-        if (fabs(sn - sigma) < a.tol) {
+        __syncthreads();
+        const double sn = sc.sig[0], nxt = sc.sig[1];
+        if (sc.sigf & 1) status |= COL_DEGENERATE;
+        if (sc.sigf & 2) {
             sigma = sn;
             break;
         }
-        double nxt = sn;
-        if (r > 0 && r + 1 < a.maxit && !(status & COL_DEGENERATE))
-            nxt = sigma_step(s_prev, (float)(f_prev - s_prev), sigma, sn, (float)(sn - sigma));
         s_prev = sigma;
         f_prev = sn;
         sigma = nxt;
@@ -2640,7 +2832,7 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
     }
     // b_j into row j of BT (a list where it fits, see coef_cap), row j of Theta cleared
     T* brow = a.BT + (size_t)j * ldp;
-    const int nb = block_support_list<T>(b, a.p, list, sc, par);
+    const int nb = support();
     if (nb <= coef_cap(ldp)) {
         int* idx = coef_idx(brow, ldp);
         for (int t = tid; t < nb; t += BLK_THREADS) {

@@ -66,10 +66,10 @@ BATCH_PREC = "mixed"
 TOL, MAXIT = 1e-6, 1000
 # kernels of one batched mixed step: split/transpose, tcgen05 Gram, prep_diag,
 # prep_matrix, the column order (heat histogram, offsets, scatter), lazy
-# solver, block solver over the handed-over columns, Theta.  (A batch with a
+# solver, block solver over the handed-over columns, 1/sigma^2, Theta.  (A batch with a
 # fit of 4096 or more columns adds the block solver over the heavy columns on
 # a side stream; no fit of this workload is that large.)
-KERNELS_PER_STEP = 10
+KERNELS_PER_STEP = 11
 # fits of the batch the oracle solves (accuracy, CPU baseline, reference arm)
 ORACLE_SAMPLE = list(range(N_FITS))
 REFERENCE_SAMPLE = list(range(0, N_FITS, 32))
@@ -925,11 +925,11 @@ def run_single(args):
             "latency": {"p50_ms": statistics.median(per),
                         "p99_ms": srt[min(len(srt) - 1, int(math.ceil(0.99 * len(srt))) - 1)]},
             "roofline": roof, "roofline_gram": roof_gram,
-            # Gram (split + tcgen05, or SIMT); prep_diag, prep_matrix, [column
+            # Gram (split or digits + tcgen05, or SIMT); prep_diag, prep_matrix, [column
             # order: more columns than resident warps, or heavy routing],
             # [block solver on the heavy columns: p >= 4096], lazy, block solver
             # on the handed-over columns, row count, Theta
-            "gpu_launches": ((2 if prec == sp.MIXED else 1) + 6 + (1 if p >= 4096 else 0)
+            "gpu_launches": ((1 if prec == sp.FP32 else 2) + 6 + (1 if p >= 4096 else 0)
                              + (1 if p >= 3648 else 0)) * args.steps,
             "clocks": clk.summary()}
     print(json.dumps(line), flush=True)
@@ -1035,8 +1035,8 @@ def run_residual(args):
                          "note": "each formed 128-coordinate gradient slice reads n rows of W "
                                  "(512 B each) through L2 in one warp's dependent chain; the "
                                  "covariance form reads 1 + |support| rows of S per slice"},
-            # the head value's timed steps: stats, build, coordinate descent,
-            # Theta zeroing and Theta per residual fit
+            # the head value's timed steps: stats, build, chunk maxima, coordinate
+            # descent and Theta per residual fit
             "gpu_launches": 5 * args.steps, "clocks": clk.summary()}
     print(json.dumps(line), flush=True)
 

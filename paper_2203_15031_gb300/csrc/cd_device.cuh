@@ -252,13 +252,12 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // (double)x without the FP64 pipe, where a conversion takes as long as an
 // addition: the exponent rebased and the fraction moved, by integer
-// instructions.  Exact for zero and normal x; a denormal FP32 value (below
-// 2^-126, 26 decades under any sigma^2 it could enter) gives zero.
+// instructions.  Denormal FP32 values, infinities and NaN take the conversion.
 __device__ __forceinline__ double exact_double(float x) {
-    const unsigned u = __float_as_uint(x);
-    const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
-    const bool normal = (u & 0x7f800000u) != 0u;
-    return __hiloint2double(normal ? (int)hi : 0, normal ? (int)(u << 29) : 0);
+    const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)x;
+    const unsigned hi = (u & 0x80000000u) | (m != 0u ? (m >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
 }
 __device__ __forceinline__ double exact_double(double x) { return x; }
 
@@ -1610,7 +1609,8 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
         double q = residual_quadratic_form_list<T>(j, s, a, sb, prev[2]);
         // q <= 1e-12 S_jj, decided on the upper words where they decide it
         const double sjj = prev[2];
-        if (__double2hiint(q) <= __double2hiint(sjj) - (39 << 20)) {   // q < 2^-38 S_jj (or negative)
+        // (q < 2^-38 S_jj, negative, or denormal)
+        if (__double2hiint(q) <= max(__double2hiint(sjj) - (39 << 20), 1 << 20)) {
             const double floor2 = 1e-12 * sjj;
             if (q <= floor2) {
                 q = floor2;

@@ -8,19 +8,21 @@ import numpy as np
 
 def exact_double(x):
     u = x.view(np.uint32)
-    hi = (u & np.uint32(0x80000000)) | (((u & np.uint32(0x7fffffff)) >> np.uint32(3)) + np.uint32(0x38000000))
-    lo = (u << np.uint32(29)).astype(np.uint64)
-    bits = (hi.astype(np.uint64) << np.uint64(32)) | lo
-    return np.where((u & np.uint32(0x7f800000)) != 0, bits, np.uint64(0)).view(np.float64)
+    m = u & np.uint32(0x7fffffff)
+    direct = (m - np.uint32(0x00800000) >= np.uint32(0x7f000000)) & (m != 0)
+    hi = (u & np.uint32(0x80000000)) | np.where(m != 0, (m >> np.uint32(3)) + np.uint32(0x38000000), np.uint32(0))
+    bits = (hi.astype(np.uint64) << np.uint64(32)) | (u << np.uint32(29)).astype(np.uint64)
+    return np.where(direct, x.astype(np.float64), bits.view(np.float64))
 
 
-def test_exact_double_of_normal_floats_and_zero():
+def test_exact_double_of_every_kind_of_float():
     rng = np.random.default_rng(0)
     u = rng.integers(0, 1 << 32, 1 << 20, dtype=np.uint64).astype(np.uint32)
-    e = (u >> 23) & 0xff
-    x = np.concatenate([u[(e > 0) & (e < 255)].view(np.float32),
-                        np.array([0.0, -0.0, 1.0, -1.0, 2.0 ** -126, 3.4028234e38], np.float32)])
-    assert np.array_equal(exact_double(x), x.astype(np.float64))
+    x = np.concatenate([u.view(np.float32),
+                        np.array([0.0, -0.0, 1.0, -1.0, 2.0 ** -126, 2.0 ** -149, -(2.0 ** -127), np.inf,
+                                  -np.inf, np.nan, 3.4028234e38], np.float32)])
+    with np.errstate(invalid="ignore"):
+        assert np.array_equal(exact_double(x), x.astype(np.float64), equal_nan=True)
 
 
 def test_below_and_sign_on_the_bits():
@@ -41,6 +43,8 @@ def test_the_floor_screen_keeps_every_floored_value():
     q = 1e-12 * sjj * f
     q[::7] *= -1.0
     hi = lambda v: (v.view(np.int64) >> 32).astype(np.int32)  # noqa: E731
-    assert (hi(q) <= hi(sjj) - (39 << 20)).all()
+    assert (hi(q) <= np.maximum(hi(sjj) - (39 << 20), 1 << 20)).all()
+    tiny = np.exp2(-rng.uniform(900, 1020, 20000))       # S_jj of raw FP64 data
+    assert (hi(1e-12 * tiny) <= np.maximum(hi(tiny) - (39 << 20), 1 << 20)).all()
     # and values well above the floor do not reach the exact test
     assert not (hi(sjj * 2.0 ** -37) <= hi(sjj) - (39 << 20)).any()

@@ -1609,10 +1609,12 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
         double q = residual_quadratic_form_list<T>(j, s, a, sb, prev[2]);
         // q <= 1e-12 S_jj, decided on the upper words where they decide it
         const double sjj = prev[2];
-        // (q < 2^-38 S_jj, negative, or denormal)
-        if (__double2hiint(q) <= max(__double2hiint(sjj) - (39 << 20), 1 << 20)) {
+        // (q < 2^-38 S_jj, negative, denormal, infinite or NaN, as on a matrix that is
+        // not positive semidefinite; a NaN is at the floor too)
+        const int low = max(__double2hiint(sjj) - (39 << 20), 1 << 20) + 1;
+        if ((unsigned)(__double2hiint(q) - low) >= (unsigned)(0x7ff00000 - low)) {
             const double floor2 = 1e-12 * sjj;
-            if (q <= floor2) {
+            if (!(q > floor2)) {
                 q = floor2;
                 status |= COL_DEGENERATE;
             }
@@ -2813,7 +2815,7 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
             q = block_quadratic_form<T>(j, b, list, n, a, sc);
         if (tid < 32) {                                   // one warp on the FP64 pipe
             int f = (status & COL_DEGENERATE) ? 1 : 0;
-            if (q <= floor2) {
+            if (!(q > floor2)) {
                 q = floor2;
                 f = 1;
             }

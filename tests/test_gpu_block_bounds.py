@@ -35,3 +35,13 @@ def test_refreshes_by_chunk(p, kind, prec, tol, route):
     ref = oracle.spmesl(S, prob.lambda0, tol=1e-11, maxit=1000)
     res = compare_theta(T.cpu().numpy(), ref["Theta"], ref["B"], ref["sigma"], rel=BAR[prec])
     assert res["ok"], res
+
+
+def test_an_indefinite_matrix_is_refused():
+    """Coefficients that grow beyond FP32 end at the sigma floor, not as NaN in Theta."""
+    X = np.random.default_rng(0).standard_normal((60, 40))
+    A = X.T @ X / 60
+    A[0, 1] = A[1, 0] = 5.0
+    A[2, 3] = A[3, 2] = -4.0
+    with pytest.raises(sp.SpmeslError):
+        sp.fit(torch.from_numpy(A.astype(np.float32)).cuda(), 0.1, maxit=30)

@@ -329,7 +329,8 @@ spmesl_status spmesl_fit_residual(const void* X, int n, int p, int ldx, double l
 
 /* The regression coefficients of Eq. (5) (b_j of each column problem,
  * Algorithm 2): copy the coefficients of the last fit in `workspace` to B (p x p FP64
- * device buffer, original scale, B[j*p + k] = b_jk, zero diagonal). */
+ * device buffer, original scale, B[j*p + k] = b_jk, zero diagonal).  A fit that
+ * ended in ENONFINITE leaves B as it is. */
 spmesl_status spmesl_fit_coefficients(const void* workspace, int p, int precision, double* B,
                                       void* stream);
 

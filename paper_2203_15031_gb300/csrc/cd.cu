@@ -456,7 +456,9 @@ __global__ void lasso_export_kernel(const T* __restrict__ BT, const int* __restr
     if (k == 0) sigma_out[0] = sigma[r] / cs[r];
 }
 
-// B[j][k] = b_jk in the original scale: b^o_jk = b^C_jk c_j / c_k.
+// B[j][k] = b_jk in the original scale: b^o_jk = b^C_jk c_j / c_k.  A refused
+// fit has solved no column (its list lengths are whatever the workspace held),
+// so B is left as it is; a length is never taken beyond the list's room.
 template <typename T>
 __global__ void export_b_kernel(const T* __restrict__ BT, const int* __restrict__ nsup,
                                 const FitCtrl* __restrict__ ctrl, int p, int ldp, const double* cs,
@@ -464,10 +466,12 @@ __global__ void export_b_kernel(const T* __restrict__ BT, const int* __restrict_
     __shared__ T tile[32][33];
     const int j0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
     const int tx = threadIdx.x, ty = threadIdx.y;
+    if (ctrl->err == DEV_ERR_NONFINITE) return;
     const bool lists = ctrl->compact_b != 0;
     for (int rr = ty; rr < 32; rr += 8) {
         const int k = k0 + rr, j = j0 + tx;
-        const int n = (lists && k < p) ? nsup[k] : -1;      // warp-uniform (one ty per warp)
+        const int n = (lists && k < p) ? min(nsup[k], coef_cap(ldp)) : -1;   // warp-uniform (one ty
+                                                                             // per warp)
         const T* __restrict__ row = BT + (size_t)k * ldp;
         if (n < 0) {
             tile[rr][tx] = (k < p && j < p) ? row[j] : T(0);

@@ -35,7 +35,8 @@
 // n = 200, FP32, a fit: 16.9 ms with a whole slice formed per visit and per move;
 // 4.3 ms with quiet chunks; 3.5 ms with the growth bounded per chunk; 1.77 ms
 // with rows staged through shared memory (a visit 3800 -> under 1000 cycles)
-// and single coordinates formed after a move.  The same iterates bit for bit.
+// and single coordinates formed after a move.  Testing a quiet chunk again after each of
+// its moves takes 3.6 % of that fit.  The same iterates bit for bit.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -197,8 +198,6 @@ struct ResScan {
     unsigned nmoves;
 };
 
-// Chunks of [from, from + 32) that the sweep must visit (standardised data),
-// and in `full` those of them whose slice must be formed.
 // A chunk is quiet when none of its coordinates at zero can reach
 // the threshold.  Since the chunk was scanned, each move delta_m changed the
 // exact dot w_k' r by |delta_m w_k' w_m| <= |delta_m| cmax[m][chunk] (the bound
@@ -213,10 +212,24 @@ struct ResScan {
 // itself.  A coordinate at zero
 // in a quiet chunk would therefore have computed |g_k| < lambda and not moved:
 // a quiet chunk without support is skipped, and in one with support only the
-// support coordinates are formed and tested, in their order, so the sweep is
+// support coordinates are formed and tested, in their order, for as long as the
+// chunk stays quiet under their moves; after a move that may have carried a
+// coordinate at zero to the threshold the rest of the chunk is scanned.  So the sweep is
 // the same as a full scan.  (maxabs covers the coordinates that were zero
 // when the chunk was scanned; one that has come to zero since marks its chunk,
 // maxabs = infinity.)
+__device__ __forceinline__ bool quiet_chunk(const ResChunk& c, unsigned nmoves, float lam, float rmax,
+                                            int n) {
+    const unsigned dm = nmoves - c.moves_at;
+    if (dm > 4096u) return false;
+    const float bound = c.maxabs * (1.0f + 0x1p-22f) + c.grow * (1.0f + 0x1p-10f) +
+                        c.grow * (float)(dm + 2u) * 0x1p-23f +
+                        rmax * (float)(n + (int)dm + 2) * 0x1p-22f + lam * 0x1p-20f;
+    return bound < lam;
+}
+
+// Chunks of [from, from + 32) that the sweep must visit (standardised data),
+// and in `full` those of them whose slice must be formed (see quiet_chunk).
 template <bool STD>
 __device__ __forceinline__ unsigned res_chunks_to_visit(const ResScan& cs, int from, int nch,
                                                         float lam, float rmax, int n,
@@ -226,14 +239,8 @@ __device__ __forceinline__ unsigned res_chunks_to_visit(const ResScan& cs, int f
     if constexpr (STD) {
         if (scan) {
             const ResChunk c = cs.ci[ci];
-            const unsigned dm = cs.nmoves - c.moves_at;
-            if (dm <= 4096u) {
-                const float bound = c.maxabs * (1.0f + 0x1p-22f) + c.grow * (1.0f + 0x1p-10f) +
-                                    c.grow * (float)(dm + 2u) * 0x1p-23f +
-                                    rmax * (float)(n + (int)dm + 2) * 0x1p-22f + lam * 0x1p-20f;
-                scan = !(bound < lam);
-                visit = scan || c.nsupp != 0;
-            }
+            scan = !quiet_chunk(c, cs.nmoves, lam, rmax, n);
+            visit = scan || c.nsupp != 0;
         }
     }
     full = __ballot_sync(FULL_MASK, scan);
@@ -297,6 +304,7 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restri
         int e1 = e0;
         while (e1 < s.n && s.idx[e1] < cb + CHUNK) ++e1;
         const unsigned nmoves0 = cs.nmoves;
+        int cursor = cb;
         if constexpr (STD) {
             if (!((full >> bit) & 1u)) {
                 // a quiet chunk: its support coordinates in turn.  One costs a
@@ -304,6 +312,10 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restri
                 // under the chain before it; the whole slice it replaces read
                 // n rows of 512 bytes from L2.
                 T nx[RES_ROW];
+                bool quiet = true;
+                // of the coordinates that were zero when the chunk was visited: one that comes
+                // to zero now is behind the sweep and opens the chunk for the next one
+                const float maxabs = cs.ci[ci].maxabs;
                 if (a.stage && e0 < e1) load_row<T>(a, s.idx[e0], nx);
                 for (int e = e0; e < e1;) {
                     const int k = s.idx[e];
@@ -329,15 +341,24 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restri
                     maxd = fmax(maxd, fabs(delta));
                     note_residual_move<T, STD>(r, k, a, v, delta, cs, rn);
                     ++moves;
+                    ResChunk c = cs.ci[ci];
+                    c.maxabs = maxabs;
+                    if (!quiet_chunk(c, cs.nmoves, (float)lam, rn.rmax, a.n)) {
+                        quiet = false;            // the coordinates after k are scanned
+                        cursor = k + 1;
+                        break;
+                    }
                 }
-                if (lane == 0) cs.ci[ci].nsupp = e1 - e0;
-                __syncwarp();
-                if (cs.nmoves != nmoves0) {
-                    mbase = ci + 1;
-                    if (mbase >= nch) break;
-                    mask = res_chunks_to_visit<STD>(cs, mbase, nch, (float)lam, rn.rmax, a.n, full);
+                if (quiet) {
+                    if (lane == 0) cs.ci[ci].nsupp = e1 - e0;
+                    __syncwarp();
+                    if (cs.nmoves != nmoves0) {
+                        mbase = ci + 1;
+                        if (mbase >= nch) break;
+                        mask = res_chunks_to_visit<STD>(cs, mbase, nch, (float)lam, rn.rmax, a.n, full);
+                    }
+                    continue;
                 }
-                continue;
             }
         }
         const int k0 = cb + lane * SCAN_V;
@@ -361,7 +382,6 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restri
         bool fresh = true, gone = false;
         float grow = 0.f;
         unsigned formed_at = cs.nmoves;
-        int cursor = cb;
         for (;;) {
             const float reach = (float)lam - (grow * (1.0f + 0x1p-10f) +
                                               rn.rmax * (float)(a.n + 64) * 0x1p-21f +

@@ -19,8 +19,8 @@
 // rounding of v (2^-56 of the column's largest value) and the digit products
 // of level 7 and beyond, is below the rounding of an FP64 sum over the samples
 // relative to sqrt(S_jj S_kk).  Columns with non-finite values or extreme
-// exponents are not scaled: the epilogue forms every entry of their row and
-// column directly in FP64, in sample order.
+// exponents are not scaled: every entry of their row and column is an FP64 sum in
+// sample order (direct_tile, after the CTA's last tile).
 //
 // Measured, 50 fits of p = 500, n = 250 in one launch: 0.08 ms for the digits
 // and 0.18 ms for the products, against 3.21 ms of FP64 fused multiply-adds at
@@ -122,15 +122,78 @@ struct F64Many {
     __device__ const F64Fit& fit_at(int fi) const { return fits[fi]; }
 };
 
-// S_jk of a column that is not scaled: the FP64 sum in sample order.
-__device__ __noinline__ double direct_entry(const F64Fit& f, int j, int k) {
-    const double mj = f.mu ? f.mu[j] : 0.0, mk = f.mu ? f.mu[k] : 0.0;
-    double acc = 0.0;
-    for (int i = 0; i < f.n; ++i) {
-        const double* row = f.X + (size_t)i * f.ldx;
-        acc = fma(row[j] - mj, row[k] - mk, acc);
+// The tile's entries whose row or column is not scaled (F64_EXPO_DIRECT): FP64
+// sums in sample order, by the whole CTA once its scaled tiles are done and no
+// role waits any more (one such column takes n times the epilogue's work, which no
+// bounded wait can cover).  Bound by the FP64 pipe; a warp (8 of them, 32 x 32
+// entries each, 8 x 4 a lane) forms only what one of its lanes needs.
+constexpr int F64_DIRECT_BK = 16;
+__device__ __noinline__ void direct_tile(const F64Fit& f, int tm, int tn, double* __restrict__ sm) {
+    double (*As)[TC_BM] = reinterpret_cast<double (*)[TC_BM]>(sm);
+    double (*Bs)[F64_BN] = reinterpret_cast<double (*)[F64_BN]>(sm + F64_DIRECT_BK * TC_BM);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int m0 = tm * TC_BM, n0 = tn * F64_BN, p = f.p;
+    const int r0 = 32 * (warp & 3) + 8 * (lane >> 3), c0 = 32 * (warp >> 2) + 4 * (lane & 7);
+    unsigned need = 0u;                       // bit 4 u + v: entry (r0 + u, c0 + v)
+    if (warp < 8) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int row = m0 + r0 + u;
+            if (row >= p) break;
+            const bool dr = f.expo[row] == F64_EXPO_DIRECT;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int col = n0 + c0 + v;
+                if (col < p && col >= row && (dr || f.expo[col] == F64_EXPO_DIRECT))
+                    need |= 1u << (4 * u + v);
+            }
+        }
     }
-    return acc * f.inv_n;
+    const unsigned wneed = __reduce_or_sync(FULL_MASK, need);
+    if (!__syncthreads_or(wneed != 0u)) return;
+    double acc[8][4];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+    for (int i0 = 0; i0 < f.n; i0 += F64_DIRECT_BK) {
+        for (int e = tid; e < F64_DIRECT_BK * (TC_BM + F64_BN); e += F64_THREADS) {
+            const int kk = e / (TC_BM + F64_BN), c = e % (TC_BM + F64_BN);
+            const int col = c < TC_BM ? m0 + c : n0 + c - TC_BM;
+            double x = 0.0;
+            if (i0 + kk < f.n && col < p)
+                x = f.X[(size_t)(i0 + kk) * f.ldx + col] - (f.mu ? f.mu[col] : 0.0);
+            if (c < TC_BM) As[kk][c] = x;
+            else Bs[kk][c - TC_BM] = x;
+        }
+        __syncthreads();
+        if (wneed) {
+#pragma unroll 1
+            for (int kk = 0; kk < F64_DIRECT_BK; ++kk) {
+                double b[4];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) b[v] = Bs[kk][c0 + v];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const double a = As[kk][r0 + u];
+#pragma unroll
+                    for (int v = 0; v < 4; ++v)
+                        if ((wneed >> (4 * u + v)) & 1u) acc[u][v] = fma(a, b[v], acc[u][v]);
+                }
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            if ((need >> (4 * u + v)) & 1u) {
+                const size_t row = m0 + r0 + u, col = n0 + c0 + v;
+                const double s = acc[u][v] * f.inv_n;
+                f.S[row * f.lds + col] = s;
+                f.S[col * f.lds + row] = s;
+            }
 }
 
 // W = L_0 256^6 + .. + L_6 from the seven integer-valued level sums: the
@@ -164,6 +227,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
     volatile int* fail = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* issued_slot = fail + 1;
     volatile int* consumed_slot = fail + 2;
+    volatile int* direct_slot = fail + 3;     // some column of the CTA's tiles is not scaled
     volatile int* kt_ring = fail + 4;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -180,6 +244,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
         *fail = 0;
         *issued_slot = 0;
         *consumed_slot = 0;
+        *direct_slot = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -341,7 +406,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
                 if (!ok) {
                     acc[i] = __longlong_as_double(0x7ff8000000000000ll);
                 } else if (Ej == F64_EXPO_DIRECT || Ek == F64_EXPO_DIRECT) {
-                    acc[i] = (row < p && c0 + i < p) ? direct_entry(f, row, c0 + i) : 0.0;
+                    acc[i] = 0.0;                         // formed by direct_tile
+                    *direct_slot = 1;
                 } else {
                     acc[i] *= __longlong_as_double(__double_as_longlong(sj) + ((long long)Ek << 52));
                 }
@@ -380,6 +446,15 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (*direct_slot) {
+        // (the stage buffers are idle, and the CTA's own tiles hold these entries)
+        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+            const F64Fit& f = src.fit_at(src.fit_index(tile));
+            int tm, tn;
+            f.g.coords(tile - f.tile_start, tm, tn);
+            direct_tile(f, tm, tn, reinterpret_cast<double*>(stages));
+        }
+    }
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),

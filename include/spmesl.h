@@ -190,10 +190,12 @@ double spmesl_lambda(int rule, int n, int p);
  *   workspace  device scratch of at least spmesl_gram_workspace_bytes(n, p,
  *              precision) bytes (may be NULL when that is 0).
  * SPMESL_FP32 accumulates in FP32 on the CUDA cores.  SPMESL_FP64 forms the
- * products without error as 8-bit digit products on the tensor cores and sums
- * them to FP64 accuracy relative to sqrt(S_jj S_kk) (columns with non-finite or
- * extreme values as FP64 sums in sample order).  SPMESL_MIXED splits X = hi + lo into two BF16 parts and forms
- * hi'hi + hi'lo + lo'hi on the tensor cores (tcgen05, TMEM accumulators)
+ * products on the tensor cores from 8-bit digits of each column's values, 56 bits
+ * below its largest, with the error of an FP64 sum over the samples or less relative to
+ * sqrt(S_jj S_kk).  Columns with non-finite or extreme values (beyond 2^+-400), and
+ * those with more than a quarter of their nonzero samples 2^10 times and more below the
+ * largest, are FP64 sums in sample order.  SPMESL_MIXED splits X = hi + lo into two
+ * BF16 parts and forms hi'hi + hi'lo + lo'hi on the tensor cores (tcgen05, TMEM accumulators)
  * with FP32 accumulation.
  * Errors: EINVAL for n < 1, p < 1, ldx < p, lds < p, NULL pointers, a short
  * workspace; ECUDA if a launch fails.

@@ -8,34 +8,44 @@
 // of X (centred if asked) is scaled by its largest magnitude, |x_ij| < 2^E_j,
 // and rounded to the integer v_ij = x_ij 2^(55 - E_j), whose seven balanced
 // base-256 digits are exact in BF16.  Digit products are integers of at most
-// 2^14, and a level L_l = sum over s + t = l of sum_i d_is d_it, l = 0..6, is
+// 2^14, and a level L_l = sum over s + t = l of sum_i d_is d_it, l = 0..7, is
 // summed by tcgen05.mma in one FP32 accumulator exactly while it stays below
 // 2^24: for up to 256 samples that holds for every input in the levels 0 to 3;
-// the levels 4 to 6 (weights 2^-32 and below) can pass 2^24 only when nearly
+// the levels 4 to 7 (weights 2^-32 and below) can pass 2^24 only when nearly
 // all digits are extreme and of one sign, and are then off by units that weigh
 // less than 2^-50 of the sum.  After at most 256 samples the levels are
-// combined as W = sum_l L_l 256^(6-l), two exact 64-bit integers and one
-// FP64 rounding, and S_jk = W 2^(E_j + E_k - 62) / n.  What is left out, the
-// rounding of v (2^-56 of the column's largest value) and the digit products
-// of level 7 and beyond, is below the rounding of an FP64 sum over the samples
-// relative to sqrt(S_jj S_kk).  Columns with non-finite values or extreme
-// exponents are not scaled: every entry of their row and column is an FP64 sum in
-// sample order (direct_tile, after the CTA's last tile).
+// combined as W = sum_l L_l 256^(7-l), two exact 64-bit integers and one
+// FP64 rounding, and S_jk = W 2^(E_j + E_k - 70) / n.
 //
-// Measured, 50 fits of p = 500, n = 250 in one launch: 0.08 ms for the digits
-// and 0.18 ms for the products, against 3.21 ms of FP64 fused multiply-adds at
-// the FP64 pipe's rate (1.84e9, 0.58 T/s).  One fit: p = 100, n = 50 31 us
-// against 72, p = 1500, n = 1000 283 us against 2050.  Error of an entry
-// relative to sqrt(S_jj S_kk) against exact rational sums, N(0, 1) data,
-// n = 250: rms 1.4e-17, largest 3.7e-17, against 3.1e-17 and 9.2e-17 of the FP64
-// sum in sample order; n = 30: 2.3e-17 and 6.3e-17 against 4.0e-17 and 1.7e-16.
+// What is left out: the rounding of v, 2^-56 of the column's largest value
+// a sample, and the digit products of level 8 and beyond (2^-64 of both largest
+// values).  Relative to sqrt(S_jj S_kk) the first is a random sum of about
+// 2^-56.8 R / sqrt(n), R = 2^E over the column's root mean square, which is at most
+// 2 sqrt(n): below the FP64 sum's own error, whatever the tails.  (Without level
+// 7 it was 2^-56.3 R_j R_k / sqrt(n): 4 times the FP64 sum's error for Student t
+// with 2 degrees at n = 1000, 30 times for log-normal data.)  Where one sample
+// outweighs the rest and an entry does not see it, an FP64 sum is closer still: a column
+// with non-finite values, extreme exponents or that many small samples (f64_digit_columns) is
+// not scaled, every entry of its row and column is an FP64 sum in sample order
+// (direct_tile, after the CTA's last tile).
+//
+// Error of an entry off the diagonal relative to sqrt(S_jj S_kk) against 113-bit sums, a CPU
+// restatement, rms, against the FP64 sum in sample order: N(0, 1) n = 30 1.5e-17
+// (3.4e-17), n = 250 5.4e-18 (3.7e-17); t with 5 degrees, n = 250 6.8e-18 (3.5e-17);
+// with 2, n = 1000 9.9e-18 (4.6e-17); log-normal s = 1, n = 1000 6.0e-17 (3.1e-16).
+//
+// Measured: p = 100, n = 50 29 us against 72 of FP64 fused multiply-adds at the FP64
+// pipe's rate (1.84e9, 0.58 T/s), p = 1500, n = 1000 222 us against 2050, 50 fits of
+// p = 500, n = 250 in one launch 0.23 ms with the digits against 3.21.  (Seven levels,
+// an instruction per pair of digits: 30, 259 us and 0.26 ms; eight levels so 0.28.)
 //
 // Kernel: persistent, one CTA of 10 warps per SM over 128 x 64 tiles that hold
-// an entry of the upper triangle.  Seven 64-column accumulators fill the
-// tensor memory (448 of 512 columns), which sets the tile: 128 x 128 would need
-// 896.  Per K block of 32 samples, warp 0 loads the seven digit planes of the
+// an entry of the upper triangle.  Eight 64-column accumulators fill the
+// tensor memory, which sets the tile.  Per K block of 32 samples, warp 0 loads the seven digit planes of the
 // tile's rows and columns (two TMA boxes, 84 KB, 64-byte swizzle, two stages);
-// one lane of warp 1 issues 28 products for each 16 samples; warps 2 to 9
+// one lane of warp 1 issues the 34 digit products of each 16 samples as 12 instructions
+// over neighbouring planes (an instruction of one 64-column plane waits for its 6 KB of
+// operands longer than for its products); warps 2 to 9
 // combine the levels, 32 rows x 32 columns each, hand the accumulators back,
 // and write the tile and its mirror while the next tile's products run.
 // Waits, failure and tensor-memory release as in gram_tc.cu.
@@ -68,11 +78,15 @@ constexpr int F64_NBARS = 2 * F64_STAGES + 3;
 constexpr size_t F64_SMEM = (size_t)F64_STAGES * F64_STAGE_BYTES + F64_EPI_WARPS * F64_EPI_BYTES +
                             F64_NBARS * 8 + 64 + 1024;
 static_assert(F64_SMEM <= 232448, "shared memory of one block");
-static_assert(F64_SLICES * F64_BN <= F64_TMEM_COLS, "tensor memory");
+static_assert(F64_LEVELS * F64_BN <= F64_TMEM_COLS, "tensor memory");
+static_assert(F64_SLICES == 7 && F64_LEVELS == 8, "the products are listed for these");
 static_assert(F64_FLUSH % F64_KB == 0 && TC_NPAD % F64_KB == 0, "K blocks");
-// instruction descriptor: BF16 x BF16 -> FP32, both K-major, M = 128, N = 64
-constexpr unsigned F64_IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
-                               ((unsigned)(F64_BN >> 3) << 17) | ((unsigned)(TC_BM >> 4) << 24);
+// instruction descriptor: BF16 x BF16 -> FP32, both K-major, M = 128, N = m digit
+// planes of F64_BN columns
+__host__ __device__ constexpr unsigned f64_idesc(int m) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)((m * F64_BN) >> 3) << 17) |
+           ((unsigned)(TC_BM >> 4) << 24);
+}
 
 // Shared-memory descriptor of a K-major operand plane with 64-byte rows and
 // 64-byte swizzle (8-row groups 512 bytes apart; planes start on 512 bytes).
@@ -87,11 +101,12 @@ __device__ __forceinline__ unsigned long long plane_desc(unsigned addr) {
 }
 
 __device__ __forceinline__ void mma_digits(unsigned tmem_d, unsigned long long a,
-                                           unsigned long long b, unsigned accumulate) {
+                                           unsigned long long b, unsigned idesc,
+                                           unsigned accumulate) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(F64_IDESC), "r"(accumulate));
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
 __device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap* map, int x, int y,
@@ -196,17 +211,17 @@ __device__ __noinline__ void direct_tile(const F64Fit& f, int tm, int tn, double
             }
 }
 
-// W = L_0 256^6 + .. + L_6 from the seven integer-valued level sums: the
-// upper four and the lower three levels as 64-bit integers (below 2^50), made
+// W = L_0 256^7 + .. + L_7 from the eight integer-valued level sums: the
+// upper and the lower four levels as 64-bit integers (below 2^50), made
 // FP64 by the 1.5 2^52 offset, and one rounding.
-__device__ __forceinline__ double combine_levels(const unsigned (&L)[F64_SLICES][8], int c) {
+__device__ __forceinline__ double combine_levels(const unsigned (&L)[F64_LEVELS][8], int c) {
     auto I = [&](int l) { return (long long)__float2int_rn(__uint_as_float(L[l][c])); };
     const long long hi = ((I(0) * 256 + I(1)) * 256 + I(2)) * 256 + I(3);
-    const long long lo = (I(4) * 256 + I(5)) * 256 + I(6);
+    const long long lo = ((I(4) * 256 + I(5)) * 256 + I(6)) * 256 + I(7);
     const double off = 6755399441055744.0;
     const double h = __longlong_as_double(0x4338000000000000ll + hi) - off;
     const double l = __longlong_as_double(0x4338000000000000ll + lo) - off;
-    return fma(h, 16777216.0, l);
+    return fma(h, 4294967296.0, l);
 }
 
 template <class Src>
@@ -326,14 +341,27 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
                     for (int kk = 0; kk < F64_KB / 16; ++kk) {
                         // 16 bf16 = 32 bytes along K inside the swizzled rows
                         const unsigned long long off = (unsigned long long)((32 * kk) >> 4);
-#pragma unroll
-                        for (int l = 0; l < F64_SLICES; ++l)
-#pragma unroll
-                            for (int t = 0; t <= l; ++t)
-                                mma_digits(tmem + l * F64_BN,
-                                           a0 + off + (unsigned long long)((t * F64_A_PLANE) >> 4),
-                                           b0 + off + (unsigned long long)(((l - t) * F64_B_PLANE) >> 4),
-                                           (!first || kk || t) ? 1u : 0u);
+                        // plane t of the rows by planes u .. u + m - 1 of the columns, which follow
+                        // one another in shared memory as the levels t + u .. do in tensor memory
+                        auto products = [&](int t, int u, int m, bool add) {
+                            mma_digits(tmem + (t + u) * F64_BN,
+                                       a0 + off + (unsigned long long)((t * F64_A_PLANE) >> 4),
+                                       b0 + off + (unsigned long long)((u * F64_B_PLANE) >> 4),
+                                       f64_idesc(m), add ? 1u : 0u);
+                        };
+                        const bool add = !first || kk;
+                        products(0, 0, 4, add);
+                        products(0, 4, 3, add);
+                        products(1, 0, 4, true);
+                        products(1, 4, 2, true);
+                        products(1, 6, 1, add);            // level 7's first
+                        products(2, 0, 4, true);
+                        products(2, 4, 2, true);
+                        products(3, 0, 3, true);
+                        products(3, 3, 2, true);
+                        products(4, 0, 4, true);
+                        products(5, 0, 3, true);
+                        products(6, 0, 2, true);
                     }
                     mma_commit(smem_u32(&empty[s]));
                     if ((kt + 1) % (F64_FLUSH / F64_KB) == 0 || kt + 1 == KT) {
@@ -375,9 +403,9 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
                 if (any && ok) {
 #pragma unroll
                     for (int c = 0; c < 32; c += 8) {
-                        unsigned L[F64_SLICES][8];
+                        unsigned L[F64_LEVELS][8];
 #pragma unroll
-                        for (int l = 0; l < F64_SLICES; ++l)
+                        for (int l = 0; l < F64_LEVELS; ++l)
                             tmem_ld8(tmem + ((unsigned)(32 * q) << 16) +
                                          (unsigned)(l * F64_BN + 32 * half + c),
                                      L[l]);
@@ -397,8 +425,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
             double* __restrict__ S = f.S;
             const int row = m0 + lane;
             const int Ej = row < p ? f.expo[row] : 0;
-            // inv_n 2^(E_j - 62); E_k is added to its exponent per column
-            const double sj = Ej == F64_EXPO_DIRECT ? f.inv_n : scalbn(f.inv_n, Ej - 62);
+            // inv_n 2^(E_j - 70); E_k is added to its exponent per column
+            const double sj = Ej == F64_EXPO_DIRECT ? f.inv_n : scalbn(f.inv_n, Ej - 70);
             const int my_E = c0 + lane < p ? f.expo[c0 + lane] : 0;
 #pragma unroll
             for (int i = 0; i < 32; ++i) {

@@ -12,6 +12,7 @@
 namespace spmesl {
 
 constexpr int F64_SLICES = 7;         // 8-bit digits of a column's scaled values
+constexpr int F64_LEVELS = 8;         // sums of digit products by weight (see gram_f64.cu)
 constexpr int F64_BN = 64;            // output tile: TC_BM rows x F64_BN columns
 constexpr int F64_EXPO_DIRECT = INT_MAX;   // column whose products are formed directly in FP64
 constexpr int F64_EXPO_MAX = 400;     // largest |exponent| that the digits' scaling handles
@@ -55,10 +56,25 @@ __device__ __forceinline__ void f64_digits(double x, int E, int (&d)[F64_SLICES]
     d[0] = (int)v;
 }
 
+// Whether x counts for F64_EXPO_DIRECT's rule: 1 for a nonzero value, and 2^16
+// more when it is below 2^(E - F64_SMALL).
+constexpr int F64_SMALL = 10;
+__device__ __forceinline__ unsigned f64_small(double x, int E) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x) << 1;
+    const int e = (int)(u >> 53);                     // |x| in [2^(e - 1023), 2^(e - 1022))
+    return u == 0ull ? 0u : (e - 1022 <= E - F64_SMALL ? 0x10001u : 1u);
+}
+
 // Exponents and digit planes of columns c0 .. c0 + 31 of X, centred by mu when
 // given (block 32 x 8).  The largest magnitude of a column sets its exponent
 // E (|x| < 2^E); a column with a non-finite value or an exponent beyond
-// F64_EXPO_MAX is marked F64_EXPO_DIRECT and gets zero digits.  Magnitudes are
+// F64_EXPO_MAX is marked F64_EXPO_DIRECT and gets zero digits.  So is, by its
+// digits' own pass, a column with more than a quarter of its nonzero samples
+// below 2^(E - F64_SMALL): a few samples that large set the digits' unit, and an FP64
+// sum in which they meet small partners is closer than the digits are.  Normal samples
+// pass the rule by far (0.5 % of them are that small), Student t with 2 degrees too;
+// log-normal (s = 3) and Cauchy columns and a column of ordinary samples with one of
+// 10^3 or more are marked.  Magnitudes are
 // compared and digits formed on the integer pipe: the FP64 pipe takes 16 cycles
 // an instruction.  Samples n .. n_pad - 1 are written as zeros.  Each pass of 64
 // samples loads the next one's (81 -> 78 us for 50 fits of p = 500, n = 250).
@@ -68,6 +84,7 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
                                                   __nv_bfloat16* __restrict__ D, int n_pad, int c0) {
     __shared__ long long red[8][33];
     __shared__ int sE[32];
+    __shared__ unsigned nonzero[32], small[32];        // samples of each column (by its warp)
     __shared__ double tile[32][65];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int cl = c0 + tx;
@@ -90,6 +107,7 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
         int E = mx == 0 ? 0 : e - 1022;
         if (e == 0x7ff || E > F64_EXPO_MAX || E < -F64_EXPO_MAX) E = F64_EXPO_DIRECT;
         sE[tx] = E;
+        nonzero[tx] = small[tx] = 0u;
         if (cl < p) expo[cl] = E;
     }
     __syncthreads();
@@ -117,8 +135,14 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
 #pragma unroll
                     for (int s = 0; s < F64_SLICES; ++s) d0[s] = d1[s] = 0;
                 } else {
-                    f64_digits(tile[r][2 * tx], E, d0);
-                    f64_digits(tile[r][2 * tx + 1], E, d1);
+                    const double x0 = tile[r][2 * tx], x1 = tile[r][2 * tx + 1];
+                    f64_digits(x0, E, d0);
+                    f64_digits(x1, E, d1);
+                    const unsigned few = __reduce_add_sync(FULL_MASK, f64_small(x0, E) + f64_small(x1, E));
+                    if (tx == 0) {
+                        nonzero[r] += few & 0xffffu;
+                        small[r] += few >> 16;
+                    }
                 }
                 __nv_bfloat16* out = D + (size_t)c * n_pad + i0 + 2 * tx;
 #pragma unroll
@@ -134,6 +158,9 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
         }
         __syncthreads();
     }
+    if (tx == 0)
+        for (int r = ty; r < 32; r += 8)
+            if (c0 + r < p && 4ull * small[r] > nonzero[r]) expo[c0 + r] = F64_EXPO_DIRECT;
 }
 
 // Fill f (host side).  False if the tensor maps could not be encoded.

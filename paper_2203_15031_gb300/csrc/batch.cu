@@ -123,12 +123,12 @@ __global__ void batch_split_kernel(const BatchFit* __restrict__ fits,
 // of 32 x 8 per 32 columns.
 __global__ void __launch_bounds__(256) batch_digits_kernel(const BatchFit* __restrict__ fits,
                                                           const int* __restrict__ split_prefix,
-                                                          int count) {
+                                                          int count, int* __restrict__ marks) {
     const int fi = find_fit(split_prefix, count, blockIdx.x);
     const BatchFit& f = fits[fi];
     f64_digit_columns(static_cast<const double*>(f.X), f.n, f.p, f.p,
                       static_cast<const double*>(f.mu), static_cast<int*>(f.XlT),
-                      static_cast<__nv_bfloat16*>(f.XhT), tc_pad_n(f.n),
+                      marks + blockIdx.x, static_cast<__nv_bfloat16*>(f.XhT), tc_pad_n(f.n),
                       (blockIdx.x - f.split_start) * 32);
 }
 
@@ -530,6 +530,9 @@ struct spmesl_batch {
     // SPMESL_MIXED, SPMESL_FP64: tensor-core Gram table, fit of every tile, split prefixes
     size_t off_tcfit = 0, off_tilefit = 0, off_splitp = 0;
     int total_split = 0;
+    // SPMESL_FP64: marks of the columns that the Gram does not scale, and their blocks
+    size_t off_marks = 0;
+    int total_direct = 0;
     size_t ws_bytes = 0;
     int total_cols = 0, total_gram = 0, total_theta = 0, max_ldp = 32, max_p = 2, max_n = 1;
     bool any_x = false;
@@ -586,11 +589,13 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
                 return e;
         } else if constexpr (sizeof(T) == 8) {
             batch_digits_kernel<<<b->total_split, dim3(32, 8), 0, st>>>(
-                fits, reinterpret_cast<const int*>(ws + b->off_splitp), count);
-            if ((e = launch_gram_f64_batch(reinterpret_cast<const F64Fit*>(ws + b->off_tcfit),
-                                           reinterpret_cast<const int*>(ws + b->off_tilefit),
-                                           b->total_gram, st)) != cudaSuccess)
-                return e;
+                fits, reinterpret_cast<const int*>(ws + b->off_splitp), count,
+                reinterpret_cast<int*>(ws + b->off_marks));
+            const F64Batch g{reinterpret_cast<const F64Fit*>(ws + b->off_tcfit),
+                             reinterpret_cast<const int*>(ws + b->off_tilefit),
+                             reinterpret_cast<const int*>(ws + b->off_marks), count, b->total_gram,
+                             b->total_split, b->total_direct};
+            if ((e = launch_gram_f64_batch(g, st)) != cudaSuccess) return e;
         } else {
             batch_gram_kernel<<<b->total_gram, GRAM_THREADS, 0, st>>>(fits, gramp, count);
         }
@@ -785,6 +790,7 @@ bool stage_table(spmesl_batch* b, unsigned char* ws) {
             if (f.X) {
                 if (!f64_encode_fit(dgf[i], static_cast<const double*>(f.X), f.n, f.p, f.p,
                                     static_cast<const double*>(d.mu), static_cast<const int*>(d.XlT),
+                                    reinterpret_cast<const int*>(ws + b->off_marks) + f.split_start,
                                     d.XhT, static_cast<double*>(d.Sg), f.p, f.gram_start))
                     return false;
                 const int nt = dgf[i].g.count();
@@ -887,6 +893,7 @@ spmesl_status spmesl_batch_create(const spmesl_problem* probs, int count, double
     b->table_bytes = off - b->off_desc;
     b->off_ctrls = off; off += (size_t)256 * count;      // one FitCtrl slot per fit
     int cols = 0, gram = 0, theta = 0, split = 0, prep = 0;
+    long long direct = 0;
     for (int k = 0; k < count; ++k) {
         const spmesl_problem& q = probs[order[k]];
         FitPlan f{};
@@ -930,6 +937,7 @@ spmesl_status spmesl_batch_create(const spmesl_problem* probs, int count, double
         if (q.X && tc) {
             gram += tc_tile_grid(f.p, tc_bn).count();
             split += (mixed ? tc_pad_n(f.n) / 64 : 1) * ((f.p + 31) / 32);
+            if (!mixed) direct = std::min<long long>(direct + f64_direct_blocks(f.p), INT_MAX);
         } else if (q.X) {
             const int t = (f.p + GRAM_BM - 1) / GRAM_BM;
             gram += t * (t + 1) / 2;
@@ -947,6 +955,11 @@ spmesl_status spmesl_batch_create(const spmesl_problem* probs, int count, double
     b->total_cols = cols;
     b->total_gram = gram;
     b->total_split = split;
+    b->total_direct = (int)direct;
+    if (tc && !mixed) {
+        b->off_marks = off;
+        off += align_up(sizeof(int) * (size_t)std::max(split, 1), 256);
+    }
     b->total_theta = theta;
     b->total_prep = prep;
     if (b->count_rows) {

@@ -27,7 +27,7 @@
 // outweighs the rest and an entry does not see it, an FP64 sum is closer still: a column
 // with non-finite values, extreme exponents or that many small samples (f64_digit_columns) is
 // not scaled, every entry of its row and column is an FP64 sum in sample order
-// (direct_tile, after the CTA's last tile).
+// (direct_entries).
 //
 // Error of an entry off the diagonal relative to sqrt(S_jj S_kk) against 113-bit sums, a CPU
 // restatement, rms, against the FP64 sum in sample order: N(0, 1) n = 30 1.5e-17
@@ -123,92 +123,143 @@ struct F64One {
     int n_tiles;
     static constexpr bool kTableMaps = false;
     __device__ int tiles() const { return n_tiles; }
+    __device__ int fits() const { return 1; }
     __device__ int fit_index(int) const { return 0; }
     __device__ const F64Fit& fit_at(int) const { return f; }
+    __device__ const int* marks() const { return f.marks; }
+    __device__ int n_marks() const { return (f.p + 31) / 32; }
 };
 
 struct F64Many {
-    const F64Fit* fits;
-    const int* tile_fit;
-    int n_tiles;
+    F64Batch b;
     static constexpr bool kTableMaps = true;
-    __device__ int tiles() const { return n_tiles; }
-    __device__ int fit_index(int tile) const { return __ldg(tile_fit + tile); }
-    __device__ const F64Fit& fit_at(int fi) const { return fits[fi]; }
+    __device__ int tiles() const { return b.n_tiles; }
+    __device__ int fits() const { return b.n_fits; }
+    __device__ int fit_index(int tile) const { return __ldg(b.tile_fit + tile); }
+    __device__ const F64Fit& fit_at(int fi) const { return b.fits[fi]; }
+    __device__ const int* marks() const { return b.marks; }
+    __device__ int n_marks() const { return b.n_marks; }
 };
 
-// The tile's entries whose row or column is not scaled (F64_EXPO_DIRECT): FP64
-// sums in sample order, by the whole CTA once its scaled tiles are done and no
-// role waits any more (one such column takes n times the epilogue's work, which no
-// bounded wait can cover).  Bound by the FP64 pipe; a warp (8 of them, 32 x 32
-// entries each, 8 x 4 a lane) forms only what one of its lanes needs.
-constexpr int F64_DIRECT_BK = 16;
-__device__ __noinline__ void direct_tile(const F64Fit& f, int tm, int tn, double* __restrict__ sm) {
-    double (*As)[TC_BM] = reinterpret_cast<double (*)[TC_BM]>(sm);
-    double (*Bs)[F64_BN] = reinterpret_cast<double (*)[F64_BN]>(sm + F64_DIRECT_BK * TC_BM);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = tm * TC_BM, n0 = tn * F64_BN, p = f.p;
-    const int r0 = 32 * (warp & 3) + 8 * (lane >> 3), c0 = 32 * (warp >> 2) + 4 * (lane & 7);
-    unsigned need = 0u;                       // bit 4 u + v: entry (r0 + u, c0 + v)
-    if (warp < 8) {
+// The entries of rows r0 .. r0 + 31 and columns c0 .. c0 + 63 whose row or column is
+// not scaled (F64_EXPO_DIRECT): FP64 sums in sample order.  Bound by the FP64 pipe
+// (16 cycles of the SM an instruction of a warp), so a warp's instruction is a group of 32
+// entries that are wanted: half a row that is not scaled, or a column that is not scaled
+// over the 32 rows; when these come to more than the block's 64 half rows, the half rows.
+// Blocks of 32 x 64, in turn over the grid, keep every SM at work: p = 500, n = 250 48 us
+// without such columns, 82 with one, 197 with all of them (567 and 624 when each CTA
+// formed them for its own 128 x 64 tiles); p = 1500, n = 1000 221, 345 and 2573
+// (the products alone take 1.94 ms of the FP64 pipe).
+constexpr int F64_DIRECT_BK = 64;
+constexpr int F64_DIRECT_WARPS = 8;                   // that form them: 64 groups come out even
+constexpr int F64_DIRECT_GROUPS = 64 / F64_DIRECT_WARPS;
+static_assert(F64_DIRECT_BK * (32 + F64_BN) * 8 <= F64_STAGES * F64_STAGE_BYTES, "stage buffers");
+__device__ __noinline__ void direct_block(const F64Fit& f, int r0, int c0, double* __restrict__ sm) {
+    double (*As)[32] = reinterpret_cast<double (*)[32]>(sm);
+    double (*Bs)[F64_BN] = reinterpret_cast<double (*)[F64_BN]>(sm + F64_DIRECT_BK * 32);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, p = f.p;
+    auto unscaled = [&](int c) { return c < p && f.expo[c] == F64_EXPO_DIRECT; };
+    const unsigned rows = __ballot_sync(FULL_MASK, unscaled(r0 + lane));
+    const unsigned lo = __ballot_sync(FULL_MASK, unscaled(c0 + lane));
+    const unsigned hi = __ballot_sync(FULL_MASK, unscaled(c0 + 32 + lane));
+    const int nr = 2 * __popc(rows), nlo = __popc(lo), nc = nlo + __popc(hi);
+    const bool half_rows = nr + nc > 64;
+    const int groups = half_rows ? 64 : nr + nc;
+    int ia[F64_DIRECT_GROUPS], ib[F64_DIRECT_GROUPS], cnt = 0;
+    unsigned valid = 0u;
+    double acc[F64_DIRECT_GROUPS];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int row = m0 + r0 + u;
-            if (row >= p) break;
-            const bool dr = f.expo[row] == F64_EXPO_DIRECT;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const int col = n0 + c0 + v;
-                if (col < p && col >= row && (dr || f.expo[col] == F64_EXPO_DIRECT))
-                    need |= 1u << (4 * u + v);
-            }
+    for (int q = 0; q < F64_DIRECT_GROUPS; ++q) {
+        const int g = warp + q * F64_DIRECT_WARPS;
+        acc[q] = 0.0;
+        ia[q] = ib[q] = 0;
+        if (warp < F64_DIRECT_WARPS && g < groups) {
+            const bool column = !half_rows && g >= nr;
+            int r = lane, c = 32 * (g & 1) + lane;
+            if (half_rows) r = g >> 1;
+            else if (!column) r = (int)__fns(rows, 0, (g >> 1) + 1);
+            else if (g - nr < nlo) c = (int)__fns(lo, 0, g - nr + 1);
+            else c = 32 + (int)__fns(hi, 0, g - nr - nlo + 1);
+            const bool dr = (rows >> r) & 1u, dc = ((c < 32 ? lo : hi) >> (c & 31)) & 1u;
+            if (r0 + r < p && c0 + c < p && c0 + c >= r0 + r && (dr || dc) && !(column && dr))
+                valid |= 1u << q;
+            ia[q] = r;
+            ib[q] = c;
+            cnt = q + 1;
         }
     }
-    const unsigned wneed = __reduce_or_sync(FULL_MASK, need);
-    if (!__syncthreads_or(wneed != 0u)) return;
-    double acc[8][4];
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
     for (int i0 = 0; i0 < f.n; i0 += F64_DIRECT_BK) {
-        for (int e = tid; e < F64_DIRECT_BK * (TC_BM + F64_BN); e += F64_THREADS) {
-            const int kk = e / (TC_BM + F64_BN), c = e % (TC_BM + F64_BN);
-            const int col = c < TC_BM ? m0 + c : n0 + c - TC_BM;
-            double x = 0.0;
-            if (i0 + kk < f.n && col < p)
-                x = f.X[(size_t)(i0 + kk) * f.ldx + col] - (f.mu ? f.mu[col] : 0.0);
-            if (c < TC_BM) As[kk][c] = x;
-            else Bs[kk][c - TC_BM] = x;
+        const int nk = min(F64_DIRECT_BK, f.n - i0);
+        __syncthreads();                      // the last samples' readers are done
+#pragma unroll 4
+        for (int e = tid; e < nk * (32 + F64_BN); e += F64_THREADS) {
+            const int kk = e / (32 + F64_BN), c = e % (32 + F64_BN);
+            const int col = c < 32 ? r0 + c : c0 + c - 32;
+            const double x = col < p ? f.X[(size_t)(i0 + kk) * f.ldx + col] - (f.mu ? f.mu[col] : 0.0)
+                                     : 0.0;
+            if (c < 32) As[kk][c] = x;
+            else Bs[kk][c - 32] = x;
         }
         __syncthreads();
-        if (wneed) {
-#pragma unroll 1
-            for (int kk = 0; kk < F64_DIRECT_BK; ++kk) {
-                double b[4];
 #pragma unroll
-                for (int v = 0; v < 4; ++v) b[v] = Bs[kk][c0 + v];
+        for (int q = 0; q < F64_DIRECT_GROUPS; ++q) {
+            if (q >= cnt) break;
+#pragma unroll 4
+            for (int kk = 0; kk < nk; ++kk) acc[q] = fma(As[kk][ia[q]], Bs[kk][ib[q]], acc[q]);
+        }
+    }
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const double a = As[kk][r0 + u];
-#pragma unroll
-                    for (int v = 0; v < 4; ++v)
-                        if ((wneed >> (4 * u + v)) & 1u) acc[u][v] = fma(a, b[v], acc[u][v]);
+    for (int q = 0; q < F64_DIRECT_GROUPS; ++q)
+        if ((valid >> q) & 1u) {
+            const size_t row = r0 + ia[q], col = c0 + ib[q];
+            const double s = acc[q] * f.inv_n;
+            f.S[row * f.lds + col] = s;
+            f.S[col * f.lds + row] = s;
+        }
+    __syncthreads();
+}
+
+// Blocks of direct_block that hold an entry of the upper triangle: the two halves
+// of each 64 x 64 tile.
+__host__ __device__ inline int direct_blocks(int p) {
+    const int t = (p + 63) / 64;
+    return t * (t + 1);
+}
+
+// All such entries of all fits, their blocks in turn over the grid (each entry is
+// written here only): after the CTA's last tile, when no role waits, since they take n
+// times the epilogue's work.  32 blocks are looked at at once, by every warp alike.
+template <class Src>
+__device__ __forceinline__ void direct_entries(const Src& src, double* sm) {
+    const int lane = threadIdx.x & 31, G = gridDim.x;
+    int first = blockIdx.x;                   // of the fit's blocks, modulo G
+    for (int fi = 0; fi < src.fits(); ++fi) {
+        const F64Fit& f = src.fit_at(fi);
+        if (f.p == 0) continue;
+        const int nm = (f.p + 31) / 32, t = (f.p + 63) / 64, nb = direct_blocks(f.p);
+        bool any = false;
+        for (int i = lane; i < nm; i += 32) any |= f.marks[i] != 0;
+        if (__any_sync(FULL_MASK, any)) {
+            for (int s0 = first; s0 < nb; s0 += 32 * G) {
+                const long long s = s0 + (long long)lane * G;
+                int tm = 0, tn = 0;
+                bool hit = false;
+                if (s < nb) {
+                    upper_tile((int)(s >> 1), t, tm, tn);
+                    const int rb = 2 * tm + (int)(s & 1);
+                    hit = rb < nm && (f.marks[rb] || f.marks[2 * tn] ||
+                                      (2 * tn + 1 < nm && f.marks[2 * tn + 1]));
+                }
+                unsigned left = __ballot_sync(FULL_MASK, hit);
+                for (; left; left &= left - 1u) {
+                    const int l = __ffs(left) - 1;
+                    const int rm = __shfl_sync(FULL_MASK, tm, l), rn = __shfl_sync(FULL_MASK, tn, l);
+                    direct_block(f, 64 * rm + 32 * ((s0 + l * G) & 1), 64 * rn, sm);
                 }
             }
         }
-        __syncthreads();
+        first = (first + G - nb % G) % G;
     }
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-            if ((need >> (4 * u + v)) & 1u) {
-                const size_t row = m0 + r0 + u, col = n0 + c0 + v;
-                const double s = acc[u][v] * f.inv_n;
-                f.S[row * f.lds + col] = s;
-                f.S[col * f.lds + row] = s;
-            }
 }
 
 // W = L_0 256^7 + .. + L_7 from the eight integer-valued level sums: the
@@ -380,6 +431,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
         const int ew = warp - 2;
         const int q = warp & 3, half = ew >> 2;
         double* buf = epi + ew * (F64_EPI_BYTES / 8);     // 32 rows x 16 columns, XOR-swizzled
+        for (int i = 32 * ew + lane; i < src.n_marks(); i += 32 * F64_EPI_WARPS)
+            if (src.marks()[i]) *direct_slot = 1;
         bool ok = true;
         int flush = 0;
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
@@ -428,14 +481,15 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
             // inv_n 2^(E_j - 70); E_k is added to its exponent per column
             const double sj = Ej == F64_EXPO_DIRECT ? f.inv_n : scalbn(f.inv_n, Ej - 70);
             const int my_E = c0 + lane < p ? f.expo[c0 + lane] : 0;
+            // rows and columns of the block that direct_entries forms
+            const unsigned dr = __ballot_sync(FULL_MASK, Ej == F64_EXPO_DIRECT);
+            const unsigned dc = __ballot_sync(FULL_MASK, my_E == F64_EXPO_DIRECT);
+            const unsigned skip = Ej == F64_EXPO_DIRECT ? FULL_MASK : dc;
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
                 const int Ek = __shfl_sync(FULL_MASK, my_E, i);
                 if (!ok) {
                     acc[i] = __longlong_as_double(0x7ff8000000000000ll);
-                } else if (Ej == F64_EXPO_DIRECT || Ek == F64_EXPO_DIRECT) {
-                    acc[i] = 0.0;                         // formed by direct_tile
-                    *direct_slot = 1;
                 } else {
                     acc[i] *= __longlong_as_double(__double_as_longlong(sj) + ((long long)Ek << 52));
                 }
@@ -445,7 +499,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
                     const int col = c0 + i;
-                    if (col < p && col > row) S[(size_t)col * lds + row] = acc[i];
+                    if (col < p && col > row && !((skip >> i) & 1u)) S[(size_t)col * lds + row] = acc[i];
                 }
             }
             // S_jk, two rows of 128 bytes per store, through shared memory
@@ -459,7 +513,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
                 const int col = c0 + h + (lane & 15);
                 for (int jj = 0; jj < 32; jj += 2) {
                     const int j = jj + (lane >> 4), r = m0 + j;
-                    if (r < p && col < p && col >= r)
+                    if (r < p && col < p && col >= r && !((dr >> j) & 1u) &&
+                        !((dc >> (h + (lane & 15))) & 1u))
                         S[(size_t)r * lds + col] = buf[j * F64_EPI_COLS + ((lane & 15) ^ (j & 15))];
                 }
             }
@@ -474,15 +529,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (*direct_slot) {
-        // (the stage buffers are idle, and the CTA's own tiles hold these entries)
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-            const F64Fit& f = src.fit_at(src.fit_index(tile));
-            int tm, tn;
-            f.g.coords(tile - f.tile_start, tm, tn);
-            direct_tile(f, tm, tn, reinterpret_cast<double*>(stages));
-        }
-    }
+    if (*direct_slot) direct_entries(src, reinterpret_cast<double*>(stages));   // (idle by now)
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
@@ -492,9 +539,9 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
 
 __global__ void __launch_bounds__(256) f64_digits_kernel(const double* __restrict__ X, int n, int p,
                                                         int ldx, const double* __restrict__ mu,
-                                                        int* __restrict__ expo,
+                                                        int* __restrict__ expo, int* __restrict__ marks,
                                                         __nv_bfloat16* __restrict__ D, int n_pad) {
-    f64_digit_columns(X, n, p, ldx, mu, expo, D, n_pad, blockIdx.x * 32);
+    f64_digit_columns(X, n, p, ldx, mu, expo, marks + blockIdx.x, D, n_pad, blockIdx.x * 32);
 }
 
 __global__ void f64_mean_kernel(const double* __restrict__ X, int n, int p, int ldx, double* mu) {
@@ -502,7 +549,7 @@ __global__ void f64_mean_kernel(const double* __restrict__ X, int n, int p, int 
 }
 
 template <class Src>
-cudaError_t launch_tiles(const Src& src, int n_tiles, cudaStream_t st) {
+cudaError_t launch_tiles(const Src& src, int n_tiles, int n_blocks, cudaStream_t st) {
     auto kern = gram_f64_kernel<Src>;
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F64_SMEM);
@@ -512,7 +559,9 @@ cudaError_t launch_tiles(const Src& src, int n_tiles, cudaStream_t st) {
         (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return e;
     if (n_tiles <= 0) return cudaSuccess;
-    kern<<<n_tiles < sms ? n_tiles : sms, F64_THREADS, F64_SMEM, st>>>(src);
+    // (a CTA without a tile costs little, and the blocks of direct_entries are more than the tiles)
+    const int grid = n_tiles > n_blocks ? n_tiles : n_blocks;
+    kern<<<grid < sms ? grid : sms, F64_THREADS, F64_SMEM, st>>>(src);
     return cudaGetLastError();
 }
 
@@ -523,7 +572,8 @@ size_t gram_f64_ws_bytes(int n, int p) {
 }
 
 bool f64_encode_fit(F64Fit& f, const double* X, int n, int p, int ldx, const double* mu,
-                    const int* expo, const void* D, double* S, int lds, int tile_start) {
+                    const int* expo, const int* marks, const void* D, double* S, int lds,
+                    int tile_start) {
     f = F64Fit{};
     f.n_pad = tc_pad_n(n);
     const unsigned long long dims[3] = {(unsigned long long)f.n_pad, (unsigned long long)p,
@@ -537,6 +587,7 @@ bool f64_encode_fit(F64Fit& f, const double* X, int n, int p, int ldx, const dou
     f.X = X;
     f.mu = mu;
     f.expo = expo;
+    f.marks = marks;
     f.S = S;
     f.n = n;
     f.p = p;
@@ -555,17 +606,20 @@ cudaError_t launch_gram_f64(const double* X, int n, int p, int ldx, int center, 
     int* expo = reinterpret_cast<int*>(base + align_up((size_t)p * 8, 256));
     __nv_bfloat16* D = reinterpret_cast<__nv_bfloat16*>(base + align_up((size_t)p * 8, 256) +
                                                         f64_expo_bytes(p));
+    int* marks = expo + p;
     F64One one;
-    if (!f64_encode_fit(one.f, X, n, p, ldx, mu, expo, D, S, lds, 0)) return cudaErrorInvalidValue;
+    if (!f64_encode_fit(one.f, X, n, p, ldx, mu, expo, marks, D, S, lds, 0)) return cudaErrorInvalidValue;
     one.n_tiles = one.f.g.count();
     if (center) f64_mean_kernel<<<(p + 31) / 32, dim3(32, MEAN_GROUPS), 0, st>>>(X, n, p, ldx, mu);
-    f64_digits_kernel<<<(p + 31) / 32, dim3(32, 8), 0, st>>>(X, n, p, ldx, mu, expo, D, one.f.n_pad);
-    return launch_tiles(one, one.n_tiles, st);
+    f64_digits_kernel<<<(p + 31) / 32, dim3(32, 8), 0, st>>>(X, n, p, ldx, mu, expo, marks, D,
+                                                            one.f.n_pad);
+    return launch_tiles(one, one.n_tiles, direct_blocks(p), st);
 }
 
-cudaError_t launch_gram_f64_batch(const F64Fit* fits, const int* tile_fit, int n_tiles,
-                                  cudaStream_t st) {
-    return launch_tiles(F64Many{fits, tile_fit, n_tiles}, n_tiles, st);
+int f64_direct_blocks(int p) { return direct_blocks(p); }
+
+cudaError_t launch_gram_f64_batch(const F64Batch& b, cudaStream_t st) {
+    return launch_tiles(F64Many{b}, b.n_tiles, b.n_blocks, st);
 }
 
 }  // namespace spmesl

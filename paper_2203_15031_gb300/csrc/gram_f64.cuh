@@ -24,17 +24,30 @@ struct F64Fit {
     const double* X;
     const double* mu;
     const int* expo;
+    const int* marks;     // per 32 columns whether one of them is F64_EXPO_DIRECT
     double* S;
     int n, p, n_pad, ldx, lds, tile_start;
     double inv_n;
     TileGrid g;
 };
 
-// Bytes of the digit planes and of the exponents (256-byte aligned each).
+// The fits of one launch: device table, tile_start ascending, the fit of each tile,
+// and the marks of all fits in one array.
+struct F64Batch {
+    const F64Fit* fits;
+    const int* tile_fit;
+    const int* marks;
+    int n_fits, n_tiles, n_marks;
+    int n_blocks;         // sum of f64_direct_blocks
+};
+
+// Bytes of the digit planes, and of the exponents followed by the marks (256-byte
+// aligned each).
 inline size_t f64_digit_bytes(int n, int p) {
     return align_up((size_t)F64_SLICES * p * tc_pad_n(n) * 2, 256);
 }
-inline size_t f64_expo_bytes(int p) { return align_up((size_t)p * 4, 256); }
+inline size_t f64_expo_bytes(int p) { return align_up(((size_t)p + (p + 31) / 32) * 4, 256); }
+int f64_direct_blocks(int p);
 
 // x as an integer v = round(x 2^(55 - E)) for |x| < 2^E, and its balanced
 // base-256 digits: v = sum_s d[s] 256^(6 - s), |d[s]| <= 128.
@@ -66,7 +79,7 @@ __device__ __forceinline__ unsigned f64_small(double x, int E) {
 }
 
 // Exponents and digit planes of columns c0 .. c0 + 31 of X, centred by mu when
-// given (block 32 x 8).  The largest magnitude of a column sets its exponent
+// given (block 32 x 8), and the block's mark.  The largest magnitude of a column sets its exponent
 // E (|x| < 2^E); a column with a non-finite value or an exponent beyond
 // F64_EXPO_MAX is marked F64_EXPO_DIRECT and gets zero digits.  So is, by its
 // digits' own pass, a column with more than a quarter of its nonzero samples
@@ -80,7 +93,7 @@ __device__ __forceinline__ unsigned f64_small(double x, int E) {
 // samples loads the next one's (81 -> 78 us for 50 fits of p = 500, n = 250).
 __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, int n, int p,
                                                   int ldx, const double* __restrict__ mu,
-                                                  int* __restrict__ expo,
+                                                  int* __restrict__ expo, int* __restrict__ mark,
                                                   __nv_bfloat16* __restrict__ D, int n_pad, int c0) {
     __shared__ long long red[8][33];
     __shared__ int sE[32];
@@ -158,17 +171,25 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
         }
         __syncthreads();
     }
-    if (tx == 0)
-        for (int r = ty; r < 32; r += 8)
-            if (c0 + r < p && 4ull * small[r] > nonzero[r]) expo[c0 + r] = F64_EXPO_DIRECT;
+    bool direct = false;                  // (lane 0) a column of this warp
+    if (tx == 0) {
+        for (int r = ty; r < 32; r += 8) {
+            if (c0 + r >= p) continue;
+            const bool few = 4ull * small[r] > nonzero[r];
+            if (few) expo[c0 + r] = F64_EXPO_DIRECT;
+            direct |= few || sE[r] == F64_EXPO_DIRECT;
+        }
+    }
+    direct = __syncthreads_or(direct);
+    if (tx == 0 && ty == 0) *mark = direct ? 1 : 0;
 }
 
 // Fill f (host side).  False if the tensor maps could not be encoded.
 bool f64_encode_fit(F64Fit& f, const double* X, int n, int p, int ldx, const double* mu,
-                    const int* expo, const void* D, double* S, int lds, int tile_start);
+                    const int* expo, const int* marks, const void* D, double* S, int lds,
+                    int tile_start);
 
 // One persistent launch over the tiles of a batch (as launch_gram_tc_batch).
-cudaError_t launch_gram_f64_batch(const F64Fit* fits, const int* tile_fit, int n_tiles,
-                                  cudaStream_t st);
+cudaError_t launch_gram_f64_batch(const F64Batch& b, cudaStream_t st);
 
 }  // namespace spmesl

@@ -22,6 +22,7 @@ def _data(n, p, seed):
 @pytest.mark.parametrize("n,p,cols", [
     (1, 1, [0]), (17, 65, [64]), (300, 140, [0, 31, 32, 63, 64, 127, 128, 139]),
     (520, 257, [5, 256]), (600, 1700, [3, 127, 128, 1000, 1699]), (300, 200, list(range(200))),
+    (70, 130, list(range(0, 130, 2))), (65, 96, list(range(40, 90))), (64, 33, [32]), (129, 5000, [2500]),
 ])
 @pytest.mark.parametrize("center", [False, True])
 def test_unscaled_columns(n, p, cols, center):

@@ -194,7 +194,8 @@ double spmesl_lambda(int rule, int n, int p);
  * below its largest, with the error of an FP64 sum over the samples or less relative to
  * sqrt(S_jj S_kk).  Columns with non-finite or extreme values (beyond 2^+-400), and
  * those with more than a quarter of their nonzero samples 2^10 times and more below the
- * largest, are FP64 sums in sample order.  SPMESL_MIXED splits X = hi + lo into two
+ * largest, are FP64 sums in sample order.  The digits take 14 bytes of workspace a sample
+ * and column, of at most 4096 samples.  SPMESL_MIXED splits X = hi + lo into two
  * BF16 parts and forms hi'hi + hi'lo + lo'hi on the tensor cores (tcgen05, TMEM accumulators)
  * with FP32 accumulation.
  * Errors: EINVAL for n < 1, p < 1, ldx < p, lds < p, NULL pointers, a short

@@ -123,13 +123,15 @@ __global__ void batch_split_kernel(const BatchFit* __restrict__ fits,
 // of 32 x 8 per 32 columns.
 __global__ void __launch_bounds__(256) batch_digits_kernel(const BatchFit* __restrict__ fits,
                                                           const int* __restrict__ split_prefix,
-                                                          int count, int* __restrict__ marks) {
+                                                          int count, int* __restrict__ marks, int s0) {
     const int fi = find_fit(split_prefix, count, blockIdx.x);
     const BatchFit& f = fits[fi];
+    if (f.n <= s0) return;
+    int* expo = static_cast<int*>(f.XlT);
     f64_digit_columns(static_cast<const double*>(f.X), f.n, f.p, f.p,
-                      static_cast<const double*>(f.mu), static_cast<int*>(f.XlT),
-                      marks + blockIdx.x, static_cast<__nv_bfloat16*>(f.XhT), tc_pad_n(f.n),
-                      (blockIdx.x - f.split_start) * 32);
+                      static_cast<const double*>(f.mu), expo, marks + blockIdx.x,
+                      f64_counts(expo, f.p), static_cast<__nv_bfloat16*>(f.XhT),
+                      (blockIdx.x - f.split_start) * 32, s0);
 }
 
 template <typename T>
@@ -532,7 +534,7 @@ struct spmesl_batch {
     int total_split = 0;
     // SPMESL_FP64: marks of the columns that the Gram does not scale, and their blocks
     size_t off_marks = 0;
-    int total_direct = 0;
+    int total_direct = 0, max_nx = 1;   // largest n of the fits given as X
     size_t ws_bytes = 0;
     int total_cols = 0, total_gram = 0, total_theta = 0, max_ldp = 32, max_p = 2, max_n = 1;
     bool any_x = false;
@@ -588,14 +590,17 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
                                           b->total_gram, st)) != cudaSuccess)
                 return e;
         } else if constexpr (sizeof(T) == 8) {
-            batch_digits_kernel<<<b->total_split, dim3(32, 8), 0, st>>>(
-                fits, reinterpret_cast<const int*>(ws + b->off_splitp), count,
-                reinterpret_cast<int*>(ws + b->off_marks));
-            const F64Batch g{reinterpret_cast<const F64Fit*>(ws + b->off_tcfit),
-                             reinterpret_cast<const int*>(ws + b->off_tilefit),
-                             reinterpret_cast<const int*>(ws + b->off_marks), count, b->total_gram,
-                             b->total_split, b->total_direct};
-            if ((e = launch_gram_f64_batch(g, st)) != cudaSuccess) return e;
+            for (long long s = 0; s < b->max_nx; s += F64_SLAB) {
+                const int s0 = (int)s;
+                batch_digits_kernel<<<b->total_split, dim3(32, 8), 0, st>>>(
+                    fits, reinterpret_cast<const int*>(ws + b->off_splitp), count,
+                    reinterpret_cast<int*>(ws + b->off_marks), s0);
+                const F64Batch g{reinterpret_cast<const F64Fit*>(ws + b->off_tcfit),
+                                 reinterpret_cast<const int*>(ws + b->off_tilefit),
+                                 reinterpret_cast<const int*>(ws + b->off_marks), count, b->total_gram,
+                                 b->total_split, b->total_direct, s0};
+                if ((e = launch_gram_f64_batch(g, st)) != cudaSuccess) return e;
+            }
         } else {
             batch_gram_kernel<<<b->total_gram, GRAM_THREADS, 0, st>>>(fits, gramp, count);
         }
@@ -927,6 +932,7 @@ spmesl_status spmesl_batch_create(const spmesl_problem* probs, int count, double
                 f.off_XlT = off; off += f64_expo_bytes(f.p);
             }
             b->any_x = true;
+            b->max_nx = std::max(b->max_nx, f.n);
         }
         f.off_SC = off;     off += mat;
         f.off_BT = off;     off += mat;

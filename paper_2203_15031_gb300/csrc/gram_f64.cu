@@ -48,7 +48,8 @@
 // operands longer than for its products); warps 2 to 9
 // combine the levels, 32 rows x 32 columns each, hand the accumulators back,
 // and write the tile and its mirror while the next tile's products run.
-// Waits, failure and tensor-memory release as in gram_tc.cu.
+// Waits, failure and tensor-memory release as in gram_tc.cu.  More than F64_SLAB samples
+// are a pair of launches (digits, products) for each F64_SLAB of them.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -120,7 +121,7 @@ __device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap* map
 
 struct F64One {
     F64Fit f;
-    int n_tiles;
+    int n_tiles, s0;
     static constexpr bool kTableMaps = false;
     __device__ int tiles() const { return n_tiles; }
     __device__ int fits() const { return 1; }
@@ -128,6 +129,7 @@ struct F64One {
     __device__ const F64Fit& fit_at(int) const { return f; }
     __device__ const int* marks() const { return f.marks; }
     __device__ int n_marks() const { return (f.p + 31) / 32; }
+    __device__ int first() const { return s0; }
 };
 
 struct F64Many {
@@ -139,7 +141,15 @@ struct F64Many {
     __device__ const F64Fit& fit_at(int fi) const { return b.fits[fi]; }
     __device__ const int* marks() const { return b.marks; }
     __device__ int n_marks() const { return b.n_marks; }
+    __device__ int first() const { return b.s0; }
 };
+
+// K blocks of a fit in the slab that starts at sample s0 (0 or less: it has none), and
+// whether it is the fit's last.
+__device__ __forceinline__ int slab_blocks(const F64Fit& f, int s0) {
+    return min(tc_pad_n(f.n) - s0, F64_SLAB) / F64_KB;
+}
+__device__ __forceinline__ bool last_slab(const F64Fit& f, int s0) { return f.n - s0 <= F64_SLAB; }
 
 // The entries of rows r0 .. r0 + 31 and columns c0 .. c0 + 63 whose row or column is
 // not scaled (F64_EXPO_DIRECT): FP64 sums in sample order.  Bound by the FP64 pipe
@@ -235,7 +245,7 @@ __device__ __forceinline__ void direct_entries(const Src& src, double* sm) {
     int first = blockIdx.x;                   // of the fit's blocks, modulo G
     for (int fi = 0; fi < src.fits(); ++fi) {
         const F64Fit& f = src.fit_at(fi);
-        if (f.p == 0) continue;
+        if (f.p == 0 || f.n <= src.first() || !last_slab(f, src.first())) continue;
         const int nm = (f.p + 31) / 32, t = (f.p + 63) / 64, nb = direct_blocks(f.p);
         bool any = false;
         for (int i = lane; i < nm; i += 32) any |= f.marks[i] != 0;
@@ -297,7 +307,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
     volatile int* kt_ring = fail + 4;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tiles = src.tiles();
+    const int n_tiles = src.tiles(), s0 = src.first();
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < F64_STAGES; ++s) {
@@ -329,11 +339,12 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
             // producer
             int kb = 0, li = 0;
             const F64Fit* last = nullptr;
-            for (int tile = blockIdx.x; tile < n_tiles && !*fail; tile += gridDim.x, ++li) {
+            for (int tile = blockIdx.x; tile < n_tiles && !*fail; tile += gridDim.x) {
                 const F64Fit& f = src.fit_at(src.fit_index(tile));
+                const int KT = slab_blocks(f, s0);
+                if (KT <= 0) continue;              // a shorter fit of the batch
                 int tm, tn;
                 f.g.coords(tile - f.tile_start, tm, tn);
-                const int KT = f.n_pad / F64_KB;
                 kt_ring[li % F64_RING] = KT;        // published by the first expect_tx below
                 if (Src::kTableMaps && &f != last) {
                     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
@@ -359,6 +370,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
                                 tn * F64_BN, 0, fb);
                     *issued_slot = kb + 1;
                 }
+                ++li;
             }
         }
     } else if (warp == 1) {
@@ -366,7 +378,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
             // MMA issuer
             int kb = 0, li = 0, flush = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++li) {
+            for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+                if (s0 != 0 && slab_blocks(src.fit_at(src.fit_index(tile)), s0) <= 0) continue;
                 int KT = 1;                          // read once the first K block has landed
                 for (int kt = 0; kt < KT; ++kt, ++kb) {
                     const bool first = kt % (F64_FLUSH / F64_KB) == 0;
@@ -420,6 +433,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
                         ++flush;
                     }
                 }
+                ++li;
             }
             if (!ok) *fail = 1;
             mma_commit(smem_u32(done));
@@ -437,6 +451,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
         int flush = 0;
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
             const F64Fit& f = src.fit_at(src.fit_index(tile));
+            const int KT = slab_blocks(f, s0);
+            if (KT <= 0) continue;
             int tm, tn;
             f.g.coords(tile - f.tile_start, tm, tn);
             const int m0 = tm * TC_BM + 32 * q, c0 = tn * F64_BN + 32 * half;
@@ -444,7 +460,16 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
             // warp-uniform: this warp's 32 x 32 block holds an entry to write
             const bool any = m0 < p && c0 < p && c0 + 31 >= m0;
             double acc[32];
-            const int nf = (f.n_pad + F64_FLUSH - 1) / F64_FLUSH;
+            double* __restrict__ S = f.S;
+            const int row = m0 + lane;
+            if (s0 != 0 && any) {                         // the slabs before this one
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    const int col = c0 + i;
+                    acc[i] = (col < p && col >= row) ? S[(size_t)col * lds + row] : 0.0;
+                }
+            }
+            const int nf = (KT * F64_KB + F64_FLUSH - 1) / F64_FLUSH;
             for (int fl = 0; fl < nf; ++fl, ++flush) {
                 if (ok) {
                     int got = 0;
@@ -466,7 +491,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const double w = combine_levels(L, i);
-                            acc[c + i] = fl == 0 ? w : acc[c + i] + w;
+                            acc[c + i] = (fl == 0 && s0 == 0) ? w : acc[c + i] + w;
                         }
                     }
                 }
@@ -475,8 +500,15 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
                 if (lane == 0) mbar_arrive(smem_u32(acc_empty));
             }
             if (!any) continue;
-            double* __restrict__ S = f.S;
-            const int row = m0 + lane;
+            if (!last_slab(f, s0)) {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    const int col = c0 + i;
+                    if (col < p && col >= row)
+                        S[(size_t)col * lds + row] = ok ? acc[i] : __longlong_as_double(0x7ff8000000000000ll);
+                }
+                continue;
+            }
             const int Ej = row < p ? f.expo[row] : 0;
             // inv_n 2^(E_j - 70); E_k is added to its exponent per column
             const double sj = Ej == F64_EXPO_DIRECT ? f.inv_n : scalbn(f.inv_n, Ej - 70);
@@ -540,8 +572,9 @@ __global__ void __launch_bounds__(F64_THREADS, 1) gram_f64_kernel(const __grid_c
 __global__ void __launch_bounds__(256) f64_digits_kernel(const double* __restrict__ X, int n, int p,
                                                         int ldx, const double* __restrict__ mu,
                                                         int* __restrict__ expo, int* __restrict__ marks,
-                                                        __nv_bfloat16* __restrict__ D, int n_pad) {
-    f64_digit_columns(X, n, p, ldx, mu, expo, marks + blockIdx.x, D, n_pad, blockIdx.x * 32);
+                                                        __nv_bfloat16* __restrict__ D, int s0) {
+    f64_digit_columns(X, n, p, ldx, mu, expo, marks + blockIdx.x, f64_counts(expo, p), D,
+                      blockIdx.x * 32, s0);
 }
 
 __global__ void f64_mean_kernel(const double* __restrict__ X, int n, int p, int ldx, double* mu) {
@@ -575,11 +608,9 @@ bool f64_encode_fit(F64Fit& f, const double* X, int n, int p, int ldx, const dou
                     const int* expo, const int* marks, const void* D, double* S, int lds,
                     int tile_start) {
     f = F64Fit{};
-    f.n_pad = tc_pad_n(n);
-    const unsigned long long dims[3] = {(unsigned long long)f.n_pad, (unsigned long long)p,
-                                        (unsigned long long)F64_SLICES};
-    const unsigned long long strides[2] = {(unsigned long long)f.n_pad * 2,
-                                           (unsigned long long)f.n_pad * 2 * p};
+    const unsigned long long ldd = f64_plane_n(n);
+    const unsigned long long dims[3] = {ldd, (unsigned long long)p, (unsigned long long)F64_SLICES};
+    const unsigned long long strides[2] = {ldd * 2, ldd * 2 * p};
     const unsigned box_a[3] = {F64_KB, TC_BM, F64_SLICES}, box_b[3] = {F64_KB, F64_BN, F64_SLICES};
     if (!tc_encode_bf16_3d(f.ma, D, dims, strides, box_a) ||
         !tc_encode_bf16_3d(f.mb, D, dims, strides, box_b))
@@ -611,9 +642,13 @@ cudaError_t launch_gram_f64(const double* X, int n, int p, int ldx, int center, 
     if (!f64_encode_fit(one.f, X, n, p, ldx, mu, expo, marks, D, S, lds, 0)) return cudaErrorInvalidValue;
     one.n_tiles = one.f.g.count();
     if (center) f64_mean_kernel<<<(p + 31) / 32, dim3(32, MEAN_GROUPS), 0, st>>>(X, n, p, ldx, mu);
-    f64_digits_kernel<<<(p + 31) / 32, dim3(32, 8), 0, st>>>(X, n, p, ldx, mu, expo, marks, D,
-                                                            one.f.n_pad);
-    return launch_tiles(one, one.n_tiles, direct_blocks(p), st);
+    for (long long s0 = 0; s0 < n; s0 += F64_SLAB) {
+        one.s0 = (int)s0;
+        f64_digits_kernel<<<(p + 31) / 32, dim3(32, 8), 0, st>>>(X, n, p, ldx, mu, expo, marks, D, one.s0);
+        const cudaError_t e = launch_tiles(one, one.n_tiles, direct_blocks(p), st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 int f64_direct_blocks(int p) { return direct_blocks(p); }

@@ -13,11 +13,20 @@ namespace spmesl {
 
 constexpr int F64_SLICES = 7;         // 8-bit digits of a column's scaled values
 constexpr int F64_LEVELS = 8;         // sums of digit products by weight (see gram_f64.cu)
+constexpr int F64_SLAB = 4096;        // samples whose digits are held at a time
 constexpr int F64_BN = 64;            // output tile: TC_BM rows x F64_BN columns
 constexpr int F64_EXPO_DIRECT = INT_MAX;   // column whose products are formed directly in FP64
 constexpr int F64_EXPO_MAX = 400;     // largest |exponent| that the digits' scaling handles
 
-// One fit: TMA maps over its digit planes D ([F64_SLICES][p][n_pad] bf16; boxes
+// Samples of a digit plane's row.  The planes take 14 bytes a sample, 1.75 times X:
+// data of more than F64_SLAB samples go through them in slabs, with the sums of the
+// digit products kept in S's lower triangle between two.
+__host__ __device__ inline int f64_plane_n(int n) {
+    return tc_pad_n(n) < F64_SLAB ? tc_pad_n(n) : F64_SLAB;
+}
+static_assert(F64_SLAB % TC_NPAD == 0, "slabs");
+
+// One fit: TMA maps over its digit planes D ([F64_SLICES][p][f64_plane_n] bf16; boxes
 // of 128 and 64 columns of X), the columns' exponents, the data and the output.
 struct F64Fit {
     CUtensorMap ma, mb;
@@ -26,7 +35,7 @@ struct F64Fit {
     const int* expo;
     const int* marks;     // per 32 columns whether one of them is F64_EXPO_DIRECT
     double* S;
-    int n, p, n_pad, ldx, lds, tile_start;
+    int n, p, ldx, lds, tile_start;
     double inv_n;
     TileGrid g;
 };
@@ -39,14 +48,20 @@ struct F64Batch {
     const int* marks;
     int n_fits, n_tiles, n_marks;
     int n_blocks;         // sum of f64_direct_blocks
+    int s0;               // first sample of the slab
 };
 
-// Bytes of the digit planes, and of the exponents followed by the marks (256-byte
-// aligned each).
-inline size_t f64_digit_bytes(int n, int p) {
-    return align_up((size_t)F64_SLICES * p * tc_pad_n(n) * 2, 256);
+// The counts behind the exponents.
+__host__ __device__ inline unsigned* f64_counts(int* expo, int p) {
+    return reinterpret_cast<unsigned*>(expo + p + (p + 31) / 32);
 }
-inline size_t f64_expo_bytes(int p) { return align_up(((size_t)p + (p + 31) / 32) * 4, 256); }
+
+// Bytes of the digit planes, and of the exponents followed by the marks and, per column,
+// the two counts of the rule on small samples (256-byte aligned each).
+inline size_t f64_digit_bytes(int n, int p) {
+    return align_up((size_t)F64_SLICES * p * f64_plane_n(n) * 2, 256);
+}
+inline size_t f64_expo_bytes(int p) { return align_up((3 * (size_t)p + (p + 31) / 32) * 4, 256); }
 int f64_direct_blocks(int p);
 
 // x as an integer v = round(x 2^(55 - E)) for |x| < 2^E, and its balanced
@@ -89,12 +104,15 @@ __device__ __forceinline__ unsigned f64_small(double x, int E) {
 // log-normal (s = 3) and Cauchy columns and a column of ordinary samples with one of
 // 10^3 or more are marked.  Magnitudes are
 // compared and digits formed on the integer pipe: the FP64 pipe takes 16 cycles
-// an instruction.  Samples n .. n_pad - 1 are written as zeros.  Each pass of 64
+// an instruction.  Samples from n to the next multiple of 64 are written as zeros.  Each pass of 64
 // samples loads the next one's (81 -> 78 us for 50 fits of p = 500, n = 250).
+// One slab of samples a call, s0 its first; the first one forms the exponents of all, the
+// last one the marks.
 __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, int n, int p,
                                                   int ldx, const double* __restrict__ mu,
                                                   int* __restrict__ expo, int* __restrict__ mark,
-                                                  __nv_bfloat16* __restrict__ D, int n_pad, int c0) {
+                                                  unsigned* __restrict__ counts,
+                                                  __nv_bfloat16* __restrict__ D, int c0, int s0) {
     __shared__ long long red[8][33];
     __shared__ int sE[32];
     __shared__ unsigned nonzero[32], small[32];        // samples of each column (by its warp)
@@ -103,7 +121,7 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
     const int cl = c0 + tx;
     const double m = (mu && cl < p) ? mu[cl] : 0.0;
     long long mx = 0;
-    if (cl < p) {
+    if (cl < p && s0 == 0) {
 #pragma unroll 8
         for (int i = ty; i < n; i += 8) {
             double v = X[(size_t)i * ldx + cl];
@@ -119,12 +137,14 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
         const int e = (int)(mx >> 52);
         int E = mx == 0 ? 0 : e - 1022;
         if (e == 0x7ff || E > F64_EXPO_MAX || E < -F64_EXPO_MAX) E = F64_EXPO_DIRECT;
+        if (s0 != 0) E = cl < p ? expo[cl] : 0;
         sE[tx] = E;
         nonzero[tx] = small[tx] = 0u;
         if (cl < p) expo[cl] = E;
     }
     __syncthreads();
-    const size_t plane = (size_t)p * n_pad;
+    const int ldd = f64_plane_n(n), end = s0 + min(tc_pad_n(n) - s0, F64_SLAB);
+    const size_t plane = (size_t)p * ldd;
     double nx[8];                         // the next 64 samples, on their way during the digits
     auto fetch = [&](int i0) {
 #pragma unroll
@@ -133,12 +153,12 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
             nx[r] = (i < n && cl < p) ? X[(size_t)i * ldx + cl] : m;
         }
     };
-    fetch(0);
-    for (int i0 = 0; i0 < n_pad; i0 += 64) {
+    fetch(s0);
+    for (int i0 = s0; i0 < end; i0 += 64) {
 #pragma unroll
         for (int r = 0; r < 8; ++r) tile[tx][ty + 8 * r] = mu ? nx[r] - m : nx[r];
         __syncthreads();
-        if (i0 + 64 < n_pad) fetch(i0 + 64);
+        if (i0 + 64 < end) fetch(i0 + 64);
         for (int r = ty; r < 32; r += 8) {
             const int c = c0 + r;
             if (c < p) {
@@ -157,7 +177,7 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
                         small[r] += few >> 16;
                     }
                 }
-                __nv_bfloat16* out = D + (size_t)c * n_pad + i0 + 2 * tx;
+                __nv_bfloat16* out = D + (size_t)c * ldd + (i0 - s0) + 2 * tx;
 #pragma unroll
                 for (int s = 0; s < F64_SLICES; ++s) {
                     // |d| <= 128 is exact in bf16: the upper half of its FP32 bits
@@ -175,6 +195,15 @@ __device__ __forceinline__ void f64_digit_columns(const double* __restrict__ X, 
     if (tx == 0) {
         for (int r = ty; r < 32; r += 8) {
             if (c0 + r >= p) continue;
+            if (s0 != 0) {
+                nonzero[r] += counts[2 * (c0 + r)];
+                small[r] += counts[2 * (c0 + r) + 1];
+            }
+            if (end < n) {
+                counts[2 * (c0 + r)] = nonzero[r];
+                counts[2 * (c0 + r) + 1] = small[r];
+                continue;
+            }
             const bool few = 4ull * small[r] > nonzero[r];
             if (few) expo[c0 + r] = F64_EXPO_DIRECT;
             direct |= few || sE[r] == F64_EXPO_DIRECT;

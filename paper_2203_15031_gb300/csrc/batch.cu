@@ -1,5 +1,5 @@
 // Batched SPMESL: many independent fits of different p and n in one pass of
-// four launches (Gram tiles, standardisation, coordinate descent, Theta).
+// launches over all of them (Gram, standardisation, column order, coordinate descent, Theta).
 // With SPMESL_MIXED the Gram of every fit given as X runs as split-BF16
 // products on the tensor cores (one batched split/transpose launch, then one
 // persistent tcgen05 launch over the tiles of all fits); the rest runs in
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(32 * PREP_ROWS) batch_prep_matrix_kernel(
     int cnt = 0;
     float top = 0.f;
     const bool bad = standardize_row<T>(static_cast<const T*>(f.S), f.p, f.ldp, r, f.cs, f.csf,
-                                        static_cast<T*>(f.SC), nullptr, nullptr,
+                                        static_cast<T*>(f.SC), nullptr,
                                         static_cast<T*>(f.diag), lane, 32, (T)f.lambda0,
                                         heat ? &cnt : nullptr, f.cmax, &top);
     if (f.cmax && lane == 0) static_cast<T*>(f.diag)[r] = (T)top;
@@ -272,33 +272,22 @@ __global__ void batch_rows_count_kernel(const BatchFit* __restrict__ fits) {
         count_rows_moved(f.rows, rows_bitmap_bytes(f.p) / 4, f.ctrl, threadIdx.x, blockDim.x);
 }
 
-// Eager gradient over all columns of all fits, or (from_queue) over the
-// global columns the lazy kernel handed over.
+// Eager gradient over all columns of all fits.
 template <typename T, bool STD>
 __global__ void __launch_bounds__(512) batch_cd_kernel(const BatchFit* __restrict__ fits,
                                                        const int* __restrict__ col_prefix,
                                                        int count, int total_cols, int max_ldp,
                                                        double tol, float tolf, int maxit,
-                                                       BatchHeader* hdr, const int* ovf_list,
-                                                       int from_queue) {
+                                                       BatchHeader* hdr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     T* g = reinterpret_cast<T*>(smem_raw + (size_t)warp * warp_smem_bytes<T>(max_ldp));
-    const int nq = from_queue ? *reinterpret_cast<volatile int*>(&hdr->ovf_count) : 0;
     for (;;) {
         int gc = 0;
-        if (from_queue) {
-            int t = 0;
-            if (lane == 0) t = atomicAdd(&hdr->ovf_next, 1);
-            t = __shfl_sync(FULL_MASK, t, 0);
-            if (t >= nq) break;
-            gc = ovf_list[t];
-        } else {
-            if (lane == 0) gc = atomicAdd(&hdr->next_col, 1);
-            gc = __shfl_sync(FULL_MASK, gc, 0);
-            if (gc >= total_cols) break;
-        }
+        if (lane == 0) gc = atomicAdd(&hdr->next_col, 1);
+        gc = __shfl_sync(FULL_MASK, gc, 0);
+        if (gc >= total_cols) break;
         const int fi = find_fit(col_prefix, count, gc);
         const BatchFit& f = fits[fi];
         if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) continue;
@@ -696,7 +685,7 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
         per_sm = std::max(per_sm, 1);
         const int grid = std::min((b->total_cols + EW - 1) / EW, num_sms() * per_sm);
         kern<<<grid, 32 * EW, smem, st>>>(fits, colp, count, b->total_cols, b->max_ldp, b->tol, tolf,
-                                          b->maxit, hdr, ovf, 0);
+                                          b->maxit, hdr);
     }
     if (timed) cudaEventRecord(b->ev[1], st);
     if (b->count_rows) batch_rows_count_kernel<<<count, 256, 0, st>>>(fits);

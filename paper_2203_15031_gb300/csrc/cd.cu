@@ -30,10 +30,9 @@ namespace spmesl {
 // Per-column rule (Algorithms 1-2): every warp takes the next unsolved column
 // and runs the whole scaled lasso for it; no grid-wide synchronisation.
 // ---------------------------------------------------------------------------
-// Eager gradient (g_j and b_j in shared memory).  With from_queue the warps
-// take the columns the lazy solver handed over instead of 0..p-1.
+// Eager gradient (g_j and b_j in shared memory).
 template <typename T, bool STD>
-__global__ void __launch_bounds__(512) cd_column_kernel(CDArgs<T> a, int from_queue) {
+__global__ void __launch_bounds__(512) cd_column_kernel(CDArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -42,21 +41,12 @@ __global__ void __launch_bounds__(512) cd_column_kernel(CDArgs<T> a, int from_qu
     int* list = reinterpret_cast<int*>(b + a.ldp);
     FitCtrl* ctrl = a.ctrl;
     if (*reinterpret_cast<volatile int*>(&ctrl->err) != 0) return;
-    const int nq = from_queue ? *reinterpret_cast<volatile int*>(a.ovf_count) : 0;
     ColCounters cnt;
     for (;;) {
         int j = 0;
-        if (from_queue) {
-            int t = 0;
-            if (lane == 0) t = atomicAdd(&ctrl->ovf_next, 1);
-            t = __shfl_sync(FULL_MASK, t, 0);
-            if (t >= nq) break;
-            j = a.ovf_list[t];
-        } else {
-            if (lane == 0) j = atomicAdd(&ctrl->next_col, 1);
-            j = __shfl_sync(FULL_MASK, j, 0);
-            if (j >= a.p) break;
-        }
+        if (lane == 0) j = atomicAdd(&ctrl->next_col, 1);
+        j = __shfl_sync(FULL_MASK, j, 0);
+        if (j >= a.p) break;
         solve_column<T, STD>(j, g, b, list, a, cnt);
     }
     flush_counters(ctrl, cnt);
@@ -378,7 +368,7 @@ __global__ void prep_matrix_kernel(const T* __restrict__ S, int p, int ldp, cons
     for (int r = blockIdx.x; r < p; r += gridDim.x) {
         int cnt = 0;
         float m = 0.f;
-        bad |= standardize_row<T>(S, p, ldp, r, cs, csf, SC, init_g ? GT : nullptr, nullptr,
+        bad |= standardize_row<T>(S, p, ldp, r, cs, csf, SC, init_g ? GT : nullptr,
                                   diag, threadIdx.x, blockDim.x, heat_lam, heat ? &cnt : nullptr,
                                   cmax, &m);
         if (cnt) atomicAdd(&heat[r], cnt);
@@ -755,7 +745,7 @@ static cudaError_t run_fit(const FitLaunch& f, const FitLayout& L, cudaStream_t 
                 return e;
             per_sm = auto_shape ? 1 : std::max(per_sm, 1);
             const int grid = std::min((f.p + W - 1) / W, g_num_sms * per_sm);
-            kern<<<grid, threads, smem, st>>>(a, 0);
+            kern<<<grid, threads, smem, st>>>(a);
         }
     } else {
         auto kern = cd_joint_kernel<T, STD>;

@@ -25,7 +25,7 @@ struct CDArgs {
     int p, ldp, maxit;
     double lambda0, tol;
     float tolf;          // the smallest float not below tol (see float_at_least)
-    int* ovf_list;       // columns handed from the lazy solver to the block (or eager) solver
+    int* ovf_list;       // columns handed from the lazy solver to the block solver
     int* ovf_count;
     const int* order;    // queue order of the lazy solver (nullptr: 0..p-1)
     int n_queue;         // columns the lazy solver takes from its queue
@@ -389,12 +389,6 @@ __device__ __forceinline__ bool chunk_skippable(const ChunkInfo& c, const ColSca
     return bound < lam;
 }
 
-__device__ __forceinline__ float warp_sum_f(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL_MASK, v, o);
-    return v;
-}
-
 // An upper bound of the warp's sum of |x| (one hardware reduction): each |x|
 // rounded up to a multiple of 2^-20; infinite when the sum reaches 64.
 __device__ __forceinline__ float warp_l1_bound(float x) {
@@ -586,7 +580,7 @@ __device__ double residual_quadratic_form(int j, const T* __restrict__ b, const 
 }
 
 // Row r of S^C = C S C into SC (zero padding up to ldp), optionally copied
-// into GT, with BT's row cleared.  FP32 data is scaled in FP32 by the scales
+// into GT.  FP32 data is scaled in FP32 by the scales
 // rounded once to FP32 (csf); FP64 data in FP64.  One warp takes one
 // 128-coordinate chunk of the row at a time (threads tid, tid + nthr, ...;
 // nthr a multiple of 32).  Optional outputs: heat, this thread's count of
@@ -605,7 +599,7 @@ __device__ __forceinline__ bool standardize_row(const T* __restrict__ S, int p, 
                                                 const double* __restrict__ cs,
                                                 const float* __restrict__ csf,
                                                 T* __restrict__ SC, T* __restrict__ GT,
-                                                T* __restrict__ BT, T* __restrict__ diag, int tid,
+                                                T* __restrict__ diag, int tid,
                                                 int nthr, T heat_lam = T(0), int* heat = nullptr,
                                                 float* __restrict__ cmax = nullptr,
                                                 float* rowmax = nullptr) {
@@ -616,7 +610,6 @@ __device__ __forceinline__ bool standardize_row(const T* __restrict__ S, int p, 
     const T* __restrict__ srow = S + (size_t)r * p;
     T* __restrict__ out = SC + (size_t)r * ldp;
     T* __restrict__ grow = GT ? GT + (size_t)r * ldp : nullptr;
-    T* __restrict__ brow = BT ? BT + (size_t)r * ldp : nullptr;
     const int nch = num_chunks(ldp);
     const int wstep = nthr >> 5;
     // 16-byte accesses when the rows of S are 16-byte aligned (same arithmetic)
@@ -676,7 +669,6 @@ __device__ __forceinline__ bool standardize_row(const T* __restrict__ S, int p, 
                     const float4 q = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
                     *reinterpret_cast<float4*>(out + c) = q;
                     if (grow) *reinterpret_cast<float4*>(grow + c) = q;
-                    if (brow) *reinterpret_cast<float4*>(brow + c) = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             } else {
 #pragma unroll
@@ -685,7 +677,6 @@ __device__ __forceinline__ bool standardize_row(const T* __restrict__ S, int p, 
                     if (c < ldp) {
                         out[c] = v[t];
                         if (grow) grow[c] = v[t];
-                        if (brow) brow[c] = T(0);
                     }
                 }
             }
@@ -845,7 +836,7 @@ __device__ void solve_column(int j, T* __restrict__ g, T* __restrict__ b, int* _
 // g -= S_.k delta is applied at once to the rest of the chunk and reaches
 // every later chunk when that chunk forms its slice from the updated support.
 // This is the covariance form of c = S_kj - sum_{l != k} S_kl b_l.  With about
-// 5 KB of shared memory per column instead of two p-vectors, many more columns
+// 7 KB of shared memory per column instead of two p-vectors, many more columns
 // stay resident per SM.
 // If the support outgrows the phase or the list, the column is handed to the
 // block solver (solve_column_block) through a queue.
@@ -1517,7 +1508,7 @@ __device__ __forceinline__ void store_solved_lazy(int j, const Support<T>& s, co
 // block solver continues from this iterate.  Any (b, sigma) is a valid start
 // for the coordinate descent, and the hand-over point depends only on the
 // column's data, so the result is the same wherever the column is solved.
-template <typename T, bool HS>
+template <typename T>
 __device__ __forceinline__ void hand_over_lazy(int j, const Support<T>& s, const CDArgs<T>& a, double sigma,
                                double s_prev, double f_prev, int r, int status) {
     if (!a.hand) return;
@@ -1534,8 +1525,8 @@ __device__ __forceinline__ void hand_over_lazy(int j, const Support<T>& s, const
 }
 
 // Algorithm 1 for column j with the lazy gradient.  Returns false when the
-// support outgrew the list (nothing written; the caller queues the column
-// for the eager solver).  HS keeps the last sigma step in the warp's shared
+// support outgrew the phase or the list (its state is handed over; the caller queues
+// the column for the block solver).  HS keeps the last sigma step in the warp's shared
 // memory instead of registers (for kernels at a tight register cap).
 template <typename T, bool STD, bool HS = false, int U = 2, int SCAN_G = scan_group<T>()>
 __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a, ColCounters& cnt) {
@@ -1601,7 +1592,7 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
             }
         }
         if (overflow) {
-            hand_over_lazy<T, HS>(j, s, a, sigma, HS ? prev[0] : s_prev, HS ? prev[1] : f_prev, r,
+            hand_over_lazy<T>(j, s, a, sigma, HS ? prev[0] : s_prev, HS ? prev[1] : f_prev, r,
                                   status);
             return false;
         }

@@ -307,14 +307,18 @@ constexpr int PREFIX_SMEM = 1024;
 // belong to it from the start.
 // At most 8 warps a block; MINB blocks an SM.  Three (80 registers) carry most
 // columns a second; two (128 registers) solve one column sooner, with more of its
-// loads in flight and no spills, which decides while the longest columns do:
-// up to LAZY_WIDE_COLS columns per resident warp of the two-block form (20:
-// 48640 columns on 152 SMs), and in FP64, where 80 registers spill most.
-// 256 fits (133 k columns) 2.04 ms with three, 2.18 with two; 128 (62 k) 1.30
-// and 1.17; 96 (44 k) 1.17 and 1.03; ten p = 2000 fits (20 k) 0.42 and 0.38, twenty
-// (40 k) 0.64 and 0.68, forty (80 k) 1.24 and 1.32; FP64 study (25 k) 1.33 and 1.26.
+// loads in flight and no spills, which decides while the longest columns do, and in FP64,
+// where 80 registers spill most.  How long that is depends on the networks too; by
+// sizes, a batch of unlike fits, whose longest columns are longer than the mean, has
+// two up to LAZY_WIDE_MIXED columns per resident warp of that form (45: 109440 on 152
+// SMs), one of like fits up to LAZY_WIDE_COLS (14: 34048).  A whole pass in ms, two and three:
+// fits of p 50 to 2000, 128 (62 k columns) 1.03 and 1.20, 200 (98 k) 1.41 and 1.47, 256
+// (133 k) 1.90 and 1.81; Erdos-Renyi p = 2000, 14 fits (28 k) 0.466 and 0.505, 20 (40 k)
+// 0.629 and 0.614, 40 (80 k) 1.21 and 1.15; p = 500, 80 (40 k) 0.457 and 0.441.  Left on the
+// slower side: AR(1) p = 2000, 10 fits (20 k) 0.491 and 0.468; p = 4000, 12 (48 k) 1.05
+// and 1.09.
 constexpr int LAZY_MAX_WARPS = 8;
-constexpr int LAZY_WIDE_COLS = 20;
+constexpr int LAZY_WIDE_COLS = 14, LAZY_WIDE_MIXED = 45;
 template <typename T, bool STD, int MINB>
 __global__ void __launch_bounds__(32 * LAZY_MAX_WARPS, MINB) batch_cd_lazy_kernel(const BatchFit* __restrict__ fits,
                                                             const int* __restrict__ col_prefix,
@@ -548,6 +552,14 @@ struct spmesl_batch {
 
 namespace {
 
+// Columns per resident warp up to which the lazy kernel runs two blocks an SM: the fits are
+// unlike when the largest has 1.5 times the chunks of the mean column's.
+int lazy_wide_cols(const spmesl_batch* b) {
+    long long chunks = 0;
+    for (const FitPlan& f : b->plan) chunks += (long long)f.p * row_chunks(f.ldp);
+    return 2ll * row_chunks(b->max_ldp) * b->total_cols >= 3 * chunks ? LAZY_WIDE_MIXED : LAZY_WIDE_COLS;
+}
+
 template <typename T>
 cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, int W) {
     const BatchFit* fits = reinterpret_cast<const BatchFit*>(ws + b->off_desc);
@@ -650,7 +662,7 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
         const size_t lsm = lper * LW;
         auto lk = b->standardize ? batch_cd_lazy_kernel<T, true, 2> : batch_cd_lazy_kernel<T, false, 2>;
         if constexpr (sizeof(T) == 4)
-            if (b->total_cols > LAZY_WIDE_COLS * num_sms() * 2 * LAZY_MAX_WARPS)
+            if (b->total_cols > lazy_wide_cols(b) * num_sms() * 2 * LAZY_MAX_WARPS)
                 lk = b->standardize ? batch_cd_lazy_kernel<T, true, 3> : batch_cd_lazy_kernel<T, false, 3>;
         if ((e = cudaFuncSetAttribute(lk, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)lsm)) != cudaSuccess)

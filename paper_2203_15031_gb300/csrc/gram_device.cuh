@@ -31,7 +31,8 @@ constexpr int GRAM_BM = 64;             // tile of small fits and batches
 constexpr int GRAM_THREADS = 128;
 constexpr int GRAM_WIDE = 128;          // tile of large fits
 constexpr int GRAM_WIDE_THREADS = 128;
-constexpr int GRAM_WIDE_TILES = 250;    // 128 x 128 tiles from which they are taken
+constexpr int GRAM_WIDE_TILES = 250;    // 128 x 128 tiles from which they are taken (152 SMs, two a
+                                        // SM: four fifths of a wave)
 constexpr int GRAM_BK = 16;             // rows of X per stage
 constexpr int GRAM_WIDE_BK = 8;         // (the prefetch shares the registers with 128 entries)
 

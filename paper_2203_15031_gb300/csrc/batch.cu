@@ -422,14 +422,15 @@ __global__ void batch_theta_kernel(const BatchFit* __restrict__ fits,
                   f.ctrl, blockIdx.x - f.theta_start);
 }
 
-// 1 / sigma_j^2 of every column, one per lane: an FP64 division takes a warp
-// some 250 cycles of the FP64 pipe whatever its active lanes, so the lists'
-// pass below reads it.
+// The last step of sigma_j's square root (sqrt_last) and 1 / sigma_j^2 of every column, one
+// per lane: an FP64 division takes a warp some 250 cycles of the FP64 pipe whatever its
+// active lanes, so the lists' pass below reads it.
 __global__ void __launch_bounds__(256) batch_inv_kernel(const BatchFit* __restrict__ fits) {
     const BatchFit& f = fits[blockIdx.y];
     if (*reinterpret_cast<volatile int*>(&f.ctrl->err) != 0) return;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < f.p; j += gridDim.x * blockDim.x) {
-        const double s = f.sigma[j];
+        const double s = sqrt_last(f.hand[2 * (size_t)j + 1], f.sigma[j]);
+        f.sigma[j] = s;
         f.hand[2 * (size_t)j] = 1.0 / (s * s);
     }
 }
@@ -701,12 +702,12 @@ cudaError_t enqueue_batch(spmesl_batch* b, unsigned char* ws, cudaStream_t st, i
     }
     if (timed) cudaEventRecord(b->ev[1], st);
     if (b->count_rows) batch_rows_count_kernel<<<count, 256, 0, st>>>(fits);
+    if (lazy) batch_inv_kernel<<<dim3((b->max_p + 255) / 256, count), 256, 0, st>>>(fits);
     if (b->diagnostics) {
         const int dgrid = std::max(1, std::min(b->total_cols, num_sms() * 16));
         batch_diag_kernel<T><<<dgrid, 32 * DIAG_WARPS, 0, st>>>(fits, colp, count, b->total_cols);
     }
     if (lazy) {
-        batch_inv_kernel<<<dim3((b->max_p + 255) / 256, count), 256, 0, st>>>(fits);
         batch_theta_list_kernel<T><<<b->total_theta, 256, 0, st>>>(fits, thetap, count);
     } else {
         batch_theta_kernel<T><<<b->total_theta, dim3(32, 8), 0, st>>>(fits, thetap, count);

@@ -40,7 +40,8 @@ struct CDArgs {
     int rows_words;           // 32-bit words per row of that bitmap
     double* hand;             // per column the last sigma step (sigma, F(sigma)) at a hand-over
                               // from the lazy to the block solver (nullptr: the block solver
-                              // starts every column afresh)
+                              // starts every column afresh); of a batch's solved column the
+                              // second is sigma^2, for sqrt_last
     int* nsup;                // per column the entries of its list in row j of BT, -1 when the
                               // row is dense (nullptr: every row is dense)
     double* Theta;            // the column solvers clear row j of it (nullptr: not)
@@ -211,7 +212,7 @@ __device__ __forceinline__ bool abs_above(double x, double lam) {
 template <typename T>
 __device__ __forceinline__ float key_bound(unsigned m) {
     if constexpr (sizeof(T) == 4) return __uint_as_float(m);
-    else return m == 0u ? 0.0f : __double2float_ru(__hiloint2double((int)(m + 1u), 0));
+    else return __double2float_ru(__hiloint2double((int)(m + 1u), 0));
 }
 // The largest key of the warp (non-negative floats and the upper words of
 // non-negative doubles order as unsigned integers).
@@ -743,16 +744,33 @@ __device__ __forceinline__ bool below(double d, double tol) {
     return abs_bits(d) < __double_as_longlong(tol);
 }
 
+// False only where q > 1e-12 sjj (sjj > 0) holds: decided on the upper words.  True for
+// q < 2^-38 sjj, negative, denormal, infinite or NaN (as on a matrix that is not
+// positive semidefinite), which the exact test then decides.
+__device__ __forceinline__ bool may_be_floored(double q, double sjj) {
+    const int low = max(__double2hiint(sjj) - (39 << 20), 1 << 20) + 1;
+    return (unsigned)(__double2hiint(q) - low) >= (unsigned)(0x7ff00000 - low);
+}
+
 // sqrt(q) for q > 0 in FP64 by one step of Newton's (Heron's) iteration
-// y <- y + (q - y^2) / (2 y) from the FP32 root: the FP32 root's relative
-// error (at most 2^-23) is squared, so the result is within a few FP64 units
-// of the root, with five FP64 operations.  Outside the FP32 range, sqrt.
+// y <- y + (q - y^2) / (2 y) from the FP32 root, with the FP32 reciprocal: the
+// FP32 root's relative error of 2^-24 becomes 2^-47 (its square, and the reciprocal's error
+// times it), with three instructions on the FP64 pipe.  Outside the FP32 range, sqrt.
 static __device__ __noinline__ double sqrt_far(double q) { return sqrt(q); }
+__device__ __forceinline__ bool root_in_range(float yf) { return yf > 1e-18f && yf < 1e18f; }
 __device__ __forceinline__ double sqrt_heron(double q) {
     const float yf = sqrtf((float)q);
-    if (!(yf > 1e-18f && yf < 1e18f)) return sqrt_far(q);
+    if (!root_in_range(yf)) return sqrt_far(q);
     const double y0 = exact_double(yf);
     return fma(fma(-y0, y0, q), exact_double(0.5f / yf), y0);
+}
+// One more step from y = sqrt_heron(q), for a sigma that is returned: within one FP64 unit
+// of the root.  A batch takes it with a lane per column after the solvers (the FP64 pipe
+// takes as long for one lane as for a warp: a step in each column's solver took 256 mixed
+// fits from 1955 to 1993 us); single fits, whose warps leave that pipe idle, in the solver.
+__device__ __forceinline__ double sqrt_last(double q, double y) {
+    const float yf = (float)y;
+    return root_in_range(yf) ? fma(fma(-y, y, q), exact_double(0.5f / yf), y) : y;
 }
 
 // Algorithm 1 for response column j, by one warp: warm start from b = 0,
@@ -796,10 +814,10 @@ __device__ void solve_column(int j, T* __restrict__ g, T* __restrict__ b, int* _
         }
         const double sn = sqrt_heron(q);
         if (fabs(sn - sigma) < a.tol) {
-            sigma = sn;
+            sigma = sqrt_last(q, sn);
             break;
         }
-        double nxt = sn;
+        double nxt = r + 1 < a.maxit ? sn : sqrt_last(q, sn);
         if (have_prev && r + 1 < a.maxit && !(status & COL_DEGENERATE))
             nxt = sigma_step(s_prev, (float)(f_prev - s_prev), sigma, sn, (float)(sn - sigma));
         s_prev = sigma;
@@ -1526,8 +1544,8 @@ __device__ __forceinline__ void hand_over_lazy(int j, const Support<T>& s, const
 
 // Algorithm 1 for column j with the lazy gradient.  Returns false when the
 // support outgrew the phase or the list (its state is handed over; the caller queues
-// the column for the block solver).  HS keeps the last sigma step in the warp's shared
-// memory instead of registers (for kernels at a tight register cap).
+// the column for the block solver).  HS (single fits) keeps the last sigma step in the
+// warp's shared memory instead of registers and takes sigma's sqrt_last here.
 template <typename T, bool STD, bool HS = false, int U = 2, int SCAN_G = scan_group<T>()>
 __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a, ColCounters& cnt) {
     const int lane = threadIdx.x & 31;
@@ -1536,7 +1554,7 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
     s.val = reinterpret_cast<T*>(wsm + LAZY_CAP * sizeof(int));
     s.n = 0;
     ColScan cs{reinterpret_cast<ChunkInfo*>(wsm + LAZY_CAP * (sizeof(int) + sizeof(T))), 0.f, 0u};
-    double* prev = reinterpret_cast<double*>(cs.ci + num_chunks(a.ldp));   // HS: (sigma, F(sigma)); S_jj
+    double* prev = reinterpret_cast<double*>(cs.ci + num_chunks(a.ldp));   // HS: (sigma, F(sigma)); S_jj; q
     SupportBlock<T> sb;
     sb.saa = reinterpret_cast<T*>(prev + 4);
     sb.row = sb.saa + ACT_MAX * ACT_MAX;
@@ -1598,12 +1616,9 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
         }
         if (!inner_ok) status |= COL_NOT_CONVERGED;
         double q = residual_quadratic_form_list<T>(j, s, a, sb, prev[2]);
-        // q <= 1e-12 S_jj, decided on the upper words where they decide it
+        // q <= 1e-12 S_jj; a NaN is at the floor too
         const double sjj = prev[2];
-        // (q < 2^-38 S_jj, negative, denormal, infinite or NaN, as on a matrix that is
-        // not positive semidefinite; a NaN is at the floor too)
-        const int low = max(__double2hiint(sjj) - (39 << 20), 1 << 20) + 1;
-        if ((unsigned)(__double2hiint(q) - low) >= (unsigned)(0x7ff00000 - low)) {
+        if (may_be_floored(q, sjj)) {
             const double floor2 = 1e-12 * sjj;
             if (!(q > floor2)) {
                 q = floor2;
@@ -1612,6 +1627,7 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
         }
         const double sn = sqrt_heron(q);
         const double dg = sn - sigma;
+        if (lane == 0) prev[3] = q;
         if (below(dg, a.tol)) {
             sigma = sn;
             break;
@@ -1640,6 +1656,9 @@ __device__ bool solve_column_lazy(int j, unsigned char* wsm, const CDArgs<T>& a,
     }
     store_solved_lazy<T>(j, s, a);
     if (lane == 0) {
+        // (the last step's F(sigma) either way)
+        if constexpr (HS) sigma = sqrt_last(prev[3], sigma);
+        else a.hand[2 * (size_t)j + 1] = prev[3];
         a.sigma[j] = sigma;
         a.col_status[j] = status;
     }
@@ -2810,10 +2829,14 @@ __device__ void solve_column_block(int j, unsigned char* smem, const CDArgs<T>& 
                 q = floor2;
                 f = 1;
             }
-            const double sn = sqrt_heron(q);
-            double nxt = sn;
+            double sn = sqrt_heron(q);
             if (fabs(sn - sigma) < a.tol) f |= 2;
-            else if (r > 0 && r + 1 < a.maxit && !f)
+            if ((f & 2) || r + 1 == a.maxit) {            // this sigma is returned
+                sn = sqrt_last(q, sn);
+                if (tid == 0 && a.hand) a.hand[2 * (size_t)j + 1] = q;
+            }
+            double nxt = sn;
+            if (r > 0 && r + 1 < a.maxit && !f)
                 nxt = sigma_step(s_prev, (float)(f_prev - s_prev), sigma, sn, (float)(sn - sigma));
             if (tid == 0) {
                 sc.sig[0] = sn;

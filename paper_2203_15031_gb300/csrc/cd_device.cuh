@@ -2450,17 +2450,26 @@ __device__ int block_active_phase(int j, T* __restrict__ b, const int* __restric
 // One sweep of the block solver (cyclic ascending, k != j; with `frozen` the
 // coordinates of the support keep their values).  Returns max |delta b|.
 // cand holds the candidate moves (new b, delta) of every thread, two buffers.
+// Out of line on the standardised matrix (inlined it took a hub's regression at p = 10000
+// from 932 to 979 us), with what it reads of its arguments in registers: through the
+// references each move of a sweep was 10 % slower (p = 700, more than 64 coefficients a column,
+// 17.3 against 15.3 ms a fit).  Without standardisation inline (45.5 against 45.0).
 template <typename T, bool STD>
-__device__ __noinline__ T block_sweep(int j, T* __restrict__ g, T* __restrict__ b, const CDArgs<T>& a, T lam,
+__device__ __forceinline__ T block_sweep_body(int j, T* __restrict__ g, T* __restrict__ b, const CDArgs<T>& a, T lam,
                          bool frozen, T* __restrict__ cand, unsigned long long& moves,
-                         BlockScratch& sc, int& par, int sweep_idx) {
+                         BlockScratch& sc, int& par0, int sweep_idx) {
     const int tid = threadIdx.x;
     const int p = a.p, ldp = a.ldp;
+    const T* __restrict__ SC = a.SC;
+    const T* __restrict__ diag = a.diag;
+    const bool note = a.rows_moved != nullptr;
+    int par = par0;
+    unsigned n_moves = 0;
     T maxd = T(0);
     int ks = -1;                      // the move of the last pass, applied in this pass
     T delta = T(0);
     for (;;) {
-        const T* __restrict__ srow = a.SC + (size_t)(ks < 0 ? 0 : ks) * ldp;
+        const T* __restrict__ srow = SC + (size_t)(ks < 0 ? 0 : ks) * ldp;
         T* __restrict__ cb = cand + (size_t)par * 2 * BLK_THREADS;
         int kmin = INT_MAX;
         // the thread's quads q0, q0 + BLK_THREADS, ... in groups of G, the
@@ -2498,7 +2507,7 @@ __device__ __noinline__ T block_sweep(int j, T* __restrict__ g, T* __restrict__ 
                         if constexpr (STD) {
                             nb = soft<T>(gv[t] + bv[t], lam);                 // S_kk = 1
                         } else {
-                            const T skk = a.diag[k];
+                            const T skk = diag[k];
                             nb = soft<T>(gv[t] + skk * bv[t], lam) / skk;     // Soft(c, lambda)/S_kk
                         }
                         if (nb != bv[t]) {
@@ -2517,13 +2526,31 @@ __device__ __noinline__ T block_sweep(int j, T* __restrict__ g, T* __restrict__ 
         delta = cb[BLK_THREADS + owner];
         if (tid == owner) {
             b[kb] = cb[owner];
-            note_row_moved(a, sweep_idx, kb);
+            if (note) note_row_moved(a, sweep_idx, kb);
         }
         maxd = fmax(maxd, fabs(delta));
-        ++moves;
+        ++n_moves;
         ks = kb;
     }
+    moves += n_moves;
+    par0 = par;
     return maxd;
+}
+
+template <typename T>
+__device__ __noinline__ T block_sweep_std(int j, T* __restrict__ g, T* __restrict__ b, const CDArgs<T>& a,
+                                          T lam, bool frozen, T* __restrict__ cand,
+                                          unsigned long long& moves, BlockScratch& sc, int& par,
+                                          int sweep_idx) {
+    return block_sweep_body<T, true>(j, g, b, a, lam, frozen, cand, moves, sc, par, sweep_idx);
+}
+template <typename T, bool STD>
+__device__ __forceinline__ T block_sweep(int j, T* __restrict__ g, T* __restrict__ b, const CDArgs<T>& a,
+                                         T lam, bool frozen, T* __restrict__ cand,
+                                         unsigned long long& moves, BlockScratch& sc, int& par,
+                                         int sweep_idx) {
+    if constexpr (STD) return block_sweep_std<T>(j, g, b, a, lam, frozen, cand, moves, sc, par, sweep_idx);
+    else return block_sweep_body<T, false>(j, g, b, a, lam, frozen, cand, moves, sc, par, sweep_idx);
 }
 
 // sigma_j^2 = S_jj - 2 b'S_.j + b'S b in FP64 over the support list (block-wide),

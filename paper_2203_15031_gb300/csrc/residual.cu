@@ -36,7 +36,8 @@
 // 4.3 ms with quiet chunks; 3.5 ms with the growth bounded per chunk; 1.77 ms
 // with rows staged through shared memory (a visit 3800 -> under 1000 cycles)
 // and single coordinates formed after a move.  Testing a quiet chunk again after each of
-// its moves takes 3.6 % of that fit.  The same iterates bit for bit.
+// its moves takes 3.6 % of that fit.  The same iterates bit for bit.  Without standardisation
+// there are no such bounds, and every move is followed by the chunk's slice.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -263,7 +264,7 @@ __device__ __forceinline__ void note_residual_move(T* __restrict__ r, int k, con
     rn.rb = (rn.rb + fabsf((float)delta)) * (1.0f + 0x1p-19f);
     rn.rmax = fmaxf(rn.rmax, rn.rb);
     __syncwarp();                       // every lane has read r
-    if (a.stage) {
+    if (STD && a.stage) {
 #pragma unroll
         for (int i = 0; i < RES_ROW; ++i)
             if (32 * i + lane < n) r[32 * i + lane] = fma(-delta, v[i], r[32 * i + lane]);
@@ -377,8 +378,8 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restri
         // The slice is exact until the chunk's first move.  After it only the
         // coordinates that can still move are formed again, one at a time: the
         // support's and those at zero that the growth since may have carried to
-        // the threshold.  More than RES_OPEN of them (about what a slice costs),
-        // and every move without standardisation, form the slice again.
+        // the threshold.  More than RES_OPEN of them (about what a slice costs) form
+        // the slice again.
         bool fresh = true, gone = false;
         float grow = 0.f;
         unsigned formed_at = cs.nmoves;
@@ -403,7 +404,7 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restri
                         }
                         nbv[t] = nb;
                         if (nb != bv[t]) mvmask |= 1u << t;
-                    } else if (!STD || bv[t] != T(0) ||
+                    } else if (bv[t] != T(0) ||
                                !(fabsf((float)acc[t]) * (1.0f + 0x1p-22f) < reach)) {
                         mvmask |= 1u << t;
                     }
@@ -411,7 +412,7 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restri
             }
             const unsigned bal = __ballot_sync(FULL_MASK, mvmask != 0u);
             if (bal == 0u) break;
-            if (!fresh && (!STD || __reduce_add_sync(FULL_MASK, __popc(mvmask)) > RES_OPEN)) {
+            if (STD && !fresh && __reduce_add_sync(FULL_MASK, __popc(mvmask)) > RES_OPEN) {
                 if (in) slice_dot<T>(a.W, ldp, n4, k0, r, acc);
                 fresh = true;
                 grow = 0.f;
@@ -429,18 +430,14 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restri
             const int ks = cb + f * SCAN_V + tf;
             cursor = ks + 1;
             T v[RES_ROW];
-            if (a.stage) load_row<T>(a, ks, v);
-            if (!fresh) {
-                const T gk = coordinate_dot<T>(a, ks, v, stage, r);
-                if constexpr (STD) {
-                    nbs = soft<T>(gk + bs, lam);
-                } else {
-                    const T dk = a.diag[ks];
-                    nbs = soft<T>(gk + dk * bs, lam) / dk;
-                }
-                if (nbs == bs) {
-                    if (cursor >= cb + CHUNK) break;
-                    continue;
+            if (STD && a.stage) load_row<T>(a, ks, v);
+            if constexpr (STD) {
+                if (!fresh) {
+                    nbs = soft<T>(coordinate_dot<T>(a, ks, v, stage, r) + bs, lam);
+                    if (nbs == bs) {
+                        if (cursor >= cb + CHUNK) break;
+                        continue;
+                    }
                 }
             }
             const T delta = nbs - bs;
@@ -464,6 +461,10 @@ __device__ T sweep_residual(int j, Support<T>& s, T* __restrict__ r, T* __restri
             gone |= nbs == T(0);
             if constexpr (STD) grow += fabsf((float)delta) * chunk_bound(a, ks, ci);
             if (cursor >= cb + CHUNK) break;
+            if constexpr (!STD) {                 // no bounds: the slice again at once
+                if (in) slice_dot<T>(a.W, ldp, n4, k0, r, acc);
+                fresh = true;
+            }
         }
         if constexpr (STD) {
             // the summary: the slice as it was formed, and the growth since.  A
